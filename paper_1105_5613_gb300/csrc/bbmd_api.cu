@@ -787,7 +787,7 @@ bbmd_status bbmd_observe(bbmd_sim* sim, uint32_t mask, const bbmd_obs_args* args
     launch_state_sums(D, sim->st);
     launch_reduce_partials(D, sim->st, 4, sim->dout);
     if (mask & (BBMD_OBS_ENERGY | BBMD_OBS_VIRIAL)) {
-        launch_force(D, sim->st, true, false);
+        launch_energy_sums(D, sim->st);
         launch_reduce_partials(D, sim->st, -3, sim->dout + 8);
     }
     const int origin = args ? args->origin : 0;

@@ -262,8 +262,9 @@ void launch_rebuild_chain(const DevSim& s, cudaStream_t st);
 // Per block shape (namespace z1, z2, z4, z8; defined in k_force.cu compiled per shape):
 //   prepare_force_kernels  one-time kernel attributes (call before any stream capture)
 //   force/list_blocks_per_sm  resident CTAs per SM for this handle's shared memory
-//   launch_force   forces; energy: also per-particle energy and virial partials; ke: NH
-//                  kinetic partials
+//   launch_force   forces; energy: also per-particle energy and virial partials (not with
+//                  ke); ke: NH kinetic partials
+//   launch_energy_sums  energy and virial partials only
 //   launch_list_build  Verlet list build (gated)
 #define BBMD_SHAPE_API(ns)                                                             \
     namespace ns {                                                                     \
@@ -276,6 +277,7 @@ void launch_rebuild_chain(const DevSim& s, cudaStream_t st);
     int list_blocks_per_sm(const DevSim& s);                                           \
     int block_threads();                                                               \
     void launch_force(const DevSim& s, cudaStream_t st, bool energy, bool ke);         \
+    void launch_energy_sums(const DevSim& s, cudaStream_t st);                         \
     void launch_list_build(const DevSim& s, cudaStream_t st);                          \
     }
 BBMD_SHAPE_API(z1)
@@ -334,6 +336,9 @@ inline int force_blocks_per_sm(const DevSim& s) { BBMD_SHAPE_DISPATCH(s.block_z,
 inline int list_blocks_per_sm(const DevSim& s) { BBMD_SHAPE_DISPATCH(s.block_z, list_blocks_per_sm(s)) }
 inline void launch_force(const DevSim& s, cudaStream_t st, bool energy, bool ke) {
     BBMD_SHAPE_DISPATCH(s.block_z, launch_force(s, st, energy, ke))
+}
+inline void launch_energy_sums(const DevSim& s, cudaStream_t st) {
+    BBMD_SHAPE_DISPATCH(s.block_z, launch_energy_sums(s, st))
 }
 inline void launch_list_build(const DevSim& s, cudaStream_t st) {
     BBMD_SHAPE_DISPATCH(s.block_z, launch_list_build(s, st))

@@ -579,6 +579,60 @@ __device__ __forceinline__ void chunk_lane(const StageShared& ss, int item, int 
     self = act ? ss.c_off[q] + li : 0;
 }
 
+// The cell (within the block) of lane `lane`'s particle of chunk `item`.
+__device__ __forceinline__ int chunk_cell(const StageShared& ss, int item, int lane) {
+    const bool isB = item >= ss.nchA;
+    const int o = (isB ? item - ss.nchA : item) * 32 + lane;
+    const int* pref = isB ? ss.prefB : ss.prefA;
+    int q = 0, hi = kCells - 1;
+    while (q < hi) {
+        const int mid = (q + hi + 1) >> 1;
+        if (pref[mid] <= o) q = mid;
+        else hi = mid - 1;
+    }
+    return q;
+}
+
+// Describe the block's chunks (ss.c_*, ss.pref*, ss.nchA, ss.nch).  is_A(t): staged particle
+// t is of species A.  Every thread of the CTA calls it; it synchronises.
+template <class IsA>
+__device__ __forceinline__ void own_chunks(const DevSim& s, const BlockPos& bp, const Region& Rc,
+                                           StageShared& ss, IsA is_A) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int cw = w; cw < kCells; cw += kBW) {
+        const WarpCell wc = warp_cell(s, bp, cw);
+        const int cnt = wc.valid ? staged_count(Rc, wc.rq) : 0;
+        const int off = Rc.off[wc.rq];
+        int nA = 0;  // the cell's A particles come first
+        for (int t = 0; t < cnt; t += 32) {
+            const unsigned b = __ballot_sync(FULL, t + lane < cnt && is_A(off + t + lane));
+            nA += __popc(b);
+            if (b != FULL) break;
+        }
+        if (lane == 0) {
+            ss.c_off[cw] = off;
+            ss.c_i0[cw] = wc.valid ? Rc.start[wc.rq] : 0;
+            ss.c_n[cw] = cnt;
+            ss.c_nA[cw] = nA;
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int na = 0, nb = 0;
+        for (int c = 0; c < kCells; ++c) {
+            ss.prefA[c] = na;
+            ss.prefB[c] = nb;
+            na += ss.c_nA[c];
+            nb += ss.c_n[c] - ss.c_nA[c];
+        }
+        ss.prefA[kCells] = na;
+        ss.prefB[kCells] = nb;
+        ss.nchA = (na + 31) >> 5;
+        ss.nch = ss.nchA + ((nb + 31) >> 5);
+    }
+    __syncthreads();
+}
+
 // The next work item of the block for this warp (at least the item count when none is
 // left).
 __device__ __forceinline__ int take_cell(StageShared& ss, int par, int lane) {
@@ -775,39 +829,7 @@ __device__ __forceinline__ void force_body(const DevSim& s, int lb, int lg) {
         // mode its cells (the stencil is the cell's)
         int nitems = kCells;
         if constexpr (MODE == 0) {
-            for (int cw = w; cw < kCells; cw += kBW) {
-                const WarpCell wc = warp_cell(s, bp, cw);
-                const int cnt = wc.valid ? staged_count(Rc, wc.rq) : 0;
-                const int off = Rc.off[wc.rq];
-                int nA = 0;  // the cell's A particles come first
-                for (int t = 0; t < cnt; t += 32) {
-                    const unsigned b =
-                        __ballot_sync(FULL, t + lane < cnt && sm[off + t + lane].w == 0.f);
-                    nA += __popc(b);
-                    if (b != FULL) break;
-                }
-                if (lane == 0) {
-                    ss.c_off[cw] = off;
-                    ss.c_i0[cw] = wc.valid ? Rc.start[wc.rq] : 0;
-                    ss.c_n[cw] = cnt;
-                    ss.c_nA[cw] = nA;
-                }
-            }
-            __syncthreads();
-            if (threadIdx.x == 0) {
-                int na = 0, nb = 0;
-                for (int c = 0; c < kCells; ++c) {
-                    ss.prefA[c] = na;
-                    ss.prefB[c] = nb;
-                    na += ss.c_nA[c];
-                    nb += ss.c_n[c] - ss.c_nA[c];
-                }
-                ss.prefA[kCells] = na;
-                ss.prefB[kCells] = nb;
-                ss.nchA = (na + 31) >> 5;
-                ss.nch = ss.nchA + ((nb + 31) >> 5);
-            }
-            __syncthreads();
+            own_chunks(s, bp, Rc, ss, [&](int t) { return sm[t].w == 0.f; });
             nitems = ss.nch;
         }
         for (int item = take_cell(ss, par, lane); item < nitems; item = take_cell(ss, par, lane)) {
@@ -1370,13 +1392,41 @@ __global__ void __launch_bounds__(kBW * 32, 2) k_step_persistent(PersistentStep 
 // stays right after the particle itself has crossed the boundary since the last build);
 // distances are the exact integer differences rounded once to double (the rule the list
 // decisions use), pair arithmetic and accumulation in FP64.
+//
+// Bound: the FP64 pipe (2 lanes a clock per SM, 16 clocks for a warp instruction whatever
+// the number of active lanes).  So the kernel keeps everything but the arithmetic of
+// interacting pairs off that pipe, and runs it with full warps:
+//   - a candidate is classified in FP32 from the upper words of its integer position
+//     (resolution 2^(32-k)): beyond the cutoff, interacting, or too close to the cutoff to
+//     tell, which the exact rule then decides;
+//   - each lane queues its interacting candidates (shared memory) and the warp drains the
+//     queues together, so a slot of the loop computes a pair on nearly every lane, instead
+//     of once per candidate that any of the 32 lanes interacts with;
+//   - r^2 stays in integer units (the scale is folded into sigma^2), 1/r^2 and 1/r come
+//     from the hardware's approximation and one third-order step, and energies and virial
+//     come from the sums of s^12 and s^6;
+//   - sums over the system (energy, virial) take each pair from one side only.
+// Measured against the form that ran the FP64 arithmetic for every candidate some lane of
+// the warp interacts with: energy and virial sums at 16.4 M particles (lists, skin 0.4)
+// 132 -> 24 ms, at 4 M in cell mode 121 -> 13.6 ms; forces of the FP64 form at 108 000
+// 0.868 -> 0.383 ms.  (17 to 19 FP64 instructions a pair at 0.63e12 lanes a second put the
+// floor of the three at 14, 3.5 and 0.21 ms.)
 
-struct Pos64 {
-    long long x, y, z;
-    int sp, pad;
+// Staged record t: hi[t] = upper words of x, y, z and (global index << 1 | species), lo[t] =
+// lower words.
+struct Stage64 {
+    int4* hi;
+    uint4* lo;
 };
 
-__device__ void stage_block64(const DevSim& s, const BlockPos& b, Region& R, Pos64* sm) {
+__device__ __forceinline__ Stage64 stage64(const DevSim& s, float4* smem) {
+    Stage64 g;
+    g.hi = reinterpret_cast<int4*>(smem);
+    g.lo = reinterpret_cast<uint4*>(smem) + (s.smax + 1);
+    return g;
+}
+
+__device__ void stage_block64(const DevSim& s, const BlockPos& b, Region& R, const Stage64& g) {
     region_info(s, b, R);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int q = w; q < kRegion; q += kBW) {
@@ -1384,164 +1434,285 @@ __device__ void stage_block64(const DevSim& s, const BlockPos& b, Region& R, Pos
         const long long fx = R.fr[q][0], fy = R.fr[q][1], fz = R.fr[q][2];
         for (int t = lane; t < cq; t += 32) {
             const int64_t j = R.start[q] + t;
-            Pos64 p;
-            p.x = fx + min_image((long long)s.x[j] - fx, s.Lfix[0]);
-            p.y = fy + min_image((long long)s.x[s.npad + j] - fy, s.Lfix[1]);
-            p.z = fz + min_image((long long)s.x[2 * s.npad + j] - fz, s.Lfix[2]);
-            p.sp = s.sp[j];
-            p.pad = 0;
-            sm[o0 + t] = p;
+            const long long x = fx + min_image((long long)s.x[j] - fx, s.Lfix[0]);
+            const long long y = fy + min_image((long long)s.x[s.npad + j] - fy, s.Lfix[1]);
+            const long long z = fz + min_image((long long)s.x[2 * s.npad + j] - fz, s.Lfix[2]);
+            g.hi[o0 + t] = make_int4((int)(x >> 32), (int)(y >> 32), (int)(z >> 32),
+                                     (int)(((unsigned)j << 1) | s.sp[j]));
+            g.lo[o0 + t] = make_uint4((unsigned)x, (unsigned)y, (unsigned)z, 0u);
         }
     }
     if (threadIdx.x == 0) {
         // staged positions lie in (-L_fix, 2 L_fix) with L_fix < 2^62: a sentinel at 3 * 2^61
-        // on every axis is beyond every cutoff (|dx| > L/2 is never a minimum image) and no
-        // difference overflows
-        Pos64 far;
-        far.x = far.y = far.z = (long long)3 << 61;
-        far.sp = 0;
-        far.pad = 0;
-        sm[s.smax] = far;
+        // on every axis is beyond every cutoff (more than L/2 from every own particle) and
+        // no difference of upper words overflows
+        g.hi[s.smax] = make_int4(3 << 29, 3 << 29, 3 << 29, 0);
+        g.lo[s.smax] = make_uint4(0u, 0u, 0u, 0u);
     }
     __syncthreads();
 }
 
-template <bool ENERGY, bool FSHIFT>
-__device__ __forceinline__ void pair_fp64(const DevSim& s, int si, const Pos64& me, const Pos64& p,
-                                          double& fx, double& fy, double& fz, double& u,
-                                          double& w) {
-    const long long ix = p.x - me.x, iy = p.y - me.y, iz = p.z - me.z;
-    const int k = si * 2 + p.sp;
-    // integer pre-test: a separation beyond rc on some axis cannot interact.  rc < L/2 (the
-    // box holds at least three cells of side >= rc per axis), so what passes is the
-    // minimum-image copy (a region may hold a cell twice when nc = 3)
-    const long long lim = s.pt.rcfix[k];
-    if (llabs(ix) > lim || llabs(iy) > lim || llabs(iz) > lim) return;
-    double dx = __dmul_rn(__ll2double_rn(ix), s.sxd);
-    double dy = __dmul_rn(__ll2double_rn(iy), s.sxd);
-    double dz = __dmul_rn(__ll2double_rn(iz), s.sxd);
-    double r2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
-    if (r2 < s.pt.rc2[k]) {
-        double ir2 = 1.0 / r2;
-        double s2 = s.pt.dsig2[k] * ir2;
-        double s6 = s2 * s2 * s2;
-        double cp = s.pt.potential == BBMD_POT_LJ ? 0.5 : 0.0;
-        double f = s.pt.deps48[k] * ir2 * s6 * (s6 - cp);
-        double r = 0.0;
-        if (FSHIFT) {
-            r = sqrt(r2);
-            f += s.pt.dfcut[k] / r;
-        }
-        fx += f * dx;
-        fy += f * dy;
-        fz += f * dz;
-        if (ENERGY) {
-            double ce = s.pt.potential == BBMD_POT_LJ ? 1.0 : 0.0;
-            double V = s.pt.deps4[k] * s6 * (s6 - ce) - s.pt.dvshift[k];
-            if (FSHIFT) V -= (r - s.pt.drc[k]) * s.pt.dfcut[k];
-            u += V;
-            w += f * r2;
-        }
+__device__ __forceinline__ long long join64(int hi, unsigned lo) {
+    return (long long)(((unsigned long long)(unsigned)hi << 32) | lo);
+}
+
+// 1/x and 1/sqrt(x) in FP64: the hardware's approximation y (relative error e below 2^-18)
+// and one third-order step, y (1 + e + e^2 [+ ...]) with e = 1 - x y or 1 - x y^2, whose
+// own error is of order e^3 < 2^-54.
+__device__ __forceinline__ double rcp64(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x, y, 1.0);
+    return fma(y, fma(e, e, e), y);
+}
+
+__device__ __forceinline__ double rsqrt64(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double e = fma(-x * y, y, 1.0);
+    return fma(fma(e, 0.375, 0.5), e * y, y);
+}
+
+// Queue entries per lane: full rows of 8 candidates are added while at most kQ64 - 8 wait.
+constexpr int kQ64 = 32;
+constexpr unsigned kBand64 = 0x8000u;  // entry left to the exact rule (staged indices < 2^15)
+
+__device__ __forceinline__ uint16_t* warp_queue64(int w) {
+    __shared__ uint16_t q_all[kBW][kQ64 * 32];
+    return q_all[w];
+}
+
+// What the body computes: forces, per-particle energies (and their sums), or the sums of
+// energy and virial alone.
+enum : int { k64Force = 1, k64Energy = 2, k64Sums = 4 };
+
+// One lane's pair constants and accumulators, in units of 2^-k (r^2 and forces).
+struct Lane64 {
+    double sig20, sig21, e40, e41, dc0, dc1;  // sigma^2 2^2k, 4 eps, dV/dr(rc) 2^-k
+    double fx, fy, fz;                        // sum of f d, integer units
+    double s12, s6, sr;                       // sums of 4 eps s^12, 4 eps s^6, dV/dr(rc) r
+    int n0, n1;                               // interacting pairs by species of j
+};
+
+template <int WHAT, bool FSHIFT>
+__device__ __forceinline__ void pair_fp64(const DevSim& s, int si, long long mx, long long my,
+                                          long long mz, const Stage64& g, unsigned ent, Lane64& A) {
+    const int t = (int)(ent & (kBand64 - 1u));
+    const int4 h = g.hi[t];
+    const uint4 l = g.lo[t];
+    const double dx = __ll2double_rn(join64(h.x, l.x) - mx);
+    const double dy = __ll2double_rn(join64(h.y, l.y) - my);
+    const double dz = __ll2double_rn(join64(h.z, l.z) - mz);
+    const bool b = h.w & 1;
+    if (ent & kBand64) {
+        // the exact rule, in integer units (the scale is a power of two: the same roundings).
+        // rc < L/2 (the box holds at least three cells of side >= rc per axis), so what it
+        // accepts is the minimum-image copy (a region may hold a cell twice when nc = 3)
+        const double e2 = __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+        if (!(e2 * s.sxd * s.sxd < s.pt.rc2[si * 2 + (b ? 1 : 0)])) return;
+    }
+    const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+    double ir2, r = 0.0, ir = 0.0;
+    if (FSHIFT) {
+        ir = rsqrt64(r2);
+        ir2 = ir * ir;
+        r = r2 * ir;
+    } else {
+        ir2 = rcp64(r2);
+    }
+    const double s2 = (b ? A.sig21 : A.sig20) * ir2;
+    const double s6 = s2 * s2 * s2;
+    const double w6 = (b ? A.e41 : A.e40) * s6;  // 4 eps s^6
+    const bool lj = s.pt.potential == BBMD_POT_LJ;
+    if (WHAT & k64Force) {
+        // f / 12 = 4 eps s^6 (s^6 - 1/2) / r^2 (+ dV/dr(rc) / (12 r)); the 12 is applied
+        // to the finished sum
+        double f = fma(w6, s6, lj ? -0.5 * w6 : 0.0) * ir2;
+        if (FSHIFT) f = fma(b ? A.dc1 : A.dc0, ir * (1.0 / 12.0), f);
+        A.fx = fma(f, dx, A.fx);
+        A.fy = fma(f, dy, A.fy);
+        A.fz = fma(f, dz, A.fz);
+    }
+    if (WHAT & (k64Energy | k64Sums)) {
+        A.s12 = fma(w6, s6, A.s12);
+        A.s6 += w6;
+        if (FSHIFT) A.sr = fma(b ? A.dc1 : A.dc0, r, A.sr);
+        if (b) ++A.n1; else ++A.n0;
     }
 }
 
-// ENERGY: per-particle energies u_i (half of each pair energy), and the energy and virial
-// partials 1 and 2.  EONLY (with ENERGY, mixed precision): the energy pass of a
-// mixed-precision handle -- the same exact integer positions and FP64 pair arithmetic,
-// but the forces stay those of the FP32 kernel (nothing is written to F or Fd).
-template <int MODE, bool ENERGY, bool KE, bool FSHIFT, bool EONLY = false>
+// WHAT: see above (k64Force writes F and Fd; k64Energy the per-particle energies u_i, half
+// of each pair energy; with k64Energy or k64Sums the energy and virial partials 1 and 2).
+template <int MODE, int WHAT, bool KE, bool FSHIFT>
 __device__ __forceinline__ void force64_body(const DevSim& s, int lb, int lg) {
     if (!force_selected<MODE>(s)) return;  // CTA-uniform, before any barrier
     extern __shared__ float4 smem[];
-    __shared__ Region R;
+    StageShared& ss = stage_shared();
+    Region& R = ss.R[0];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    Pos64* sm = reinterpret_cast<Pos64*>(smem);
+    const Stage64 g = stage64(s, smem);
+    uint16_t* const q = warp_queue64(w) + lane;
+    const bool lj = s.pt.potential == BBMD_POT_LJ;
+    // FP32 thresholds in upper-word units: the truncation of the upper words moves a distance
+    // by less than sqrt(3) units, FP32 rounding by less than 1e-6 of it
+    const double inv_u = ldexp(1.0, s.kexp - 32);
     double acc_ke = 0.0, acc_u = 0.0, acc_w = 0.0;
     for (int64_t blk = lb; blk < s.nblocks; blk += lg) {
         const BlockPos bp = block_pos(s, blk);
-        stage_block64(s, bp, R, sm);
-        for (int cw = w; cw < kCells; cw += kBW) {
-        const WarpCell wc = warp_cell(s, bp, cw);
-        const int i0 = wc.valid ? s.cell_start[wc.c] : 0;
-        const int cnt = wc.valid ? staged_count(R, wc.rq) : 0;
-        const int self0 = R.off[wc.rq];
-        for (int ch = 0; ch * 32 < cnt; ++ch) {
-            const int li = ch * 32 + lane;
-            const bool act = li < cnt;
-            const int64_t gi = (int64_t)i0 + li;
-            Pos64 me;
-            if (act) {
-                me = sm[self0 + li];
-            } else {
-                me.x = me.y = me.z = -((long long)1 << 62);
-                me.sp = 0;
-            }
-            const int si = me.sp;
-            double fx = 0, fy = 0, fz = 0, u = 0, wv = 0;
-            if (MODE == 0) {
-                const int nkb = act ? (int)s.rows[gi] : 0;  // rows of the particle's list
-                const uint4* lp = reinterpret_cast<const uint4*>(s.list) + gi;
-                for (int kb = 0; kb < nkb; ++kb) {
-                    uint4 e = lp[(int64_t)kb * s.npad];
-                    unsigned ws[4] = {e.x, e.y, e.z, e.w};
+        stage_block64(s, bp, R, g);
+        own_chunks(s, bp, R, ss, [&](int t) { return (g.hi[t].w & 1) == 0; });
+        // chunks go to the warps in a fixed order (the sums must not depend on timing)
+        for (int item = w; item < ss.nch; item += kBW) {
+            bool act;
+            int64_t gi;
+            int self;
+            chunk_lane(ss, item, lane, act, gi, self);
+            const int si = item >= ss.nchA ? 1 : 0;
+            const int4 mh = g.hi[self];
+            const uint4 ml = g.lo[self];
+            const long long mx = join64(mh.x, ml.x), my = join64(mh.y, ml.y), mz = join64(mh.z, ml.z);
+            float in2[2], out2[2];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        pair_fp64<ENERGY, FSHIFT>(s, si, me, sm[ws[q] & 0xffffu], fx, fy, fz, u, wv);
-                        pair_fp64<ENERGY, FSHIFT>(s, si, me, sm[ws[q] >> 16], fx, fy, fz, u, wv);
+            for (int b = 0; b < 2; ++b) {
+                const float rc = (float)(s.pt.drc[si * 2 + b] * inv_u);
+                const float lo = rc * (1.0f - 2e-6f) - 2.0f, hi = rc * (1.0f + 2e-6f) + 2.0f;
+                in2[b] = lo > 0.f ? lo * lo : 0.f;
+                out2[b] = hi * hi;
+            }
+            Lane64 A;
+            A.sig20 = ldexp(s.pt.dsig2[si * 2], 2 * s.kexp);
+            A.sig21 = ldexp(s.pt.dsig2[si * 2 + 1], 2 * s.kexp);
+            A.e40 = s.pt.deps4[si * 2];
+            A.e41 = s.pt.deps4[si * 2 + 1];
+            A.dc0 = A.dc1 = 0.0;
+            if (FSHIFT) {
+                A.dc0 = s.pt.dfcut[si * 2] * s.sxd;
+                A.dc1 = s.pt.dfcut[si * 2 + 1] * s.sxd;
+            }
+            A.fx = A.fy = A.fz = A.s12 = A.s6 = A.sr = 0.0;
+            A.n0 = A.n1 = 0;
+            int cnt = 0;
+            // classify candidate t; queue it unless it is beyond the cutoff
+            auto consider = [&](int t) {
+                const int4 h = g.hi[t];
+                const float x = (float)(int)((unsigned)h.x - (unsigned)mh.x);
+                const float y = (float)(int)((unsigned)h.y - (unsigned)mh.y);
+                const float z = (float)(int)((unsigned)h.z - (unsigned)mh.z);
+                const float r2 = fmaf(x, x, fmaf(y, y, z * z));
+                const bool b = h.w & 1;
+                bool take = r2 < (b ? out2[1] : out2[0]);
+                if (WHAT & k64Sums) {
+                    // each pair from one side: the larger index where the two have the same
+                    // parity, else the smaller (half of every particle's pairs)
+                    const unsigned j = (unsigned)h.w >> 1, i = (unsigned)mh.w >> 1;
+                    take = take && ((j < i) != (((j ^ i) & 1u) != 0u));
+                }
+                if (take) {
+                    q[cnt * 32] = (uint16_t)((unsigned)t | (r2 < (b ? in2[1] : in2[0]) ? 0u : kBand64));
+                    ++cnt;
+                }
+            };
+            // pairs of the queues' tops until no lane holds more than `keep`
+            auto drain = [&](int keep) {
+                while (__any_sync(FULL, cnt > keep)) {
+                    if (cnt > 0) {
+                        --cnt;
+                        pair_fp64<WHAT, FSHIFT>(s, si, mx, my, mz, g, q[cnt * 32], A);
                     }
                 }
-            } else if (act) {
-                const int self = self0 + li;
+            };
+            if (MODE == 0) {
+                const int myrows = act ? (int)s.rows[gi] : 0;  // rows of the particle's list
+                int nkb = myrows;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) nkb = max(nkb, __shfl_xor_sync(FULL, nkb, o));
+                const uint4* lp = reinterpret_cast<const uint4*>(s.list) + gi;
+                uint4 e = make_uint4(0u, 0u, 0u, 0u);
+                if (myrows > 0) e = __ldcs(lp);
+                for (int kb = 0; kb < nkb; ++kb) {
+                    const unsigned ws[4] = {e.x, e.y, e.z, e.w};
+                    if (kb + 1 < myrows) e = __ldcs(lp + (int64_t)(kb + 1) * s.npad);
+                    if (kb < myrows) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            consider((int)lo16(ws[u]));
+                            consider((int)hi16(ws[u]));
+                        }
+                    }
+                    if (__any_sync(FULL, cnt > kQ64 - 8)) drain(kQ64 / 4);
+                }
+            } else {
+                // the lane's own 27-cell stencil (the lanes of a chunk may lie in several cells)
+                const int cq = act ? chunk_cell(ss, item, lane) : 0;
                 for (int row = 0; row < 9; ++row) {
+                    WarpCell wc;
+                    wc.wr[0] = cq % kBlockXY;
+                    wc.wr[1] = (cq / kBlockXY) % kBlockXY;
+                    wc.wr[2] = cq / (kBlockXY * kBlockXY);
                     int rs, re;
                     stencil_run(R, wc, row, rs, re);
-                    for (int t = rs; t < re; ++t) {
-                        if (t == self) continue;
-                        pair_fp64<ENERGY, FSHIFT>(s, si, me, sm[t], fx, fy, fz, u, wv);
+                    if (!act) re = rs;
+                    int len = re - rs;
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) len = max(len, __shfl_xor_sync(FULL, len, o));
+                    for (int o = 0; o < len; o += 8) {
+#pragma unroll
+                        for (int u = 0; u < 8; ++u) {
+                            const int t = rs + o + u;
+                            if (t < re && t != self) consider(t);
+                        }
+                        if (__any_sync(FULL, cnt > kQ64 - 8)) drain(kQ64 / 4);
                     }
                 }
             }
-            if (act && !EONLY) {
-                fx = -fx;
-                fy = -fy;
-                fz = -fz;
-                if (!(isfinite(fx) && isfinite(fy) && isfinite(fz))) set_status(s, ST_NONFINITE);
-                s.Fd[gi] = fx;
-                s.Fd[s.npad + gi] = fy;
-                s.Fd[2 * s.npad + gi] = fz;
-                s.F[gi] = make_float4((float)fx, (float)fy, (float)fz, 0.f);
-            }
-            if (act && ENERGY) s.ud[gi] = 0.5 * u;
-            if (KE) {
-                double k = 0.0;
+            drain(0);
+            double Fx = 0.0, Fy = 0.0, Fz = 0.0;
+            if (WHAT & k64Force) {
+                const double c = -12.0 / s.sxd;  // (a power of two: exact)
+                Fx = A.fx * c;
+                Fy = A.fy * c;
+                Fz = A.fz * c;
                 if (act) {
-                    double h = 0.5 * s.sc->dt / s.pt.dmass[si];
-                    double vx = __ll2double_rn(s.v[gi]) * 0x1p-52 + h * fx;
-                    double vy = __ll2double_rn(s.v[s.npad + gi]) * 0x1p-52 + h * fy;
-                    double vz = __ll2double_rn(s.v[2 * s.npad + gi]) * 0x1p-52 + h * fz;
-                    k = 0.5 * s.pt.dmass[si] * (vx * vx + vy * vy + vz * vz);
-                }
-                k = warp_sum_d(k);
-                if (lane == 0) acc_ke += k;
-            }
-            if (ENERGY) {
-                double uu = warp_sum_d(act ? 0.5 * u : 0.0);
-                double ww = warp_sum_d(act ? 0.5 * wv : 0.0);
-                if (lane == 0) {
-                    acc_u += uu;
-                    acc_w += ww;
+                    if (!(isfinite(Fx) && isfinite(Fy) && isfinite(Fz))) set_status(s, ST_NONFINITE);
+                    s.Fd[gi] = Fx;
+                    s.Fd[s.npad + gi] = Fy;
+                    s.Fd[2 * s.npad + gi] = Fz;
+                    s.F[gi] = make_float4((float)Fx, (float)Fy, (float)Fz, 0.f);
                 }
             }
-        }
+            if (KE && act) {
+                const double hm = 0.5 * s.sc->dt / s.pt.dmass[si];
+                const double vx = __ll2double_rn(s.v[gi]) * 0x1p-52 + hm * Fx;
+                const double vy = __ll2double_rn(s.v[s.npad + gi]) * 0x1p-52 + hm * Fy;
+                const double vz = __ll2double_rn(s.v[2 * s.npad + gi]) * 0x1p-52 + hm * Fz;
+                acc_ke += 0.5 * s.pt.dmass[si] * (vx * vx + vy * vy + vz * vz);
+            }
+            if ((WHAT & (k64Energy | k64Sums)) && act) {
+                // V = 4 eps (s^12 - s^6) - V(rc) - (r - rc) dV/dr(rc), summed; virial
+                // f r^2 = 12 (4 eps s^12) - 6 (4 eps s^6) + r dV/dr(rc) (soft sphere: no s^6)
+                const int k = si * 2;
+                double c0 = s.pt.dvshift[k], c1 = s.pt.dvshift[k + 1];
+                if (FSHIFT) {
+                    c0 -= s.pt.drc[k] * s.pt.dfcut[k];
+                    c1 -= s.pt.drc[k + 1] * s.pt.dfcut[k + 1];
+                }
+                const double s6 = lj ? A.s6 : 0.0;
+                const double u = ((A.s12 - s6) - A.sr) - ((double)A.n0 * c0 + (double)A.n1 * c1);
+                const double wv = fma(12.0, A.s12, fma(-6.0, s6, A.sr));
+                const double half = WHAT & k64Sums ? 1.0 : 0.5;
+                if (WHAT & k64Energy) s.ud[gi] = half * u;
+                acc_u += half * u;
+                acc_w += half * wv;
+            }
         }
         __syncthreads();
     }
-    if (EONLY) {
-        const double wv2[2] = {acc_u, acc_w};
-        block_partials(s, lb, wv2, 1, 2);
-    } else if (KE || ENERGY) {
-        const double wv3[3] = {acc_ke, acc_u, acc_w};
-        block_partials(s, lb, wv3, 0, 3);
+    if (KE || (WHAT & (k64Energy | k64Sums))) {
+        const double sums[3] = {warp_sum_d(acc_ke), warp_sum_d(acc_u), warp_sum_d(acc_w)};
+        if (KE)
+            block_partials(s, lb, sums, 0, WHAT & (k64Energy | k64Sums) ? 3 : 1);
+        else
+            block_partials(s, lb, sums + 1, 1, 2);
     }
 }
 
@@ -1575,17 +1746,17 @@ __global__ void __launch_bounds__(kBW * 32, BBMD_LIST_MIN_BLOCKS) k_list_build_m
     list_build_body(sh, lb, lg);
 }
 
-template <int MODE, bool ENERGY, bool KE, bool FSHIFT, bool EONLY = false>
+template <int MODE, int WHAT, bool KE, bool FSHIFT>
 __global__ void __launch_bounds__(kBW * 32) k_force64(DevSim s) {
-    force64_body<MODE, ENERGY, KE, FSHIFT, EONLY>(s, (int)blockIdx.x, (int)gridDim.x);
+    force64_body<MODE, WHAT, KE, FSHIFT>(s, (int)blockIdx.x, (int)gridDim.x);
 }
 
-template <int MODE, bool ENERGY, bool KE, bool FSHIFT>
+template <int MODE, bool KE, bool FSHIFT>
 __global__ void __launch_bounds__(kBW * 32) k_force64_many(ManySims m) {
     __shared__ DevSim sh;
     int lb, lg;
     load_replica(m, sh, lb, lg);
-    force64_body<MODE, ENERGY, KE, FSHIFT>(sh, lb, lg);
+    force64_body<MODE, k64Force, KE, FSHIFT>(sh, lb, lg);
 }
 
 // Opt every kernel with dynamic shared memory into the largest size the device allows
@@ -1609,71 +1780,74 @@ void set_smem(K kernel) {
         g_smem_ok = false;
 }
 
+// Dynamic shared memory of the FP64 kernels: upper and lower words of every staged record.
+static size_t smem64(int smax) { return (size_t)(smax + 1) * 32; }
+
 // Mixed precision: FP32 forces; an energy pass (E) adds the FP64 energy kernel, which
 // writes the per-particle energies and the energy and virial partials from exact integer
-// positions (FP32 coordinates would limit u_i to about 1e-4).
+// positions (FP32 coordinates would limit u_i to about 1e-4) and leaves the forces alone.
 template <int MODE, bool E, bool KE, bool FS>
 void run_force(const DevSim& s, cudaStream_t st) {
-    const size_t bytes64 = (size_t)(s.smax + 1) * sizeof(Pos64);
     if (s.precision == BBMD_PREC_FP64) {
-        k_force64<MODE, E, KE, FS><<<s.grid_cell, kBW * 32, bytes64, st>>>(s);
+        k_force64<MODE, E ? k64Force | k64Energy : k64Force, KE, FS>
+            <<<s.grid_cell, kBW * 32, smem64(s.smax), st>>>(s);
     } else {
         size_t bytes = kStageBuffers * (size_t)(s.smax + 1) * sizeof(float4);
         k_force<MODE, KE, FS><<<s.grid_cell, kBW * 32, bytes, st>>>(s);
-        if (E) k_force64<MODE, true, false, FS, true><<<s.grid_cell, kBW * 32, bytes64, st>>>(s);
+        if (E) k_force64<MODE, k64Energy, false, FS><<<s.grid_cell, kBW * 32, smem64(s.smax), st>>>(s);
     }
 }
 
 template <int MODE, bool KE, bool FS>
 void run_force_many(const ManySims& m, int total, bool fp64, int smax_max, cudaStream_t st) {
     if (fp64) {
-        size_t bytes = (size_t)(smax_max + 1) * sizeof(Pos64);
-        k_force64_many<MODE, false, KE, FS><<<total, kBW * 32, bytes, st>>>(m);
+        k_force64_many<MODE, KE, FS><<<total, kBW * 32, smem64(smax_max), st>>>(m);
     } else {
         size_t bytes = kStageBuffers * (size_t)(smax_max + 1) * sizeof(float4);
         k_force_many<MODE, KE, FS><<<total, kBW * 32, bytes, st>>>(m);
     }
 }
 
-template <int MODE>
-void run_force_mode(const DevSim& s, cudaStream_t st, bool energy, bool ke, bool fs) {
-    if (fs) {
-        if (energy) {
-            if (ke) run_force<MODE, true, true, true>(s, st); else run_force<MODE, true, false, true>(s, st);
-        } else {
-            if (ke) run_force<MODE, false, true, true>(s, st); else run_force<MODE, false, false, true>(s, st);
-        }
+template <int MODE, bool FS>
+void run_force_fs(const DevSim& s, cudaStream_t st, bool energy, bool ke) {
+    if (energy) {
+        run_force<MODE, true, false, FS>(s, st);  // (no caller asks for both)
     } else {
-        if (energy) {
-            if (ke) run_force<MODE, true, true, false>(s, st); else run_force<MODE, true, false, false>(s, st);
-        } else {
-            if (ke) run_force<MODE, false, true, false>(s, st); else run_force<MODE, false, false, false>(s, st);
-        }
+        if (ke) run_force<MODE, false, true, FS>(s, st); else run_force<MODE, false, false, FS>(s, st);
     }
 }
 
-template <int MODE, bool E, bool KE, bool FS>
-void prep_one() {
-    set_smem(k_force64<MODE, E, KE, FS>);
-    if (E) {
-        if (!KE) set_smem(k_force64<MODE, true, false, FS, true>);
-    } else {
-        set_smem(k_force<MODE, KE, FS>);
-        set_smem(k_force_many<MODE, KE, FS>);
-        set_smem(k_force64_many<MODE, E, KE, FS>);
-    }
+template <int MODE>
+void run_force_mode(const DevSim& s, cudaStream_t st, bool energy, bool ke, bool fs) {
+    if (fs) run_force_fs<MODE, true>(s, st, energy, ke);
+    else run_force_fs<MODE, false>(s, st, energy, ke);
+}
+
+template <int MODE>
+void run_energy_sums(const DevSim& s, cudaStream_t st, bool fs) {
+    if (fs) k_force64<MODE, k64Sums, false, true><<<s.grid_cell, kBW * 32, smem64(s.smax), st>>>(s);
+    else k_force64<MODE, k64Sums, false, false><<<s.grid_cell, kBW * 32, smem64(s.smax), st>>>(s);
+}
+
+template <int MODE, bool FS>
+void prep_mode_fs() {
+    set_smem(k_force<MODE, false, FS>);
+    set_smem(k_force<MODE, true, FS>);
+    set_smem(k_force_many<MODE, false, FS>);
+    set_smem(k_force_many<MODE, true, FS>);
+    set_smem(k_force64_many<MODE, false, FS>);
+    set_smem(k_force64_many<MODE, true, FS>);
+    set_smem(k_force64<MODE, k64Force, false, FS>);
+    set_smem(k_force64<MODE, k64Force, true, FS>);
+    set_smem(k_force64<MODE, k64Force | k64Energy, false, FS>);
+    set_smem(k_force64<MODE, k64Energy, false, FS>);
+    set_smem(k_force64<MODE, k64Sums, false, FS>);
 }
 
 template <int MODE>
 void prep_mode() {
-    prep_one<MODE, false, false, false>();
-    prep_one<MODE, false, true, false>();
-    prep_one<MODE, true, false, false>();
-    prep_one<MODE, true, true, false>();
-    prep_one<MODE, false, false, true>();
-    prep_one<MODE, false, true, true>();
-    prep_one<MODE, true, false, true>();
-    prep_one<MODE, true, true, true>();
+    prep_mode_fs<MODE, false>();
+    prep_mode_fs<MODE, true>();
 }
 
 }  // namespace
@@ -1691,10 +1865,10 @@ bool prepare_force_kernels() {
 
 int force_blocks_per_sm(const DevSim& s) {
     int nb = 0;
-    size_t bytes = s.precision == BBMD_PREC_FP64 ? (size_t)(s.smax + 1) * sizeof(Pos64)
+    size_t bytes = s.precision == BBMD_PREC_FP64 ? smem64(s.smax)
                                                  : kStageBuffers * (size_t)(s.smax + 1) * sizeof(float4);
     if (s.precision == BBMD_PREC_FP64)
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_force64<0, false, true, false>, kBW * 32, bytes);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_force64<0, k64Force, true, false>, kBW * 32, bytes);
     else if (s.nbr_mode == BBMD_NBR_CELL)  // the stencil kernel is the step's force kernel
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_force<1, true, false>, kBW * 32, bytes);
     else
@@ -1715,6 +1889,13 @@ void launch_force(const DevSim& s, cudaStream_t st, bool energy, bool ke) {
     bool fs = s.pt.shift == BBMD_SHIFT_FORCE;
     if (s.nbr_mode == BBMD_NBR_VERLET) run_force_mode<0>(s, st, energy, ke, fs);
     run_force_mode<1>(s, st, energy, ke, fs);
+}
+
+// Energy and virial sums of the current positions (partials 1 and 2) alone, both precisions.
+void launch_energy_sums(const DevSim& s, cudaStream_t st) {
+    const bool fs = s.pt.shift == BBMD_SHIFT_FORCE;
+    if (s.nbr_mode == BBMD_NBR_VERLET) run_energy_sums<0>(s, st, fs);
+    run_energy_sums<1>(s, st, fs);
 }
 
 void launch_force_many(const ManySims& m, int total, bool fp64, bool cell, bool ke, bool fshift,
