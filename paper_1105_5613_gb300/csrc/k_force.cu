@@ -761,7 +761,9 @@ __device__ __forceinline__ void compact_streams(const float4* sm, int g0, int re
     }
     const int src = self - g0;
     const int sp = __shfl_sync(FULL, pos, src & 31);
-    if (src >= 0 && src < 32) cself = sp;
+    // (a group's lanes past the end of its row belong to other rows: with few particles a
+    // cell, the lane's own may be among them)
+    if (src >= 0 && src < 32 && self < re) cself = sp;
     fill[0] += __popc(bA);
     fill[1] += __popc(bB);
 }
