@@ -38,6 +38,7 @@ struct bbmd_sim {
     long long tune_step = 0, tune_rebuilds = 0;  // counters at the last shape tuning
     double mean_cell = 0.0;          // mean particles per cell
     std::vector<int> shapes;         // block shapes that fit (candidates of the autotuner)
+    int grid_shape = -1, grid_ctas = 0;  // one-launch step: block shape it was sized for, CTAs
     float shape_ms[4][2] = {};       // autotuner: per kShapes entry, force and list-build ms
 };
 
@@ -449,6 +450,36 @@ void begin_call(bbmd_sim* sim, int64_t nsteps, double dt, const bbmd_thermostat*
     sim->last_dt = dt;
 }
 
+// The one-launch kernels (k_step_grid, k_relax_grid) run a mixed-precision system's steps
+// where that is faster than a launch per phase:
+//   - time steps: while every block has a resident CTA (one wave of blocks).  Then the phases
+//     are short against the launches they replace; beyond it, the single kernel's fewer CTAs
+//     per SM cost more than its barriers save.  Microseconds a step, list mode, launches ->
+//     one launch, at T = 2: 4000 particles 59 -> 41, 32 000 64 -> 47, 48 000 69 -> 53, 108 000 in
+//     2 x 2 x 4 blocks (256 of 304 resident) 83 -> 72; the first sizes past one wave: 144 000
+//     in 2 x 2 x 4 (352) 104 -> 109, 108 000 in 2 x 2 x 1 (1024 of 608) 94 -> 100.
+//   - steepest descent (whose launches are not a captured graph) up to kGridRelaxMax particles:
+//     79 -> 25 at 4000, 99 -> 30 at 32 000, 222 -> 118 at 256 000, 314 -> 223 at 500 000.
+constexpr int64_t kGridRelaxMax = 500000;
+constexpr int64_t kGridSteps = 1024;  // steps per launch
+
+// CTAs of the one-launch kernels for this handle's shape (0 where they do not run), and
+// whether every block has one.
+int grid_step_grid(bbmd_sim* sim, bool* one_wave) {
+    if (sim->d.precision != BBMD_PREC_MIXED) return 0;
+    if (sim->grid_shape != sim->d.block_z) {
+        int coop = 0;
+        if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, sim->device) != cudaSuccess) {
+            cudaGetLastError();
+            coop = 0;
+        }
+        sim->grid_ctas = coop ? grid_step_ctas(sim->d, sim->nsm) : 0;
+        sim->grid_shape = sim->d.block_z;
+    }
+    *one_wave = sim->grid_ctas >= sim->d.nblocks;
+    return sim->grid_ctas;
+}
+
 // Apply a pending closing half kick to the stored velocities (before velocities are read
 // out or replaced, or positions move outside a step).
 void finish_velocities(bbmd_sim* sim) { launch_finish(sim->d, sim->st); }
@@ -631,6 +662,7 @@ bbmd_status bbmd_create(const bbmd_params* params, int64_t n, const double box[3
     D.disp = (float*)A(np * 4);
     D.mtop = (float2*)A((size_t)ncell * 8);
     D.sc = (DevScalars*)A(sizeof(DevScalars));
+    D.gsync = (uint32_t*)A((size_t)kSyncWords * kSyncStride * sizeof(uint32_t));
     sim->dout = (double*)A(64 * 8);
     if (!ok) {
         bbmd_destroy(sim);
@@ -765,6 +797,21 @@ bbmd_status bbmd_step(bbmd_sim* sim, int64_t nsteps, double dt, const bbmd_therm
         }
     }
     if (nsteps == 0) return BBMD_OK;
+    bool one_wave = false;
+    const int grid = grid_step_grid(sim, &one_wave);
+    if (grid > 0 && one_wave) {
+        // (a step call cannot be captured into a caller's graph, whichever path it takes)
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        CK(cudaStreamIsCapturing(sim->st, &cap));
+        if (cap != cudaStreamCaptureStatusNone) return fail(sim, BBMD_ERR_CUDA, "the stream is capturing");
+        begin_call(sim, nsteps, dt, nh ? th : nullptr);
+        LAUNCHED("begin");
+        for (int64_t k = 0; k < nsteps; k += kGridSteps) {
+            if (k > 0) launch_clear_grid_sync(sim->d, sim->st);
+            CK(launch_grid_step(sim->d, grid, (int)std::min(kGridSteps, nsteps - k), nh != 0, sim->st));
+        }
+        return BBMD_OK;
+    }
     if (!sim->graph[nh]) {
         bbmd_status r = build_graph(sim, nh);
         if (r != BBMD_OK) return r;
@@ -897,6 +944,18 @@ bbmd_status bbmd_minimize(bbmd_sim* sim, int64_t nsteps, double hmax, double dma
     if (!sim || nsteps < 0 || !(hmax > 0.0) || !(dmax > 0.0)) return BBMD_ERR_ARG;
     DeviceGuard dg(sim->device);
     finish_velocities(sim);
+    bool one_wave = false;
+    const int grid = sim->d.n <= kGridRelaxMax ? grid_step_grid(sim, &one_wave) : 0;
+    if (grid > 0) {
+        int64_t k = 0;
+        do {
+            launch_clear_grid_sync(sim->d, sim->st);
+            CK(launch_grid_relax(sim->d, grid, (int)std::min(kGridSteps, nsteps - k), hmax, dmax, sim->st));
+            k += kGridSteps;
+        } while (k < nsteps);
+        LAUNCHED("minimize");
+        return read_status(sim);
+    }
     for (int64_t k = 0; k < nsteps; ++k) {
         launch_force(sim->d, sim->st, false, false);
         launch_sd_step(sim->d, sim->st, hmax, dmax);

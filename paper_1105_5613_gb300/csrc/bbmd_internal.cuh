@@ -47,6 +47,11 @@ enum : int32_t {
     ST_TIMEOUT = 16,
 };
 
+// Words of the grid-wide barrier, each in a cache line of its own: arrivals, release count,
+// abort flag, and two slots for the largest |F|^2 of a steepest-descent step.
+enum { kSyncArrive = 0, kSyncRelease, kSyncAbort, kSyncMax0, kSyncMax1, kSyncWords };
+constexpr int kSyncStride = 32;
+
 struct DevScalars {
     double xi, eta;          // Nose-Hoover friction and its time integral
     double K;                // kinetic energy of the stored (full-step) velocities
@@ -116,6 +121,7 @@ struct alignas(16) DevSim {
     uint16_t* rows;          // per particle: rows (8 entries each) of its Verlet list
     double* partials;        // [kMaxPartials][4]
     DevScalars* sc;
+    uint32_t* gsync;         // grid-wide barrier of the one-launch step (kSyncWords words)
     int32_t grid_part;       // grid of per-particle grid-stride kernels
     int32_t grid_cell;       // grid of the force kernel (kBlockWarps warps per CTA)
     int32_t grid_list;       // grid of the list-build kernel
@@ -266,6 +272,9 @@ void launch_rebuild_chain(const DevSim& s, cudaStream_t st);
 //                  ke); ke: NH kinetic partials
 //   launch_energy_sums  energy and virial partials only
 //   launch_list_build  Verlet list build (gated)
+//   launch_grid_step   many whole steps of a small mixed-precision system in one cooperative
+//                  launch of grid_step_ctas CTAs (0: no such launch); launch_grid_relax the
+//                  same for steepest-descent steps
 #define BBMD_SHAPE_API(ns)                                                             \
     namespace ns {                                                                     \
     bool prepare_force_kernels();                                                      \
@@ -279,6 +288,10 @@ void launch_rebuild_chain(const DevSim& s, cudaStream_t st);
     void launch_force(const DevSim& s, cudaStream_t st, bool energy, bool ke);         \
     void launch_energy_sums(const DevSim& s, cudaStream_t st);                         \
     void launch_list_build(const DevSim& s, cudaStream_t st);                          \
+    int grid_step_ctas(const DevSim& s, int nsm);                                      \
+    cudaError_t launch_grid_step(const DevSim& s, int grid, int nsteps, bool ke, cudaStream_t st); \
+    cudaError_t launch_grid_relax(const DevSim& s, int grid, int nsteps, double hmax, double dmax, \
+                                  cudaStream_t st);                                    \
     }
 BBMD_SHAPE_API(z1)
 BBMD_SHAPE_API(z2)
@@ -340,6 +353,16 @@ inline void launch_force(const DevSim& s, cudaStream_t st, bool energy, bool ke)
 inline void launch_energy_sums(const DevSim& s, cudaStream_t st) {
     BBMD_SHAPE_DISPATCH(s.block_z, launch_energy_sums(s, st))
 }
+inline int grid_step_ctas(const DevSim& s, int nsm) {
+    BBMD_SHAPE_DISPATCH(s.block_z, grid_step_ctas(s, nsm))
+}
+inline cudaError_t launch_grid_step(const DevSim& s, int grid, int nsteps, bool ke, cudaStream_t st) {
+    BBMD_SHAPE_DISPATCH(s.block_z, launch_grid_step(s, grid, nsteps, ke, st))
+}
+inline cudaError_t launch_grid_relax(const DevSim& s, int grid, int nsteps, double hmax, double dmax,
+                                     cudaStream_t st) {
+    BBMD_SHAPE_DISPATCH(s.block_z, launch_grid_relax(s, grid, nsteps, hmax, dmax, st))
+}
 inline void launch_list_build(const DevSim& s, cudaStream_t st) {
     BBMD_SHAPE_DISPATCH(s.block_z, launch_list_build(s, st))
 }
@@ -368,6 +391,7 @@ void launch_init_fcc(const DevSim& s, cudaStream_t st, int m, double jitter, uin
 void launch_init_mb(const DevSim& s, cudaStream_t st, double T0, uint64_t seed, double* tmp3);
 void launch_sd_step(const DevSim& s, cudaStream_t st, double hmax, double dmax);
 void launch_clear_rebuild(const DevSim& s, cudaStream_t st);
+void launch_clear_grid_sync(const DevSim& s, cudaStream_t st);
 // unwrapped positions by id (3 x n doubles) into ref / MSD and F_s against ref
 void launch_set_ref(const DevSim& s, cudaStream_t st, double* ref);
 void launch_msd_fs(const DevSim& s, cudaStream_t st, const double* ref, double kvec,

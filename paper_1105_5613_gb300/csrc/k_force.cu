@@ -1269,6 +1269,173 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
     });
 }
 
+// ------------------------------------------------------- one-launch step ----
+// A small system's step is a chain of kernels of a few microseconds each: 16 launches, most
+// of them gated off, took 54 us for 4000 particles.  One cooperative launch instead runs
+// many whole steps: every phase is the body that the kernels of its own run (with their CTA
+// index and count where a sum depends on it, so the states are the same bit for bit), and
+// the phases are kept apart by a grid-wide barrier (about 1.3 us) only where one is needed:
+// two in a step in which nothing came near the rebuild trigger, two more for the trigger,
+// seven more for a rebuild.  Where it is used and what it measured: grid_step_grid
+// (bbmd_api.cu).  At 4000 particles (2 x 2 x 1 blocks, one per SM) a step's 41 us are forces 14
+// (two rounds of chunks on four warps), barriers 6, finalize 6, integrate 2, and 0.2 rebuilds
+// of 70 (its list build 45).
+#include "sort_bodies.cuh"
+#include "step_bodies.cuh"
+
+__device__ __forceinline__ unsigned long long globaltimer_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+constexpr unsigned long long kGridWaitNs = 2000000000ull;  // a barrier wait gives up after it
+
+#ifndef BBMD_GRID_MIN_BLOCKS
+#define BBMD_GRID_MIN_BLOCKS (BBMD_BLOCK_Z == 1 ? 4 : 2)
+#endif
+
+// Barrier over the CTAs of the launch; gen counts the barriers passed.  With `last` set, the
+// last CTA to arrive runs on_last before the others go on.  Every CTA is resident
+// (cooperative launch), so a wait ends; should one not end within kGridWaitNs, the CTA
+// raises the abort flag and ST_TIMEOUT, and every CTA leaves (false) at its next barrier.
+template <class OnLast>
+__device__ __forceinline__ bool grid_barrier(const DevSim& s, unsigned& gen, bool last, OnLast on_last) {
+    __shared__ int verdict;  // 0: abort, 1: go on, 2: this CTA arrived last
+    volatile uint32_t* const w = s.gsync;
+    ++gen;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const unsigned target = gen * gridDim.x;
+        const bool mine = atomicAdd(&s.gsync[kSyncArrive * kSyncStride], 1u) + 1u == target;
+        int v = 1;
+        if (last && mine) {
+            v = 2;
+        } else {
+            const int word = (last ? kSyncRelease : kSyncArrive) * kSyncStride;
+            const unsigned want = last ? gen : target;
+            unsigned long long t0 = 0;
+            for (unsigned it = 0; w[word] < want; ++it) {
+                if ((it & 63u) != 63u) continue;
+                if (t0 == 0) t0 = globaltimer_ns();
+                if (w[kSyncAbort * kSyncStride] != 0u || globaltimer_ns() - t0 > kGridWaitNs) {
+                    w[kSyncAbort * kSyncStride] = 1u;
+                    set_status(s, ST_TIMEOUT);
+                    v = 0;
+                    break;
+                }
+            }
+        }
+        __threadfence();
+        verdict = v;
+    }
+    __syncthreads();
+    const int v = verdict;
+    if (v == 2) {
+        on_last();
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            w[kSyncRelease * kSyncStride] = gen;
+        }
+    }
+    __syncthreads();  // (verdict is written again at the next barrier)
+    // data of earlier phases, written by other CTAs, is read by bulk copies (the async
+    // proxy) as well as by ordinary loads
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    return v != 0;
+}
+
+__device__ __forceinline__ bool grid_barrier(const DevSim& s, unsigned& gen) {
+    return grid_barrier(s, gen, false, [] {});
+}
+
+// The rebuild after its flag is up and the cell counts are zero: sort chain and list build.
+// on_last runs once at the end.
+template <class OnLast>
+__device__ __forceinline__ bool grid_rebuild(const DevSim& s, unsigned& gen, OnLast on_last) {
+    const int lb = (int)blockIdx.x, lg = (int)gridDim.x;
+    clear_list_flags(s, lb);
+    bin_body(s, lb, lg);
+    if (!grid_barrier(s, gen)) return false;
+    scan_cta_body(s, lb, lg);
+    if (!grid_barrier(s, gen)) return false;
+    scatter_body(s, lb, lg);
+    if (!grid_barrier(s, gen)) return false;
+    cellsort_body(s, lb, lg);
+    if (!grid_barrier(s, gen)) return false;
+    gather_body(s, lb, lg);
+    if (!grid_barrier(s, gen)) return false;
+    copyback_body(s, lb, lg);
+    if (s.nbr_mode == BBMD_NBR_VERLET) {
+        if (!grid_barrier(s, gen)) return false;
+        for (int b = lb; b < s.grid_list; b += lg) list_build_body(s, b, s.grid_list);
+    }
+    return grid_barrier(s, gen, true, on_last);
+}
+
+// Forces with the CTA index and count of the force kernel's own launch.
+template <bool KE, bool FSHIFT>
+__device__ __forceinline__ void grid_force(const DevSim& s) {
+    for (int b = (int)blockIdx.x; b < s.grid_cell; b += (int)gridDim.x) {
+        force_body<0, KE, FSHIFT, false>(s, b, s.grid_cell);
+        force_body<1, KE, FSHIFT, false>(s, b, s.grid_cell);
+    }
+}
+
+template <bool KE, bool FSHIFT>
+__global__ void __launch_bounds__(kBW * 32, BBMD_GRID_MIN_BLOCKS) k_step_grid(DevSim s, int nsteps) {
+    const int lb = (int)blockIdx.x, lg = (int)gridDim.x;
+    unsigned gen = 0;
+    for (int step = 0; step < nsteps; ++step) {
+        integrate_body<false>(s, lb, lg);
+        if (!grid_barrier(s, gen)) return;
+        if (*(volatile int*)&s.sc->near) {
+            celltop_body(s, lb, lg);
+            zero_counts(s, lb, lg);
+            if (!grid_barrier(s, gen)) return;
+            check_body(s, lb, lg);
+            if (!grid_barrier(s, gen)) return;
+            if (*(volatile int*)&s.sc->rebuild)
+                if (!grid_rebuild(s, gen, [] {})) return;
+        }
+        grid_force<KE, FSHIFT>(s);
+        if (!grid_barrier(s, gen, true, [&] { finalize_body(s, KE ? 1 : 0); })) return;
+    }
+}
+
+// Steepest descent: x += h F, h = min(hmax, dmax / max |F|), nsteps times, then the forces.
+template <bool FSHIFT>
+__global__ void __launch_bounds__(kBW * 32, BBMD_GRID_MIN_BLOCKS)
+    k_relax_grid(DevSim s, int nsteps, double hmax, double dmax) {
+    const int lb = (int)blockIdx.x, lg = (int)gridDim.x;
+    unsigned gen = 0;
+    for (int step = 0; step < nsteps; ++step) {
+        // (squares of FP32 forces are not negative: their bits order like the values)
+        uint32_t* const slot = &s.gsync[(kSyncMax0 + (step & 1)) * kSyncStride];
+        grid_force<false, FSHIFT>(s);
+        if (!grid_barrier(s, gen)) return;
+        const float m = maxf_body(s, lb, lg);
+        if ((threadIdx.x & 31) == 0) atomicMax(slot, __float_as_uint(m));
+        zero_counts(s, lb, lg);
+        if (!grid_barrier(s, gen)) return;
+        const double fm = sqrt((double)__uint_as_float(*(volatile uint32_t*)slot));
+        if (lb == 0 && threadIdx.x == 0) s.gsync[(kSyncMax0 + ((step + 1) & 1)) * kSyncStride] = 0u;
+        sd_move_body<false>(s, lb, lg, fm, hmax, dmax);
+        if (!grid_barrier(s, gen)) return;
+        if (*(volatile int*)&s.sc->rebuild)
+            if (!grid_rebuild(s, gen, [&] {
+                    if (threadIdx.x == 0) {
+                        s.sc->n_rebuilds += 1;
+                        s.sc->rebuild = 0;
+                    }
+                }))
+                return;
+    }
+    grid_force<false, FSHIFT>(s);
+}
+
 // ------------------------------------------------------- persistent batch step ----
 // One cooperative launch advances every replica of a batch by many steps.  The step of
 // each replica is a chain of phases (integrate, the two trigger passes, the seven sort
@@ -1283,15 +1450,6 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
 // overlap; an item waits only on items handed out before it, and every CTA is resident,
 // so the queue always advances.
 #if BBMD_BLOCK_Z == BBMD_PERSIST_Z
-#include "sort_bodies.cuh"
-#include "step_bodies.cuh"
-
-__device__ __forceinline__ unsigned long long globaltimer_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
 // Raise the abort flag and ST_TIMEOUT on every replica.
 __device__ __forceinline__ void persistent_abort(const PersistentStep& a) {
     if (atomicExch(a.abort, 1) == 0)
@@ -1862,6 +2020,12 @@ bool prepare_force_kernels() {
     prep_mode<1>();
     set_smem(k_list_build);
     set_smem(k_list_build_many);
+    set_smem(k_step_grid<false, false>);
+    set_smem(k_step_grid<true, false>);
+    set_smem(k_step_grid<false, true>);
+    set_smem(k_step_grid<true, true>);
+    set_smem(k_relax_grid<false>);
+    set_smem(k_relax_grid<true>);
     return g_smem_ok;
 }
 
@@ -1942,6 +2106,41 @@ void launch_list_build(const DevSim& s, cudaStream_t st) {
     // staging buffer(s), each: staged region + sentinel record
     size_t bytes = kStageBuffers * (size_t)(s.smax + 1) * sizeof(float4);
     k_list_build<<<s.grid_list, kBW * 32, bytes, st>>>(s);
+}
+
+// CTAs of the one-launch step: enough for every block and for 256 particles a CTA, at most
+// what is resident at once.
+int grid_step_ctas(const DevSim& s, int nsm) {
+    int nb = 0;
+    const size_t bytes = kStageBuffers * (size_t)(s.smax + 1) * sizeof(float4);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step_grid<true, true>, kBW * 32, bytes) !=
+        cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    int64_t want = (s.n + 255) / 256;
+    if (want < s.nblocks) want = s.nblocks;
+    return (int)(want < (int64_t)nb * nsm ? want : (int64_t)nb * nsm);
+}
+
+cudaError_t launch_grid_step(const DevSim& s, int grid, int nsteps, bool ke, cudaStream_t st) {
+    DevSim a = s;
+    void* params[] = {&a, &nsteps};
+    const bool fs = s.pt.shift == BBMD_SHIFT_FORCE;
+    const void* fn = ke ? (fs ? (const void*)k_step_grid<true, true> : (const void*)k_step_grid<true, false>)
+                        : (fs ? (const void*)k_step_grid<false, true> : (const void*)k_step_grid<false, false>);
+    const size_t bytes = kStageBuffers * (size_t)(s.smax + 1) * sizeof(float4);
+    return cudaLaunchCooperativeKernel(fn, grid, kBW * 32, params, bytes, st);
+}
+
+cudaError_t launch_grid_relax(const DevSim& s, int grid, int nsteps, double hmax, double dmax,
+                              cudaStream_t st) {
+    DevSim a = s;
+    void* params[] = {&a, &nsteps, &hmax, &dmax};
+    const void* fn = s.pt.shift == BBMD_SHIFT_FORCE ? (const void*)k_relax_grid<true>
+                                                    : (const void*)k_relax_grid<false>;
+    const size_t bytes = kStageBuffers * (size_t)(s.smax + 1) * sizeof(float4);
+    return cudaLaunchCooperativeKernel(fn, grid, kBW * 32, params, bytes, st);
 }
 
 #if BBMD_BLOCK_Z == BBMD_PERSIST_Z

@@ -28,6 +28,11 @@ constexpr unsigned FULL = 0xffffffffu;
 
 #include "step_bodies.cuh"
 
+// The words of the grid-wide barrier (k_force.cu) start at zero in every launch.
+__device__ __forceinline__ void clear_grid_sync(const DevSim& s) {
+    for (int k = 0; k < kSyncWords; ++k) s.gsync[k * kSyncStride] = 0u;
+}
+
 // Start of a call.  If the previous call's closing half kick and Nose-Hoover scale are
 // still pending (the velocities were not finished: sc->pending), they are carried into
 // the first velocity update of this call, which applies s_end (v + h F) and this call's
@@ -58,7 +63,10 @@ __global__ void k_begin(DevSim s, int64_t nsteps, double dt, int kind, double T0
         sc->s_next = s_carry;
     }
     sc->s_end = 1.0;
+    clear_grid_sync(s);
 }
+
+__global__ void k_clear_grid_sync(DevSim s) { clear_grid_sync(s); }
 
 // Four CTAs per SM (64 registers; the compiler would take 92 and fit two): the kernel is
 // bound by HBM, and more resident warps keep more of its loads in flight.
@@ -309,13 +317,7 @@ __global__ void __launch_bounds__(kThreads) k_mb_scale(DevSim s, const double* t
 // ------------------------------------------------------------ steepest descent ----
 
 __global__ void __launch_bounds__(kThreads) k_maxf(DevSim s) {
-    float m = 0.f;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < s.n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        float4 F = s.F[i];
-        m = fmaxf(m, F.x * F.x + F.y * F.y + F.z * F.z);
-    }
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(FULL, m, o));
+    const float m = maxf_body(s, (int)blockIdx.x, (int)gridDim.x);
     __shared__ float red[kThreads / 32];
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
     __syncthreads();
@@ -335,38 +337,7 @@ __global__ void k_maxf_final(DevSim s, int nb) {
 
 template <bool FP64>
 __global__ void __launch_bounds__(kThreads) k_sd_move(DevSim s, double hmax, double dmax) {
-    double fm = s.sc->maxf;
-    double h = hmax;
-    if (fm > 0.0 && dmax / fm < h) h = dmax / fm;
-    bool need = false;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < s.n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        float4 rb = s.relb[i];
-        int wb = __float_as_int(rb.w);
-        int c = wb >> 1;
-        int a3[3] = {c % s.nc[0], (c / s.nc[0]) % s.nc[1], c / (s.nc[0] * s.nc[1])};
-        float4 F = s.F[i];
-        float Fv[3] = {F.x, F.y, F.z};
-        float r[3];
-        for (int d = 0; d < 3; ++d) {
-            int64_t idx = d * s.npad + i;
-            double f = FP64 ? s.Fd[idx] : (double)Fv[d];
-            long long x = (long long)s.x[idx] + __double2ll_rn(ldexp(h * f, s.kexp));
-            if (x >= s.Lfix[d]) {
-                x -= s.Lfix[d];
-                s.img[idx] += 1;
-            } else if (x < 0) {
-                x += s.Lfix[d];
-                s.img[idx] -= 1;
-            }
-            s.x[idx] = (uint64_t)x;
-            r[d] = i64_to_f32(min_image(x - frame_axis(a3[d], s.D[d]), s.Lfix[d])) * s.sx;
-        }
-        s.rel[i] = make_float4(r[0], r[1], r[2], (float)(wb & 1));
-        float ex = r[0] - rb.x, ey = r[1] - rb.y, ez = r[2] - rb.z;
-        if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) > s.disp2) need = true;
-    }
-    if (__any_sync(FULL, need) && (threadIdx.x & 31) == 0) s.sc->rebuild = 1;
+    sd_move_body<FP64>(s, (int)blockIdx.x, (int)gridDim.x, s.sc->maxf, hmax, dmax);
 }
 
 __global__ void k_clear_rebuild(DevSim s) {
@@ -693,6 +664,8 @@ void launch_sd_step(const DevSim& s, cudaStream_t st, double hmax, double dmax) 
     else
         k_sd_move<false><<<s.grid_part, kThreads, 0, st>>>(s, hmax, dmax);
 }
+
+void launch_clear_grid_sync(const DevSim& s, cudaStream_t st) { k_clear_grid_sync<<<1, 1, 0, st>>>(s); }
 
 void launch_clear_rebuild(const DevSim& s, cudaStream_t st) { k_clear_rebuild<<<1, 1, 0, st>>>(s); }
 

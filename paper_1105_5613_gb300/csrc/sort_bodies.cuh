@@ -14,17 +14,26 @@ __host__ __device__ __forceinline__ int scan_chunks(const DevSim& s) {
     return (int)((s.ncell + kScanChunk - 1) / kScanChunk);
 }
 
-__device__ __forceinline__ void zero_body(const DevSim& s, int lb, int lg) {
-    if (!s.sc->rebuild) return;
-    if (lb == 0 && threadIdx.x == 0) {  // the list build of this rebuild sets them afresh
+// Start of a rebuild: the list build sets the cut-list flags afresh.
+__device__ __forceinline__ void clear_list_flags(const DevSim& s, int lb) {
+    if (lb == 0 && threadIdx.x == 0) {
         s.sc->list_short = 0;
         s.sc->max_len = 0;
     }
+}
+
+__device__ __forceinline__ void zero_counts(const DevSim& s, int lb, int lg) {
     for (int64_t c = lb * (int64_t)blockDim.x + threadIdx.x; c <= s.ncell;
          c += (int64_t)lg * blockDim.x) {
         s.count[c] = 0;
         s.cursor[c] = 0;
     }
+}
+
+__device__ __forceinline__ void zero_body(const DevSim& s, int lb, int lg) {
+    if (!s.sc->rebuild) return;
+    clear_list_flags(s, lb);
+    zero_counts(s, lb, lg);
 }
 
 __device__ __forceinline__ void bin_body(const DevSim& s, int lb, int lg) {

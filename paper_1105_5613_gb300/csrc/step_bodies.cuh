@@ -225,23 +225,24 @@ __device__ __forceinline__ void check_body(const DevSim& s, int lb, int lg) {
 }
 
 // Sum partials[q][0 .. nb) for q < nq (at most 8) in a fixed order: a strided sum per
-// thread, a butterfly over each warp's lanes, then the warps in order (one CTA of at most
-// 256 threads).
+// thread of kStepThreads, a butterfly over each warp's lanes, then the warps in order (one
+// CTA; a smaller one takes the warps in turn, so the sum does not depend on its size).
 __device__ void sum_partials(const DevSim& s, int nb, int nq, double* out) {
     __shared__ double red[8][kStepThreads / 32];
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (int q = 0; q < nq; ++q) {
-        double t = 0.0;
-        for (int b = threadIdx.x; b < nb; b += blockDim.x) t += s.partials[q * kMaxPartials + b];
+    const int lane = threadIdx.x & 31;
+    for (int w = threadIdx.x >> 5; w < kStepThreads / 32; w += blockDim.x >> 5)
+        for (int q = 0; q < nq; ++q) {
+            double t = 0.0;
+            for (int b = w * 32 + lane; b < nb; b += kStepThreads) t += s.partials[q * kMaxPartials + b];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kStepFull, t, o);
-        if (lane == 0) red[q][w] = t;
-    }
+            for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kStepFull, t, o);
+            if (lane == 0) red[q][w] = t;
+        }
     __syncthreads();
     if (threadIdx.x == 0)
         for (int q = 0; q < nq; ++q) {
             double t = 0.0;
-            for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += red[q][k];
+            for (int k = 0; k < kStepThreads / 32; ++k) t += red[q][k];
             out[q] = t;
         }
     __syncthreads();
@@ -283,3 +284,52 @@ __device__ __forceinline__ void finalize_body(const DevSim& s, int ke) {
     }
 }
 
+// ------------------------------------------------------------ steepest descent ----
+
+// Largest |F|^2 of the CTA's particles (every thread returns its warp's; F as FP32).
+__device__ __forceinline__ float maxf_body(const DevSim& s, int lb, int lg) {
+    float m = 0.f;
+    for (int64_t i = lb * (int64_t)blockDim.x + threadIdx.x; i < s.n; i += (int64_t)lg * blockDim.x) {
+        const float4 F = s.F[i];
+        m = fmaxf(m, F.x * F.x + F.y * F.y + F.z * F.z);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(kStepFull, m, o));
+    return m;
+}
+
+// x += h F with h = min(hmax, dmax / fm), fm the largest |F|; raises the rebuild flag.
+template <bool FP64>
+__device__ __forceinline__ void sd_move_body(const DevSim& s, int lb, int lg, double fm, double hmax,
+                                             double dmax) {
+    double h = hmax;
+    if (fm > 0.0 && dmax / fm < h) h = dmax / fm;
+    bool need = false;
+    for (int64_t i = lb * (int64_t)blockDim.x + threadIdx.x; i < s.n; i += (int64_t)lg * blockDim.x) {
+        float4 rb = s.relb[i];
+        int wb = __float_as_int(rb.w);
+        int c = wb >> 1;
+        int a3[3] = {c % s.nc[0], (c / s.nc[0]) % s.nc[1], c / (s.nc[0] * s.nc[1])};
+        float4 F = s.F[i];
+        float Fv[3] = {F.x, F.y, F.z};
+        float r[3];
+        for (int d = 0; d < 3; ++d) {
+            int64_t idx = d * s.npad + i;
+            double f = FP64 ? s.Fd[idx] : (double)Fv[d];
+            long long x = (long long)s.x[idx] + __double2ll_rn(ldexp(h * f, s.kexp));
+            if (x >= s.Lfix[d]) {
+                x -= s.Lfix[d];
+                s.img[idx] += 1;
+            } else if (x < 0) {
+                x += s.Lfix[d];
+                s.img[idx] -= 1;
+            }
+            s.x[idx] = (uint64_t)x;
+            r[d] = i64_to_f32(min_image(x - frame_axis(a3[d], s.D[d]), s.Lfix[d])) * s.sx;
+        }
+        s.rel[i] = make_float4(r[0], r[1], r[2], (float)(wb & 1));
+        float ex = r[0] - rb.x, ey = r[1] - rb.y, ez = r[2] - rb.z;
+        if (fmaf(ex, ex, fmaf(ey, ey, ez * ez)) > s.disp2) need = true;
+    }
+    if (__any_sync(kStepFull, need) && (threadIdx.x & 31) == 0) s.sc->rebuild = 1;
+}
