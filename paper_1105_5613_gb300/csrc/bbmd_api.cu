@@ -36,6 +36,7 @@ struct bbmd_sim {
     int nsm = 1;
     int graph_gen = 0;               // bumped whenever captured launch arguments go stale
     long long tune_step = 0, tune_rebuilds = 0;  // counters at the last shape tuning
+    int64_t n_species[2] = {0, 0};   // particles of each species (fixed at creation)
     double mean_cell = 0.0;          // mean particles per cell
     std::vector<int> shapes;         // block shapes that fit (candidates of the autotuner)
     int grid_shape = -1, grid_ctas = 0;  // one-launch step: block shape it was sized for, CTAs
@@ -516,11 +517,14 @@ bbmd_status bbmd_create(const bbmd_params* params, int64_t n, const double box[3
         return vs;
     }
     if (!species) return BBMD_ERR_ARG;
-    for (int64_t i = 0; i < n; ++i)
+    int64_t n_b = 0;
+    for (int64_t i = 0; i < n; ++i) {
         if (species[i] > 1) {
             std::fprintf(stderr, "bbmd_create: species labels must be 0 or 1\n");
             return BBMD_ERR_ARG;
         }
+        n_b += species[i];
+    }
     if (!(T0 >= 0.0)) return BBMD_ERR_ARG;
     if (!all_finite(pos, 3 * n) || !all_finite(vel, 3 * n)) {
         std::fprintf(stderr, "bbmd_create: non-finite positions or velocities\n");
@@ -533,6 +537,8 @@ bbmd_status bbmd_create(const bbmd_params* params, int64_t n, const double box[3
     }
     bbmd_sim* sim = new bbmd_sim();
     sim->P = *params;
+    sim->n_species[0] = n - n_b;
+    sim->n_species[1] = n_b;
     if (cudaGetDevice(&sim->device) != cudaSuccess) {
         cudaGetLastError();
         delete sim;
@@ -915,11 +921,7 @@ bbmd_status bbmd_observe(bbmd_sim* sim, uint32_t mask, const bbmd_obs_args* args
         }
     }
     if (mask & BBMD_OBS_GR) {
-        double Ns[2] = {0.0, 0.0};
-        // species counts from the pair totals are not exact for empty shells; count directly
-        std::vector<uint8_t> spc((size_t)D.n);
-        CK(cudaMemcpy(spc.data(), D.sp, (size_t)D.n, cudaMemcpyDeviceToHost));
-        for (int64_t i = 0; i < D.n; ++i) Ns[spc[(size_t)i]] += 1.0;
+        const double Ns[2] = {(double)sim->n_species[0], (double)sim->n_species[1]};
         double dr = rmax / (double)nbins;
         const double pi = 3.14159265358979323846;
         for (int a = 0; a < 2; ++a)
