@@ -23,7 +23,8 @@ struct bbmd_sim {
     std::vector<std::pair<void*, size_t>> blocks;
     int64_t bytes = 0;
     std::string err;
-    double* dout = nullptr;          // device scratch for reduction results (64 doubles)
+    double* dout = nullptr;          // results of an observation (64 doubles on the device)
+    bool pending = false;            // a step call may have left its closing half kick pending
     cudaGraphExec_t graph[2] = {nullptr, nullptr};  // [thermostatted]
     int32_t* gr_scratch = nullptr;
     int64_t gr_scratch_n = 0;
@@ -316,11 +317,14 @@ bbmd_status grow_lists(bbmd_sim* sim) {
 }
 
 // The status word: grow cut lists if needed, then report the sticky bits.  `known`: the
-// status word the caller has just read after synchronising (skips two round trips unless
-// lists were cut), or -1.
+// status word the caller has just read after synchronising, or -1.
 bbmd_status read_status(bbmd_sim* sim, int known = -1) {
     int st = known;
-    if (known < 0 || (known & ST_LIST_OVERFLOW)) {
+    if (known < 0) {
+        CK(cudaMemcpyAsync(&st, &sim->d.sc->status, sizeof(int), cudaMemcpyDeviceToHost, sim->st));
+        CK(cudaStreamSynchronize(sim->st));
+    }
+    if (st & ST_LIST_OVERFLOW) {
         bbmd_status g = grow_lists(sim);
         if (g != BBMD_OK) return g;
         CK(cudaMemcpyAsync(&st, &sim->d.sc->status, sizeof(int), cudaMemcpyDeviceToHost, sim->st));
@@ -427,10 +431,8 @@ bbmd_status autotune_shape(bbmd_sim* sim, float rebuild_rate = 0.25f) {
 bbmd_status refresh_forces_and_K(bbmd_sim* sim) {
     launch_force(sim->d, sim->st, false, false);
     launch_state_sums(sim->d, sim->st);
-    launch_reduce_partials(sim->d, sim->st, 4, sim->dout);
+    launch_set_K(sim->d, sim->st);  // sc->K <- KE of the stored velocities
     LAUNCHED("forces");
-    // sc->K <- KE of the stored velocities
-    CK(cudaMemcpyAsync(&sim->d.sc->K, sim->dout, sizeof(double), cudaMemcpyDeviceToDevice, sim->st));
     return BBMD_OK;
 }
 
@@ -446,9 +448,10 @@ void free_graphs(bbmd_sim* sim) {
 // Start of a step call: the closing half kick a previous call left pending is carried into
 // this call's first update when dt is unchanged; otherwise it is applied now.
 void begin_call(bbmd_sim* sim, int64_t nsteps, double dt, const bbmd_thermostat* th) {
-    if (dt != sim->last_dt) launch_finish(sim->d, sim->st);
+    if (dt != sim->last_dt) finish_velocities(sim);
     launch_begin(sim->d, sim->st, nsteps, dt, th);
     sim->last_dt = dt;
+    sim->pending = true;
 }
 
 // The one-launch kernels (k_step_grid, k_relax_grid) run a mixed-precision system's steps
@@ -483,7 +486,10 @@ int grid_step_grid(bbmd_sim* sim, bool* one_wave) {
 
 // Apply a pending closing half kick to the stored velocities (before velocities are read
 // out or replaced, or positions move outside a step).
-void finish_velocities(bbmd_sim* sim) { launch_finish(sim->d, sim->st); }
+void finish_velocities(bbmd_sim* sim) {
+    if (sim->pending) launch_finish(sim->d, sim->st);
+    sim->pending = false;
+}
 
 bbmd_status build_graph(bbmd_sim* sim, int nh) {
     cudaGraph_t g;
@@ -682,40 +688,19 @@ bbmd_status bbmd_create(const bbmd_params* params, int64_t n, const double box[3
         return BBMD_ERR_CUDA;
     }
 
-    // initial state (id order), through temporary device buffers
+    // initial state (id order), staged in the arrays that the first rebuild reorders into
     bbmd_status rc = BBMD_OK;
-    double* tpos = nullptr;
-    double* tvel = nullptr;
-    if (cudaMemcpyAsync(D.sp2, species, (size_t)n, cudaMemcpyHostToDevice, sim->st) != cudaSuccess)
+    double* const tpos = reinterpret_cast<double*>(D.x2);
+    double* const tvel = reinterpret_cast<double*>(D.v2);
+    if (cudaMemcpyAsync(D.sp2, species, (size_t)n, cudaMemcpyHostToDevice, sim->st) != cudaSuccess ||
+        (pos && cudaMemcpyAsync(tpos, pos, 3 * n * 8, cudaMemcpyHostToDevice, sim->st) != cudaSuccess) ||
+        (vel && cudaMemcpyAsync(tvel, vel, 3 * n * 8, cudaMemcpyHostToDevice, sim->st) != cudaSuccess))
         rc = BBMD_ERR_CUDA;
-    if (rc == BBMD_OK && pos) {
-        tpos = (double*)dev_alloc(sim, 3 * n * 8);
-        if (!tpos) rc = BBMD_ERR_OOM;
-        else if (cudaMemcpyAsync(tpos, pos, 3 * n * 8, cudaMemcpyHostToDevice, sim->st) != cudaSuccess)
-            rc = BBMD_ERR_CUDA;
-    }
-    if (rc == BBMD_OK && vel) {
-        tvel = (double*)dev_alloc(sim, 3 * n * 8);
-        if (!tvel) rc = BBMD_ERR_OOM;
-        else if (cudaMemcpyAsync(tvel, vel, 3 * n * 8, cudaMemcpyHostToDevice, sim->st) != cudaSuccess)
-            rc = BBMD_ERR_CUDA;
-    }
     if (rc == BBMD_OK) {
-        launch_pack_state(D, sim->st, tpos, tvel, nullptr, false);
+        launch_pack_state(D, sim->st, pos ? tpos : nullptr, vel ? tvel : nullptr, nullptr, false);
         if (!pos) launch_init_fcc(D, sim->st, m_fcc, params->init_jitter, seed);
-        if (!vel) {
-            double* tmp = (double*)dev_alloc(sim, (3 * n + 16) * 8);
-            if (!tmp) rc = BBMD_ERR_OOM;
-            else {
-                launch_init_mb(D, sim->st, T0, seed, tmp);
-                cudaStreamSynchronize(sim->st);
-                dev_free(sim, tmp);
-            }
-        }
+        if (!vel) launch_init_mb(D, sim->st, T0, seed, tvel, sim->dout);
     }
-    if (rc == BBMD_OK && cudaStreamSynchronize(sim->st) != cudaSuccess) rc = BBMD_ERR_CUDA;
-    dev_free(sim, tpos);
-    dev_free(sim, tvel);
     if (rc == BBMD_OK) rc = rebuild_now(sim);
     if (rc == BBMD_OK) rc = grow_lists(sim);  // lists longer than the capacity asked for
     if (rc == BBMD_OK && sim->shapes.size() > 1) rc = autotune_shape(sim);
@@ -837,12 +822,10 @@ bbmd_status bbmd_observe(bbmd_sim* sim, uint32_t mask, const bbmd_obs_args* args
     if (nbins > 4096) return fail(sim, BBMD_ERR_ARG, "nbins <= 4096");
     DevSim& D = sim->d;
     // kinetic energy and momentum
+    const bool energy = (mask & (BBMD_OBS_ENERGY | BBMD_OBS_VIRIAL)) != 0;
     launch_state_sums(D, sim->st);
-    launch_reduce_partials(D, sim->st, 4, sim->dout);
-    if (mask & (BBMD_OBS_ENERGY | BBMD_OBS_VIRIAL)) {
-        launch_energy_sums(D, sim->st);
-        launch_reduce_partials(D, sim->st, -3, sim->dout + 8);
-    }
+    if (energy) launch_energy_sums(D, sim->st);
+    launch_observe_sums(D, sim->st, energy, sim->dout);
     const int origin = args ? args->origin : 0;
     if (origin < 0 || origin >= BBMD_MAX_ORIGINS)
         return fail(sim, BBMD_ERR_ARG, "origin must be in [0, BBMD_MAX_ORIGINS)");
@@ -884,11 +867,11 @@ bbmd_status bbmd_observe(bbmd_sim* sim, uint32_t mask, const bbmd_obs_args* args
                            sim->st));
     }
     LAUNCHED("observe");
-    double h[32];
+    double h[64];
     DevScalars scl;
     CK(cudaMemcpyAsync(h, sim->dout, sizeof(h), cudaMemcpyDeviceToHost, sim->st));
-    CK(cudaMemcpyAsync(&scl, D.sc, sizeof(scl), cudaMemcpyDeviceToHost, sim->st));
     CK(cudaStreamSynchronize(sim->st));
+    std::memcpy(&scl, h + kOutScalars, sizeof(scl));
     bbmd_status rs = read_status(sim, scl.status);
     if (rs != BBMD_OK) return rs;
     double Vol = sim->box[0] * sim->box[1] * sim->box[2];
@@ -970,32 +953,29 @@ bbmd_status bbmd_minimize(bbmd_sim* sim, int64_t nsteps, double hmax, double dma
     return read_status(sim);
 }
 
+// The arrays a rebuild reorders into (x2, v2, img2) are free between rebuilds: transfers in id
+// order stage there, so that no call allocates (cudaMalloc and cudaFree took most of a small
+// system's get_state).  Everything is ordered by the handle's stream.
+double* stage_pos(bbmd_sim* sim) { return reinterpret_cast<double*>(sim->d.x2); }
+double* stage_vel(bbmd_sim* sim) { return reinterpret_cast<double*>(sim->d.v2); }
+
 bbmd_status bbmd_get_state(bbmd_sim* sim, double* pos, double* vel, int32_t* image) {
     if (!sim) return BBMD_ERR_ARG;
     DeviceGuard dg(sim->device);
-    finish_velocities(sim);
     const int64_t n = sim->d.n;
-    double* tp = pos ? (double*)dev_alloc(sim, 3 * n * 8) : nullptr;
-    double* tv = vel ? (double*)dev_alloc(sim, 3 * n * 8) : nullptr;
-    int32_t* ti = image ? (int32_t*)dev_alloc(sim, 3 * n * 4) : nullptr;
-    bbmd_status rc = BBMD_OK;
-    if ((pos && !tp) || (vel && !tv) || (image && !ti)) rc = fail(sim, BBMD_ERR_OOM, "get_state");
-    if (rc == BBMD_OK) {
-        launch_unpack_state(sim->d, sim->st, tp, tv, ti);
-        rc = cuda_check(sim, cudaGetLastError(), "unpack");
-    }
-    if (rc == BBMD_OK && pos)
-        rc = cuda_check(sim, cudaMemcpyAsync(pos, tp, 3 * n * 8, cudaMemcpyDeviceToHost, sim->st), "D2H");
-    if (rc == BBMD_OK && vel)
-        rc = cuda_check(sim, cudaMemcpyAsync(vel, tv, 3 * n * 8, cudaMemcpyDeviceToHost, sim->st), "D2H");
-    if (rc == BBMD_OK && image)
-        rc = cuda_check(sim, cudaMemcpyAsync(image, ti, 3 * n * 4, cudaMemcpyDeviceToHost, sim->st), "D2H");
-    if (rc == BBMD_OK) rc = cuda_check(sim, cudaStreamSynchronize(sim->st), "sync");
-    dev_free(sim, tp);
-    dev_free(sim, tv);
-    dev_free(sim, ti);
-    if (rc != BBMD_OK) return rc;
-    return read_status(sim);
+    double* tp = pos ? stage_pos(sim) : nullptr;
+    double* tv = vel ? stage_vel(sim) : nullptr;
+    int32_t* ti = image ? sim->d.img2 : nullptr;
+    launch_unpack_state(sim->d, sim->st, tp, tv, ti);
+    sim->pending = false;
+    LAUNCHED("unpack");
+    if (pos) CK(cudaMemcpyAsync(pos, tp, 3 * n * 8, cudaMemcpyDeviceToHost, sim->st));
+    if (vel) CK(cudaMemcpyAsync(vel, tv, 3 * n * 8, cudaMemcpyDeviceToHost, sim->st));
+    if (image) CK(cudaMemcpyAsync(image, ti, 3 * n * 4, cudaMemcpyDeviceToHost, sim->st));
+    int st = 0;
+    CK(cudaMemcpyAsync(&st, &sim->d.sc->status, sizeof(int), cudaMemcpyDeviceToHost, sim->st));
+    CK(cudaStreamSynchronize(sim->st));
+    return read_status(sim, st);
 }
 
 bbmd_status bbmd_set_state(bbmd_sim* sim, const double* pos, const double* vel,
@@ -1004,41 +984,25 @@ bbmd_status bbmd_set_state(bbmd_sim* sim, const double* pos, const double* vel,
     DeviceGuard dg(sim->device);
     finish_velocities(sim);
     const int64_t n = sim->d.n;
-    double* tp = (double*)dev_alloc(sim, 3 * n * 8);
-    double* tv = (double*)dev_alloc(sim, 3 * n * 8);
-    int32_t* ti = image ? (int32_t*)dev_alloc(sim, 3 * n * 4) : nullptr;
-    bbmd_status rc = BBMD_OK;
-    if (!tp || !tv || (image && !ti)) rc = fail(sim, BBMD_ERR_OOM, "set_state");
-    if (rc == BBMD_OK)
-        rc = cuda_check(sim, cudaMemcpyAsync(tp, pos, 3 * n * 8, cudaMemcpyHostToDevice, sim->st), "H2D");
-    if (rc == BBMD_OK)
-        rc = cuda_check(sim, cudaMemcpyAsync(tv, vel, 3 * n * 8, cudaMemcpyHostToDevice, sim->st), "H2D");
-    if (rc == BBMD_OK && image)
-        rc = cuda_check(sim, cudaMemcpyAsync(ti, image, 3 * n * 4, cudaMemcpyHostToDevice, sim->st), "H2D");
+    double* const tp = stage_pos(sim);
+    double* const tv = stage_vel(sim);
+    int32_t* const ti = image ? sim->d.img2 : nullptr;
+    CK(cudaMemcpyAsync(tp, pos, 3 * n * 8, cudaMemcpyHostToDevice, sim->st));
+    CK(cudaMemcpyAsync(tv, vel, 3 * n * 8, cudaMemcpyHostToDevice, sim->st));
+    if (image) CK(cudaMemcpyAsync(ti, image, 3 * n * 4, cudaMemcpyHostToDevice, sim->st));
     // the uploaded values are checked on the device (one pass over them at HBM speed, not
     // a serial host scan) before anything of the state is replaced
-    if (rc == BBMD_OK) {
-        int bad = 0;
-        rc = cuda_check(sim, cudaMemsetAsync(&sim->d.sc->bad_input, 0, sizeof(int), sim->st), "memset");
-        if (rc == BBMD_OK) {
-            launch_check_finite(sim->d, sim->st, tp, 3 * n);
-            launch_check_finite(sim->d, sim->st, tv, 3 * n);
-            rc = cuda_check(sim, cudaMemcpyAsync(&bad, &sim->d.sc->bad_input, sizeof(int),
-                                                 cudaMemcpyDeviceToHost, sim->st), "D2H");
-        }
-        if (rc == BBMD_OK) rc = cuda_check(sim, cudaStreamSynchronize(sim->st), "sync");
-        if (rc == BBMD_OK && bad) rc = fail(sim, BBMD_ERR_ARG, "non-finite positions or velocities");
-    }
-    if (rc == BBMD_OK) {
-        launch_pack_state(sim->d, sim->st, tp, tv, ti, true);
-        rc = cuda_check(sim, cudaGetLastError(), "pack");
-    }
-    if (rc == BBMD_OK) rc = rebuild_now(sim);
+    int bad = 0;
+    CK(cudaMemsetAsync(&sim->d.sc->bad_input, 0, sizeof(int), sim->st));
+    launch_check_finite(sim->d, sim->st, tp, 3 * n);
+    launch_check_finite(sim->d, sim->st, tv, 3 * n);
+    CK(cudaMemcpyAsync(&bad, &sim->d.sc->bad_input, sizeof(int), cudaMemcpyDeviceToHost, sim->st));
+    CK(cudaStreamSynchronize(sim->st));
+    if (bad) return fail(sim, BBMD_ERR_ARG, "non-finite positions or velocities");
+    launch_pack_state(sim->d, sim->st, tp, tv, ti, true);
+    LAUNCHED("pack");
+    bbmd_status rc = rebuild_now(sim);
     if (rc == BBMD_OK) rc = refresh_forces_and_K(sim);
-    if (rc == BBMD_OK) rc = cuda_check(sim, cudaStreamSynchronize(sim->st), "sync");
-    dev_free(sim, tp);
-    dev_free(sim, tv);
-    dev_free(sim, ti);
     if (rc != BBMD_OK) return rc;
     return read_status(sim);
 }
@@ -1083,22 +1047,12 @@ bbmd_status bbmd_get_forces(bbmd_sim* sim, double* F, double* u) {
     DeviceGuard dg(sim->device);
     const int64_t n = sim->d.n;
     launch_force(sim->d, sim->st, u != nullptr, false);
-    double* tf = (double*)dev_alloc(sim, 3 * n * 8);
-    double* tu = u ? (double*)dev_alloc(sim, n * 8) : nullptr;
-    bbmd_status rc = BBMD_OK;
-    if (!tf || (u && !tu)) rc = fail(sim, BBMD_ERR_OOM, "get_forces");
-    if (rc == BBMD_OK) {
-        launch_unpack_forces(sim->d, sim->st, tf, tu);
-        rc = cuda_check(sim, cudaGetLastError(), "unpack forces");
-    }
-    if (rc == BBMD_OK)
-        rc = cuda_check(sim, cudaMemcpyAsync(F, tf, 3 * n * 8, cudaMemcpyDeviceToHost, sim->st), "D2H");
-    if (rc == BBMD_OK && u)
-        rc = cuda_check(sim, cudaMemcpyAsync(u, tu, n * 8, cudaMemcpyDeviceToHost, sim->st), "D2H");
-    if (rc == BBMD_OK) rc = cuda_check(sim, cudaStreamSynchronize(sim->st), "sync");
-    dev_free(sim, tf);
-    dev_free(sim, tu);
-    if (rc != BBMD_OK) return rc;
+    double* const tf = stage_pos(sim);
+    double* const tu = u ? stage_vel(sim) : nullptr;
+    launch_unpack_forces(sim->d, sim->st, tf, tu);
+    LAUNCHED("unpack forces");
+    CK(cudaMemcpyAsync(F, tf, 3 * n * 8, cudaMemcpyDeviceToHost, sim->st));
+    if (u) CK(cudaMemcpyAsync(u, tu, n * 8, cudaMemcpyDeviceToHost, sim->st));
     return read_status(sim);
 }
 
@@ -1106,15 +1060,12 @@ bbmd_status bbmd_get_cells(bbmd_sim* sim, int64_t* cell) {
     if (!sim || !cell) return BBMD_ERR_ARG;
     DeviceGuard dg(sim->device);
     const int64_t n = sim->d.n;
-    int64_t* tc = (int64_t*)dev_alloc(sim, n * 8);
-    if (!tc) return fail(sim, BBMD_ERR_OOM, "get_cells");
+    int64_t* const tc = reinterpret_cast<int64_t*>(sim->d.x2);  // (see stage_pos)
     launch_unpack_cells(sim->d, sim->st, tc);
-    bbmd_status rc = cuda_check(sim, cudaGetLastError(), "unpack cells");
-    if (rc == BBMD_OK)
-        rc = cuda_check(sim, cudaMemcpyAsync(cell, tc, n * 8, cudaMemcpyDeviceToHost, sim->st), "D2H");
-    if (rc == BBMD_OK) rc = cuda_check(sim, cudaStreamSynchronize(sim->st), "sync");
-    dev_free(sim, tc);
-    return rc;
+    LAUNCHED("unpack cells");
+    CK(cudaMemcpyAsync(cell, tc, n * 8, cudaMemcpyDeviceToHost, sim->st));
+    CK(cudaStreamSynchronize(sim->st));
+    return BBMD_OK;
 }
 
 bbmd_status bbmd_get_neighbors(bbmd_sim* sim, const int64_t* ids, int64_t m, int64_t* offsets,

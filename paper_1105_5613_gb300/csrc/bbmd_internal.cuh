@@ -36,6 +36,8 @@ __host__ __device__ constexpr int region_cells_of(int bz) {
     return (block_xy_of(bz) + 2) * (block_xy_of(bz) + 2) * (block_zc_of(bz) + 2);
 }
 constexpr int kMaxPartials = 8192;     // per-block FP64 partial sums
+constexpr int kEnergyPartial = 4;      // slot of the energy partials (the virial's follows)
+constexpr int kOutScalars = 32;        // results of an observation: doubles before its DevScalars
 constexpr float kBand = 1e-5f;         // relative band around a threshold for the FP64 re-test
 
 // status bits (sticky, OR-ed on the device)
@@ -385,10 +387,17 @@ void launch_integrate(const DevSim& s, cudaStream_t st);
 void launch_finalize(const DevSim& s, cudaStream_t st, bool ke);
 // apply the closing half kick and NH scale a call left pending (no-op when none is)
 void launch_finish(const DevSim& s, cudaStream_t st);
-void launch_state_sums(const DevSim& s, cudaStream_t st);          // KE, P partials -> sc->K etc.
-void launch_reduce_partials(const DevSim& s, cudaStream_t st, int nq, double* out_dev);
+// kinetic energy and momentum partials 0..3 of the finished velocities
+void launch_state_sums(const DevSim& s, cudaStream_t st);
+// sc->K from those partials
+void launch_set_K(const DevSim& s, cudaStream_t st);
+// out[0..3] from them, with energy out[9..10] from the energy partials; the handle's DevScalars
+// after out[kOutScalars]
+void launch_observe_sums(const DevSim& s, cudaStream_t st, bool energy, double* out_dev);
 void launch_init_fcc(const DevSim& s, cudaStream_t st, int m, double jitter, uint64_t seed);
-void launch_init_mb(const DevSim& s, cudaStream_t st, double T0, uint64_t seed, double* tmp3);
+// tmp3: 3 n doubles, sums: 8 doubles of scratch
+void launch_init_mb(const DevSim& s, cudaStream_t st, double T0, uint64_t seed, double* tmp3,
+                    double* sums);
 void launch_sd_step(const DevSim& s, cudaStream_t st, double hmax, double dmax);
 void launch_clear_rebuild(const DevSim& s, cudaStream_t st);
 void launch_clear_grid_sync(const DevSim& s, cudaStream_t st);
@@ -399,8 +408,10 @@ void launch_msd_fs(const DevSim& s, cudaStream_t st, const double* ref, double k
 int launch_gr(const DevSim& s, cudaStream_t st, int nbins, double rmax,
               unsigned long long* counts_dev, int32_t* scratch_i32, float4* scratch_f4,
               int64_t scratch_n);
+// the state in id order into device buffers (each may be NULL), after applying a pending
+// closing update to the stored velocities
 void launch_unpack_state(const DevSim& s, cudaStream_t st, double* pos, double* vel,
-                         int32_t* img);   // device buffers, id order
+                         int32_t* img);
 void launch_pack_state(const DevSim& s, cudaStream_t st, const double* pos, const double* vel,
                        const int32_t* img, bool species_from_current);
 void launch_unpack_forces(const DevSim& s, cudaStream_t st, double* F, double* u);

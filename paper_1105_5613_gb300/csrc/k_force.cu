@@ -1702,7 +1702,8 @@ __device__ __forceinline__ void pair_fp64(const DevSim& s, int si, long long mx,
 }
 
 // WHAT: see above (k64Force writes F and Fd; k64Energy the per-particle energies u_i, half
-// of each pair energy; with k64Energy or k64Sums the energy and virial partials 1 and 2).
+// of each pair energy; k64Energy and k64Sums the energy and virial partials, from
+// kEnergyPartial).
 template <int MODE, int WHAT, bool KE, bool FSHIFT>
 __device__ __forceinline__ void force64_body(const DevSim& s, int lb, int lg) {
     if (!force_selected<MODE>(s)) return;  // CTA-uniform, before any barrier
@@ -1870,9 +1871,9 @@ __device__ __forceinline__ void force64_body(const DevSim& s, int lb, int lg) {
     if (KE || (WHAT & (k64Energy | k64Sums))) {
         const double sums[3] = {warp_sum_d(acc_ke), warp_sum_d(acc_u), warp_sum_d(acc_w)};
         if (KE)
-            block_partials(s, lb, sums, 0, WHAT & (k64Energy | k64Sums) ? 3 : 1);
+            block_partials(s, lb, sums, 0, 1);
         else
-            block_partials(s, lb, sums + 1, 1, 2);
+            block_partials(s, lb, sums + 1, kEnergyPartial, 2);
     }
 }
 
@@ -2057,7 +2058,7 @@ void launch_force(const DevSim& s, cudaStream_t st, bool energy, bool ke) {
     run_force_mode<1>(s, st, energy, ke, fs);
 }
 
-// Energy and virial sums of the current positions (partials 1 and 2) alone, both precisions.
+// Energy and virial partials of the current positions alone, both precisions.
 void launch_energy_sums(const DevSim& s, cudaStream_t st) {
     const bool fs = s.pt.shift == BBMD_SHIFT_FORCE;
     if (s.nbr_mode == BBMD_NBR_VERLET) run_energy_sums<0>(s, st, fs);

@@ -178,14 +178,27 @@ __global__ void __launch_bounds__(kThreads) k_state_sums(DevSim s) {
     if (threadIdx.x < 4) s.partials[threadIdx.x * kMaxPartials + blockIdx.x] = red[threadIdx.x][0];
 }
 
-__global__ void __launch_bounds__(256) k_reduce_partials(DevSim s, int nb, int nq, double* out,
-                                                        int set_K) {
+__global__ void __launch_bounds__(256) k_reduce_partials(DevSim s, int nb, int nq, double* out) {
     __shared__ double r[8];
     sum_partials(s, nb, nq, r);
-    if (threadIdx.x == 0) {
-        for (int q = 0; q < nq; ++q) out[q] = r[q];
-        if (set_K) s.sc->K = r[0];
-    }
+    if ((int)threadIdx.x < nq) out[threadIdx.x] = r[threadIdx.x];
+}
+
+__global__ void __launch_bounds__(256) k_set_K(DevSim s, int nb) {
+    __shared__ double r[1];
+    sum_partials(s, nb, 1, r);
+    if (threadIdx.x == 0) s.sc->K = r[0];
+}
+
+__global__ void __launch_bounds__(256) k_observe_sums(DevSim s, int energy, double* out) {
+    static_assert(sizeof(DevScalars) % 8 == 0 && sizeof(DevScalars) <= (64 - kOutScalars) * 8, "dout");
+    __shared__ double r[6];
+    sum_partials(s, s.grid_part, 4, r);
+    if (energy) sum_partials(s, s.grid_cell, 2, r + 4, kEnergyPartial);
+    if (threadIdx.x < 4) out[threadIdx.x] = r[threadIdx.x];
+    if (energy && threadIdx.x < 2) out[9 + threadIdx.x] = r[4 + threadIdx.x];
+    if (threadIdx.x < sizeof(DevScalars) / 8)
+        out[kOutScalars + threadIdx.x] = reinterpret_cast<const double*>(s.sc)[threadIdx.x];
 }
 
 // ------------------------------------------------------------------ initialisers ----
@@ -349,15 +362,20 @@ __global__ void k_clear_rebuild(DevSim s) {
 
 // --------------------------------------------------------------- state transfer ----
 
+template <bool FP64>
 __global__ void __launch_bounds__(kThreads) k_unpack_state(DevSim s, double* pos, double* vel,
                                                           int32_t* img) {
+    const bool pending = s.sc->pending != 0;
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < s.n;
          k += (int64_t)gridDim.x * blockDim.x) {
         int64_t id = s.id[k];
+        long long vo[3];
+        if (vel || pending) finished_velocity<FP64>(s, k, vo);
         for (int d = 0; d < 3; ++d) {
             int64_t idx = d * s.npad + k;
+            if (pending) s.v[idx] = vo[d];
             if (pos) pos[3 * id + d] = ldexp(__ll2double_rn((long long)s.x[idx]), -s.kexp);
-            if (vel) vel[3 * id + d] = __ll2double_rn(s.v[idx]) * 0x1p-52;
+            if (vel) vel[3 * id + d] = __ll2double_rn(vo[d]) * 0x1p-52;
             if (img) img[3 * id + d] = s.img[idx];
         }
     }
@@ -631,12 +649,10 @@ void launch_state_sums(const DevSim& s, cudaStream_t st) {
         k_state_sums<false><<<s.grid_part, kThreads, 0, st>>>(s);
 }
 
-void launch_reduce_partials(const DevSim& s, cudaStream_t st, int nq, double* out_dev) {
-    // nq > 0: partials written by a per-particle kernel (grid_part blocks);
-    // nq < 0: by a per-cell kernel (grid_cell blocks), |nq| quantities.
-    int nb = nq > 0 ? s.grid_part : s.grid_cell;
-    int q = nq > 0 ? nq : -nq;
-    k_reduce_partials<<<1, 256, 0, st>>>(s, nb, q, out_dev, 0);
+void launch_set_K(const DevSim& s, cudaStream_t st) { k_set_K<<<1, 256, 0, st>>>(s, s.grid_part); }
+
+void launch_observe_sums(const DevSim& s, cudaStream_t st, bool energy, double* out_dev) {
+    k_observe_sums<<<1, 256, 0, st>>>(s, energy ? 1 : 0, out_dev);
 }
 
 void launch_init_fcc(const DevSim& s, cudaStream_t st, int m, double jitter, uint64_t seed) {
@@ -646,13 +662,12 @@ void launch_init_fcc(const DevSim& s, cudaStream_t st, int m, double jitter, uin
                                                  (unsigned long long)seed);
 }
 
-void launch_init_mb(const DevSim& s, cudaStream_t st, double T0, uint64_t seed, double* tmp3) {
-    // tmp3: 3n doubles of scratch followed by 8 doubles for the sums
-    double* sums = tmp3 + 3 * s.n;
+void launch_init_mb(const DevSim& s, cudaStream_t st, double T0, uint64_t seed, double* tmp3,
+                    double* sums) {
     k_mb_draw<<<s.grid_part, kThreads, 0, st>>>(s, T0, seed, tmp3);
-    k_reduce_partials<<<1, 256, 0, st>>>(s, s.grid_part, 4, sums, 0);
+    k_reduce_partials<<<1, 256, 0, st>>>(s, s.grid_part, 4, sums);
     k_mb_shift<<<s.grid_part, kThreads, 0, st>>>(s, tmp3, sums);
-    k_reduce_partials<<<1, 256, 0, st>>>(s, s.grid_part, 1, sums + 4, 0);
+    k_reduce_partials<<<1, 256, 0, st>>>(s, s.grid_part, 1, sums + 4);
     k_mb_scale<<<s.grid_part, kThreads, 0, st>>>(s, tmp3, sums + 4, T0);
 }
 
@@ -680,12 +695,16 @@ void launch_msd_fs(const DevSim& s, cudaStream_t st, const double* ref, double k
     k_msd_fs<<<s.grid_part, kThreads, 0, st>>>(s, ref, kvec, ldexp((double)s.Lfix[0], -s.kexp),
                                                ldexp((double)s.Lfix[1], -s.kexp),
                                                ldexp((double)s.Lfix[2], -s.kexp));
-    k_reduce_partials<<<1, 256, 0, st>>>(s, s.grid_part, 6, out_dev, 0);
+    k_reduce_partials<<<1, 256, 0, st>>>(s, s.grid_part, 6, out_dev);
 }
 
 void launch_unpack_state(const DevSim& s, cudaStream_t st, double* pos, double* vel,
                          int32_t* img) {
-    k_unpack_state<<<s.grid_part, kThreads, 0, st>>>(s, pos, vel, img);
+    if (s.precision == BBMD_PREC_FP64)
+        k_unpack_state<true><<<s.grid_part, kThreads, 0, st>>>(s, pos, vel, img);
+    else
+        k_unpack_state<false><<<s.grid_part, kThreads, 0, st>>>(s, pos, vel, img);
+    k_finish_done<<<1, 1, 0, st>>>(s);
 }
 
 void launch_pack_state(const DevSim& s, cudaStream_t st, const double* pos, const double* vel,

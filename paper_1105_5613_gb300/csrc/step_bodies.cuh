@@ -224,16 +224,16 @@ __device__ __forceinline__ void check_body(const DevSim& s, int lb, int lg) {
     if (need) sc->rebuild = 1;
 }
 
-// Sum partials[q][0 .. nb) for q < nq (at most 8) in a fixed order: a strided sum per
+// Sum partials[q0 + q][0 .. nb) for q < nq (at most 8) in a fixed order: a strided sum per
 // thread of kStepThreads, a butterfly over each warp's lanes, then the warps in order (one
 // CTA; a smaller one takes the warps in turn, so the sum does not depend on its size).
-__device__ void sum_partials(const DevSim& s, int nb, int nq, double* out) {
+__device__ void sum_partials(const DevSim& s, int nb, int nq, double* out, int q0 = 0) {
     __shared__ double red[8][kStepThreads / 32];
     const int lane = threadIdx.x & 31;
     for (int w = threadIdx.x >> 5; w < kStepThreads / 32; w += blockDim.x >> 5)
         for (int q = 0; q < nq; ++q) {
             double t = 0.0;
-            for (int b = w * 32 + lane; b < nb; b += kStepThreads) t += s.partials[q * kMaxPartials + b];
+            for (int b = w * 32 + lane; b < nb; b += kStepThreads) t += s.partials[(q0 + q) * kMaxPartials + b];
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(kStepFull, t, o);
             if (lane == 0) red[q][w] = t;
