@@ -24,6 +24,8 @@
 // This file is compiled once per block shape, code BBMD_BLOCK_Z = 1, 2 or 4 (2 x 2 x Z
 // cells) or 8 (4 x 4 x 2 cells), into namespace bbmd::z<BBMD_BLOCK_Z>; the handle picks one
 // shape at creation.
+#include <cstddef>
+
 #include "bbmd_internal.cuh"
 
 #ifndef BBMD_BLOCK_Z
@@ -103,10 +105,11 @@ struct Region {
     int off[kRegion + 1];      // prefix of staged counts (clamped to smax); off[kRegion] = total
     int start[kRegion];        // first particle of each region cell
     int cnt[kRegion];          // particles of each region cell
-    float hi[kRegion][3];      // frame offset of each cell (FP32 rounding of the exact value)
+    int nstaged;
+    // used while a block is staged (and by the FP64 staging); free for the block's own work
+    alignas(16) float hi[kRegion][3];  // frame offset of each cell (FP32 rounding of the exact value)
     float lo[kRegion][3];      // exact residual of that rounding (non-zero across the seam)
     long long fr[kRegion][3];  // FP64 form: frame point + seam image of each cell
-    int nstaged;
 };
 
 // ------------------------------------------------ TMA bulk copies and mbarriers ----
@@ -702,11 +705,24 @@ __device__ __forceinline__ float keep_reach(const float* hi4, int sj) {
 // exactly those whose FP32 value could be on the wrong side.
 constexpr int kSRing = 64;  // entries per stream ring (two 32-entry words; a power of two)
 
+// One array per component, so that four (two pairs of) candidates come with one 16-byte
+// broadcast read per component, and a lane that picks one entry of a word reads one of 32
+// consecutive words per component (no bank conflicts among the lanes).
 struct StreamRings {
-    float4 rec[2][kSRing];     // (p' - c, q)
+    float x[2][kSRing], y[2][kSRing], z[2][kSRing], q[2][kSRing];  // p' = p - c, |p'|^2
     uint16_t idx[2][kSRing];   // staged index
     float4 box[2];             // (c, reach^2 of species A), (half-extents, reach^2 of B)
 };
+
+// The word of 32 entries of stream S that starts at cq (a multiple of 32).
+struct StreamWord {
+    const float *x, *y, *z, *q;
+};
+
+__device__ __forceinline__ StreamWord stream_word(const StreamRings& SR, int S, int cq) {
+    const int o = cq & (kSRing - 1);
+    return {SR.x[S] + o, SR.y[S] + o, SR.z[S] + o, SR.q[S] + o};
+}
 
 __device__ __forceinline__ StreamRings& warp_streams(int w) {
     __shared__ __align__(16) StreamRings rings_all[kBW];
@@ -739,25 +755,30 @@ __device__ __forceinline__ void compact_streams(const float4* sm, int g0, int re
     const int t = g0 + lane;
     bool keep = false;
     int sj = 0;
-    float4 rec = make_float4(0.f, 0.f, 0.f, 0.f);
+    float x = 0.f, y = 0.f, z = 0.f;
     if (t < re) {
         const float4 p = sm[t];
         const float4 c = SR.box[0], h = SR.box[1];
-        const float x = p.x - c.x, y = p.y - c.y, z = p.z - c.z;
+        x = p.x - c.x;
+        y = p.y - c.y;
+        z = p.z - c.z;
         const float ex = fmaxf(fabsf(x) - h.x, 0.f);
         const float ey = fmaxf(fabsf(y) - h.y, 0.f);
         const float ez = fmaxf(fabsf(z) - h.z, 0.f);
         sj = p.w != 0.f ? 1 : 0;
         keep = fmaf(ez, ez, fmaf(ey, ey, ex * ex)) < (sj ? h.w : c.w);
-        rec = make_float4(x, y, z, fmaf(z, z, fmaf(y, y, x * x)));
     }
     const unsigned bA = __ballot_sync(FULL, keep && sj == 0);
     const unsigned bB = __ballot_sync(FULL, keep && sj == 1);
     const unsigned lt = (1u << lane) - 1u;
     const int pos = sj ? fill[1] + __popc(bB & lt) : fill[0] + __popc(bA & lt);
     if (keep) {
-        SR.rec[sj][pos & (kSRing - 1)] = rec;
-        SR.idx[sj][pos & (kSRing - 1)] = (uint16_t)t;
+        const int o = pos & (kSRing - 1);
+        SR.x[sj][o] = x;
+        SR.y[sj][o] = y;
+        SR.z[sj][o] = z;
+        SR.q[sj][o] = fmaf(z, z, fmaf(y, y, x * x));
+        SR.idx[sj][o] = (uint16_t)t;
     }
     const int src = self - g0;
     const int sp = __shfl_sync(FULL, pos, src & 31);
@@ -773,14 +794,45 @@ __device__ __forceinline__ void compact_streams(const float4* sm, int g0, int re
 __device__ __forceinline__ void stream_pad(StreamRings& SR, int S, int fill, int lane, int sentinel) {
     const int pe = (fill + 31) & ~31;
     if (fill + lane < pe) {
-        SR.rec[S][(fill + lane) & (kSRing - 1)] = make_float4(kFar, kFar, kFar, 3.0f * kFar * kFar);
-        SR.idx[S][(fill + lane) & (kSRing - 1)] = (uint16_t)sentinel;
+        const int o = (fill + lane) & (kSRing - 1);
+        SR.x[S][o] = SR.y[S][o] = SR.z[S][o] = kFar;
+        SR.q[S][o] = 3.0f * kFar * kFar;
+        SR.idx[S][o] = (uint16_t)sentinel;
     }
 }
 
-// r^2 - R^2 of a stream entry for a lane: m2 = -2 m', cst = |m'|^2 - R^2(s_i, S).
-__device__ __forceinline__ float stream_d(const float4 r, float m2x, float m2y, float m2z, float cst) {
-    return fmaf(r.z, m2z, fmaf(r.y, m2y, fmaf(r.x, m2x, r.w + cst)));
+// r^2 - R^2 of entry u of a stream word for a lane: m2 = -2 m', cst = |m'|^2 - R^2(s_i, S).
+__device__ __forceinline__ float stream_d(const StreamWord& W, int u, float m2x, float m2y, float m2z,
+                                          float cst) {
+    return fmaf(W.z[u], m2z, fmaf(W.y[u], m2y, fmaf(W.x[u], m2x, W.q[u] + cst)));
+}
+
+// The signs of stream_d over a word (entry u in bit 31 - u: set where negative) and the
+// smallest |stream_d|.  Two-wide FP32 (each half rounds like the scalar operation), four
+// entries per 16-byte read of a component: 5.5 instructions an entry against 7.
+__device__ __forceinline__ unsigned word_signs(const StreamWord& W, float m2x, float m2y, float m2z,
+                                               float cst, float& near) {
+    const float2 mx = make_float2(m2x, m2x), my = make_float2(m2y, m2y), mz = make_float2(m2z, m2z),
+                 cc = make_float2(cst, cst);
+    unsigned in = 0u;
+#pragma unroll
+    for (int u = 0; u < 32; u += 4) {
+        const float4 x = *reinterpret_cast<const float4*>(W.x + u);
+        const float4 y = *reinterpret_cast<const float4*>(W.y + u);
+        const float4 z = *reinterpret_cast<const float4*>(W.z + u);
+        const float4 q = *reinterpret_cast<const float4*>(W.q + u);
+        const float2 d0 = __ffma2_rn(make_float2(z.x, z.y), mz, __ffma2_rn(make_float2(y.x, y.y), my,
+                          __ffma2_rn(make_float2(x.x, x.y), mx, __fadd2_rn(make_float2(q.x, q.y), cc))));
+        const float2 d1 = __ffma2_rn(make_float2(z.z, z.w), mz, __ffma2_rn(make_float2(y.z, y.w), my,
+                          __ffma2_rn(make_float2(x.z, x.w), mx, __fadd2_rn(make_float2(q.z, q.w), cc))));
+        in = __funnelshift_l(__float_as_uint(d0.x), in, 1);
+        in = __funnelshift_l(__float_as_uint(d0.y), in, 1);
+        in = __funnelshift_l(__float_as_uint(d1.x), in, 1);
+        in = __funnelshift_l(__float_as_uint(d1.y), in, 1);
+        near = fminf(near, fminf(fabsf(d0.x), fabsf(d0.y)));
+        near = fminf(near, fminf(fabsf(d1.x), fabsf(d1.y)));
+    }
+    return in;
 }
 
 // Which force kernel runs: in cell mode the stencil kernel (MODE 1); in Verlet mode the
@@ -949,16 +1001,10 @@ __device__ __forceinline__ void force_body(const DevSim& s, int lb, int lg) {
                     int fill[2] = {0, 0}, done[2] = {0, 0}, cself = -1;
                     // bitmask of the entries of stream S's word at cq inside the cutoff
                     auto filter_word = [&](int S, int cq) -> unsigned {
-                        const float4* const rp = SR.rec[S] + (cq & (kSRing - 1));
+                        const StreamWord W = stream_word(SR, S, cq);
                         const float cS = mm - s.pt.rc2lo[si * 2 + S];
-                        unsigned inw = 0u;
                         float near = far;
-#pragma unroll
-                        for (int u = 0; u < 32; ++u) {
-                            const float d = stream_d(rp[u], m2x, m2y, m2z, cS);
-                            inw = __funnelshift_l(__float_as_uint(d), inw, 1);
-                            near = fminf(near, fabsf(d));
-                        }
+                        unsigned inw = word_signs(W, m2x, m2y, m2z, cS, near);
                         const int nv = fill[S] - cq;
                         unsigned valid = nv >= 32 ? 0xffffffffu : ~(0xffffffffu >> nv);
                         if (S == si && cself >= cq && cself < cq + 32)
@@ -972,12 +1018,11 @@ __device__ __forceinline__ void force_body(const DevSim& s, int lb, int lg) {
                             while (bw) {
                                 const int u = __clz(bw);
                                 bw &= 0x7fffffffu >> u;
-                                if (!(fabsf(stream_d(rp[u], m2x, m2y, m2z, cS)) < bS)) continue;
+                                if (!(fabsf(stream_d(W, u, m2x, m2y, m2z, cS)) < bS)) continue;
                                 const unsigned bit = 0x80000000u >> u;
                                 inw &= ~bit;
-                                const float4 r = rp[u];
-                                if (!min_image_copy(s, fmaf(m2x, 0.5f, r.x), fmaf(m2y, 0.5f, r.y),
-                                                    fmaf(m2z, 0.5f, r.z)))
+                                if (!min_image_copy(s, fmaf(m2x, 0.5f, W.x[u]), fmaf(m2y, 0.5f, W.y[u]),
+                                                    fmaf(m2z, 0.5f, W.z[u])))
                                     continue;
                                 const int t = (int)SR.idx[S][(cq + u) & (kSRing - 1)];
                                 const int64_t gj = staged_global(Rc, t);
@@ -989,7 +1034,7 @@ __device__ __forceinline__ void force_body(const DevSim& s, int lb, int lg) {
                     // the forces of the set bits of stream S's word at cq
                     auto force_word = [&](int S, int cq) {
                         unsigned inw = filter_word(S, cq);
-                        const float4* const rp = SR.rec[S] + (cq & (kSRing - 1));
+                        const StreamWord W = stream_word(SR, S, cq);
                         // the constants of the species pair (s_i, S)
                         const int k = si * 2 + S;
                         const float sig2 = s.pt.sig2[k], e48 = s.pt.eps48[k];
@@ -998,10 +1043,9 @@ __device__ __forceinline__ void force_body(const DevSim& s, int lb, int lg) {
                         while (inw) {
                             const int u = __clz(inw);
                             inw &= 0x7fffffffu >> u;
-                            const float4 r = rp[u];
                             // p' - m' (0.5 m2 = -m' exactly)
-                            const float dx = fmaf(m2x, 0.5f, r.x), dy = fmaf(m2y, 0.5f, r.y),
-                                        dz = fmaf(m2z, 0.5f, r.z);
+                            const float dx = fmaf(m2x, 0.5f, W.x[u]), dy = fmaf(m2y, 0.5f, W.y[u]),
+                                        dz = fmaf(m2z, 0.5f, W.z[u]);
                             const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
                             pair_add_c<FSHIFT>(sig2, e48, cpot, fcut, dx, dy, dz, r2, a);
                         }
@@ -1075,10 +1119,46 @@ __device__ __forceinline__ void force_body(const DevSim& s, int lb, int lg) {
 // broadcast shared-memory reads: the sign of r^2 - R2lo(species of j) is shifted into a
 // 32-bit word (candidate u lands in bit 31 - u) and the smallest |r^2 - R2lo| of the word
 // is kept.  Only a word whose minimum falls inside the band goes through the exact rule,
-// candidate by candidate.  The set bits of each word are then written as list offsets,
-// two entries per 32-bit store into [kb][npad][8] uint16, at a row pointer advanced once
-// per four pairs.
+// candidate by candidate.  The set bits of each word are then appended to the lane's list.
+//
+// The append takes 45 % of the build as a loop over each lane's own bits (two entries and one
+// 4-byte store an iteration, 22 of 32 lanes active, 340 instructions a word).  With BUFFER
+// every lane looks at every candidate of the word (one predicated store into its own buffer
+// of 16 entries in shared memory, no divergent loop), and rows of 8 leave as they fill with
+// one 16-byte store.  Microseconds a build at 2.05 M particles, loop -> buffer (before either,
+// with one FP32 operation per entry and scalar reads of the streams): 4 x 4 x 2 at skin 0.4
+// (1427) 1370 -> 1282; at skin 0.3 2 x 2 x 2 (1140) 1077 -> 1030, 2 x 2 x 1 (1230) 1174 -> 1108.
+// 2 x 2 x 4 keeps the loop (1095 -> 1049): the buffers would leave room for two CTAs per SM
+// instead of three (1140).  Looks after every 4 candidates (smaller buffers) or only when some
+// buffer is full (larger ones) measured slower.
 
+// Append the low half of e if bits & mask and the high half if bits & (mask >> 1) at the
+// shared-memory address top: predicated stores, whatever the lanes' bits.
+__device__ __forceinline__ void push_entries(unsigned& top, unsigned e, unsigned bits, unsigned mask) {
+    asm volatile(
+        "{\n .reg .pred p;\n .reg .b32 t;\n .reg .b16 lo, hi;\n"
+        " mov.b32 {lo, hi}, %1;\n"
+        " and.b32 t, %2, %3;\n setp.ne.u32 p, t, 0;\n"
+        " @p st.shared.u16 [%0], lo;\n @p add.u32 %0, %0, 2;\n"
+        " and.b32 t, %2, %4;\n setp.ne.u32 p, t, 0;\n"
+        " @p st.shared.u16 [%0], hi;\n @p add.u32 %0, %0, 2;\n}"
+        : "+r"(top)
+        : "r"(e), "r"(bits), "r"(mask), "r"(mask >> 1)
+        : "memory");
+}
+
+// The lane's entry buffer: 16 entries, 16-byte aligned.  One KB per warp, in the part of the
+// region's description that is free once the block is staged (as many warps as fit), and
+// beside it for the others.
+__device__ __forceinline__ uint16_t* entry_buffer(StageShared& ss, int w, int lane) {
+    constexpr int kFree = (int)(sizeof(Region) - offsetof(Region, hi)) / 1024;  // warps
+    constexpr int kMore = kBW > kFree ? kBW - kFree : 1;
+    __shared__ __align__(16) uint16_t more[kMore][32][16];
+    if (w < kFree) return reinterpret_cast<uint16_t*>(&ss.R[0].hi[0][0]) + (w * 32 + lane) * 16;
+    return more[w - kFree][lane];
+}
+
+template <bool BUFFER>
 __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg) {
     if (!s.sc->rebuild) return;
     extern __shared__ float4 smem[];
@@ -1089,6 +1169,8 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
     const int lcap = s.lcap8 * 8;
     const int lcap2 = lcap >> 1;  // pair slots per particle
     StreamRings& SR = warp_streams(w);
+    uint16_t* buf = nullptr;
+    if constexpr (BUFFER) buf = entry_buffer(ss, w, lane);
     if (threadIdx.x == 0) {
         for (int k = 0; k < kStageBuffers; ++k) mbar_init(&mbar[k], 1);
         ss.next_cell[0] = ss.next_cell[1] = 0;
@@ -1096,9 +1178,6 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
     __syncthreads();
     int blk_it = 0;  // blocks of this CTA so far (the parity selects the cell counter)
     const float far = kFar;
-    const unsigned sentpair = (unsigned)s.smax | ((unsigned)s.smax << 16);
-    uint32_t* list32 = reinterpret_cast<uint32_t*>(s.list);
-    const int64_t rowstep = (int64_t)s.npad * 4;  // uint32 distance between kb rows
     for_each_block(s, lb, lg, smem, s.smax + 1, R, mbar, [&](const BlockPos& bp, const Region& Rc,
                                                            const float4* sm) {
         const int par = blk_it & 1;
@@ -1116,18 +1195,17 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
                 const int self = self0 + li;
                 float4 me = act ? sm[self] : make_float4(-far, -far, -far, 0.f);
                 const int si = me.w != 0.f ? 1 : 0;
-                int len = 0;
-                unsigned pend = 0u;
-                // pair slot wi (entries 2 wi, 2 wi + 1) of this particle:
-                // row0[(wi >> 2) * rowstep + (wi & 3)]
-                uint32_t* const row0 = list32 + gi * 4;
-                // next pair slot wp and the start of its row
-                int wp = 0;
-                uint32_t* rowp = row0;
+                // the row being filled (entries beyond the capacity are counted, not stored); with
+                // BUFFER its number and the shared-memory address of the lane's next entry, else
+                // the next pair slot, the entries so far and a pending odd one
+                uint4* rowp = reinterpret_cast<uint4*>(s.list) + gi;
+                const unsigned top0 = BUFFER ? smem_u32(buf) : 0u;
+                unsigned top = top0, pend = 0u;
+                int row = 0, wp = 0, len = 0;
                 auto put_pair = [&](unsigned v) {
-                    if (wp < lcap2) rowp[wp & 3] = v;
+                    if (wp < lcap2) reinterpret_cast<uint32_t*>(rowp)[wp & 3] = v;
                     ++wp;
-                    if ((wp & 3) == 0) rowp += rowstep;
+                    if ((wp & 3) == 0) rowp += s.npad;
                 };
                 const float4 fc = warp_frame(warp_box(me, act), keep_reach(s.pt.R2hi, 0),
                                              keep_reach(s.pt.R2hi, 1), SR, lane);
@@ -1140,16 +1218,10 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
                 // bitmask of the entries of stream S's word at cq (a multiple of 32) that
                 // enter this particle's list (entry u in bit 31 - u)
                 auto test_word = [&](int S, int cq) -> unsigned {
-                    const float4* const rp = SR.rec[S] + (cq & (kSRing - 1));
+                    const StreamWord W = stream_word(SR, S, cq);
                     const float cS = mm - s.pt.R2lo[si * 2 + S];
-                    unsigned inw = 0u;
                     float near = far;
-#pragma unroll
-                    for (int u = 0; u < 32; ++u) {
-                        const float d = stream_d(rp[u], m2x, m2y, m2z, cS);
-                        inw = __funnelshift_l(__float_as_uint(d), inw, 1);
-                        near = fminf(near, fabsf(d));
-                    }
+                    unsigned inw = word_signs(W, m2x, m2y, m2z, cS, near);
                     const int nv = fill[S] - cq;
                     unsigned valid = nv >= 32 ? 0xffffffffu : ~(0xffffffffu >> nv);
                     if (S == si && cself >= cq && cself < cq + 32)
@@ -1165,14 +1237,13 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
                         while (bw) {
                             const int u = __clz(bw);
                             bw &= 0x7fffffffu >> u;
-                            if (!(fabsf(stream_d(rp[u], m2x, m2y, m2z, cS)) < bS)) continue;
+                            if (!(fabsf(stream_d(W, u, m2x, m2y, m2z, cS)) < bS)) continue;
                             const unsigned bit = 0x80000000u >> u;
                             inw &= ~bit;
                             // (p' - m' is the separation up to FP32 rounding: enough to tell
                             // the minimum-image copy from one a box length away)
-                            const float4 r = rp[u];
-                            if (!min_image_copy(s, fmaf(m2x, 0.5f, r.x), fmaf(m2y, 0.5f, r.y),
-                                                fmaf(m2z, 0.5f, r.z)))
+                            if (!min_image_copy(s, fmaf(m2x, 0.5f, W.x[u]), fmaf(m2y, 0.5f, W.y[u]),
+                                                fmaf(m2z, 0.5f, W.z[u])))
                                 continue;
                             const int t = (int)SR.idx[S][(cq + u) & (kSRing - 1)];
                             const int64_t gj = staged_global(Rc, t);
@@ -1181,34 +1252,55 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
                     }
                     return inw;
                 };
-                // the set bits of stream S's word at cq as list entries, in stream order
+                // the set bits of stream S's word at cq as list entries, in stream order.  BUFFER:
+                // eight candidates at a time, each lane adds its own to its buffer, and lanes whose
+                // buffer holds a row of eight write it with one 16-byte store.  Else: each lane
+                // goes through its own bits, two at a time, one 4-byte store for both; an odd
+                // last entry waits for the next word's first
                 auto append_word = [&](int S, int cq, unsigned bits) {
-                    // the word's 32 entries are contiguous (word starts are multiples of 32
-                    // in a ring of 64)
-                    const uint16_t* const rw = SR.idx[S] + (cq & (kSRing - 1));
-                    // entries go out in pairs (one 32-bit store each at the running row
-                    // pointer; entries beyond the capacity are counted, not stored): a
-                    // pending odd entry is completed by the word's first bit, then two
-                    // bits per iteration; an odd last bit stays pending
-                    if ((len & 1) && bits) {
-                        const int u = __clz(bits);
-                        bits &= 0x7fffffffu >> u;
-                        put_pair(pend | ((unsigned)rw[u] << 16));
-                        ++len;
-                    }
-                    while (bits) {
-                        const int u1 = __clz(bits);
-                        bits &= 0x7fffffffu >> u1;
-                        const unsigned t1 = rw[u1];
-                        if (!bits) {
-                            pend = t1;
-                            ++len;
-                            break;
+                    if constexpr (BUFFER) {
+                        const uint4* const iw = reinterpret_cast<const uint4*>(SR.idx[S] + (cq & (kSRing - 1)));
+#pragma unroll
+                        for (int o = 0; o < 4; ++o) {
+                            const uint4 e = iw[o];
+                            const unsigned es[4] = {e.x, e.y, e.z, e.w};
+#pragma unroll
+                            for (int u = 0; u < 4; ++u)
+                                push_entries(top, es[u], bits, 0x80000000u >> (o * 8 + 2 * u));
+                            const bool full = top - top0 >= 16u;
+                            if (__any_sync(FULL, full) && full) {
+                                uint4* const b4 = reinterpret_cast<uint4*>(buf);
+                                if (row < s.lcap8) *rowp = b4[0];
+                                b4[0] = b4[1];
+                                top -= 16u;
+                                ++row;
+                                rowp += s.npad;
+                            }
                         }
-                        const int u2 = __clz(bits);
-                        bits &= 0x7fffffffu >> u2;
-                        put_pair(t1 | ((unsigned)rw[u2] << 16));
-                        len += 2;
+                    } else {
+                        // (the word's entries are contiguous: it starts at a multiple of 32 in a ring
+                        // of 64)
+                        const uint16_t* const rw = SR.idx[S] + (cq & (kSRing - 1));
+                        if ((len & 1) && bits) {
+                            const int u = __clz(bits);
+                            bits &= 0x7fffffffu >> u;
+                            put_pair(pend | ((unsigned)rw[u] << 16));
+                            ++len;
+                        }
+                        while (bits) {
+                            const int u1 = __clz(bits);
+                            bits &= 0x7fffffffu >> u1;
+                            const unsigned t1 = rw[u1];
+                            if (!bits) {
+                                pend = t1;
+                                ++len;
+                                break;
+                            }
+                            const int u2 = __clz(bits);
+                            bits &= 0x7fffffffu >> u2;
+                            put_pair(t1 | ((unsigned)rw[u2] << 16));
+                            len += 2;
+                        }
                     }
                 };
                 // a stream's word is tested and appended as soon as it is full (fewer than
@@ -1242,6 +1334,8 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
                 };
                 flush_last(0);
                 flush_last(1);
+                const int left = (int)(top - top0) >> 1;
+                if constexpr (BUFFER) len = row * 8 + left;
                 if (len > lcap) {
                     // the list is cut: flagged for the host (which grows the capacity at its
                     // next synchronising call) and, until then, the forces come from the
@@ -1249,20 +1343,22 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
                     set_status(s, ST_LIST_OVERFLOW);
                     s.sc->list_short = 1;
                     atomicMax(&s.sc->max_len, len);
-                    len = lcap;
-                }
-                if (act && (len & 1)) {
-                    const int wi = len >> 1;
-                    row0[(int64_t)(wi >> 2) * rowstep + (wi & 3)] = pend | ((unsigned)s.smax << 16);
-                    ++len;
                 }
                 if (act) {
-                    // the rest of the last row holds sentinel pairs; the particle's row count
-                    // tells the force kernels where its list ends
-                    const int rows = (len + 7) >> 3;
-                    for (int wi = len >> 1; wi < rows * 4; ++wi)
-                        row0[(int64_t)(wi >> 2) * rowstep + (wi & 3)] = sentpair;
-                    s.rows[gi] = (uint16_t)rows;
+                    // the rest of the last row holds the sentinel; the particle's row count tells
+                    // the force kernels where its list ends
+                    if constexpr (BUFFER) {
+                        if (left > 0) {
+                            for (int k = left; k < 8; ++k) buf[k] = (uint16_t)s.smax;
+                            if (row < s.lcap8) *rowp = *reinterpret_cast<const uint4*>(buf);
+                            ++row;
+                        }
+                    } else {
+                        if (len & 1) put_pair(pend | ((unsigned)s.smax << 16));
+                        while (wp & 3) put_pair((unsigned)s.smax | ((unsigned)s.smax << 16));
+                        row = wp >> 2;
+                    }
+                    s.rows[gi] = (uint16_t)min(row, s.lcap8);
                 }
             }
         }
@@ -1370,7 +1466,7 @@ __device__ __forceinline__ bool grid_rebuild(const DevSim& s, unsigned& gen, OnL
     copyback_body(s, lb, lg);
     if (s.nbr_mode == BBMD_NBR_VERLET) {
         if (!grid_barrier(s, gen)) return false;
-        for (int b = lb; b < s.grid_list; b += lg) list_build_body(s, b, s.grid_list);
+        for (int b = lb; b < s.grid_list; b += lg) list_build_body<true>(s, b, s.grid_list);
     }
     return grid_barrier(s, gen, true, on_last);
 }
@@ -1469,7 +1565,7 @@ __device__ __forceinline__ void run_phase(int phase, const DevSim& s, int lb, in
         case kPhCellsort: cellsort_body(s, lb, lg); break;
         case kPhGather: gather_body(s, lb, lg); break;
         case kPhCopyback: copyback_body(s, lb, lg); break;
-        case kPhList: list_build_body(s, lb, lg); break;
+        case kPhList: list_build_body<true>(s, lb, lg); break;
         case kPhForce:
             // the list body, or for a replica whose lists are cut (and in cell mode) the
             // stencil body: each returns at once when not selected
@@ -1896,15 +1992,17 @@ __global__ void __launch_bounds__(kBW * 32, MODE == 1 ? BBMD_CELL_MIN_BLOCKS : B
     force_body<MODE, KE, FSHIFT>(sh, lb, lg);
 }
 
+constexpr bool kListBuffer = BBMD_BLOCK_Z != 4;  // (see the list build)
+
 __global__ void __launch_bounds__(kBW * 32, BBMD_LIST_MIN_BLOCKS) k_list_build(DevSim s) {
-    list_build_body(s, (int)blockIdx.x, (int)gridDim.x);
+    list_build_body<kListBuffer>(s, (int)blockIdx.x, (int)gridDim.x);
 }
 
 __global__ void __launch_bounds__(kBW * 32, BBMD_LIST_MIN_BLOCKS) k_list_build_many(ManySims m) {
     __shared__ DevSim sh;
     int lb, lg;
     load_replica(m, sh, lb, lg);
-    list_build_body(sh, lb, lg);
+    list_build_body<kListBuffer>(sh, lb, lg);
 }
 
 template <int MODE, int WHAT, bool KE, bool FSHIFT>
