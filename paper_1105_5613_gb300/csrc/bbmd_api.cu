@@ -40,6 +40,7 @@ struct bbmd_sim {
     int64_t n_species[2] = {0, 0};   // particles of each species (fixed at creation)
     double mean_cell = 0.0;          // mean particles per cell
     std::vector<int> shapes;         // block shapes that fit (candidates of the autotuner)
+    int sums_shape = 0;              // block shape of the FP64 energy passes
     int grid_shape = -1, grid_ctas = 0;  // one-launch step: block shape it was sized for, CTAs
     float shape_ms[4][2] = {};       // autotuner: per kShapes entry, force and list-build ms
 };
@@ -261,27 +262,57 @@ bool shape_fits(const bbmd_sim* sim, int bz) {
     return smax <= 65000 && bytes <= 200 * 1024;
 }
 
-// Select block shape bz: geometry, staged capacity and the grids of the block kernels.
-void apply_shape(bbmd_sim* sim, int bz) {
-    DevSim& D = sim->d;
+// Geometry and staged capacity of block shape bz.
+void shape_geometry(const bbmd_sim* sim, int bz, DevSim& D) {
     D.block_z = bz;
     D.region_cells = region_cells_of(bz);
     D.smax = shape_smax(sim, bz);
     const int bxy = block_xy_of(bz), bzc = block_zc_of(bz);
     D.nblocks = (int64_t)((D.nc[0] + bxy - 1) / bxy) * ((D.nc[1] + bxy - 1) / bxy) *
                 ((D.nc[2] + bzc - 1) / bzc);
-    int64_t g = (int64_t)sim->nsm * force_blocks_per_sm(D);
-    if (g > D.nblocks) g = D.nblocks;
-    if (g > kMaxPartials) g = kMaxPartials;
-    D.grid_cell = (int32_t)(g > 0 ? g : 1);
-    g = (int64_t)sim->nsm * list_blocks_per_sm(D);
-    if (g > D.nblocks) g = D.nblocks;
-    D.grid_list = (int32_t)(g > 0 ? g : 1);
+}
+
+int32_t block_grid(const bbmd_sim* sim, const DevSim& D, int per_sm) {
+    return (int32_t)std::max<int64_t>(
+        1, std::min({(int64_t)sim->nsm * per_sm, (int64_t)D.nblocks, (int64_t)kMaxPartials}));
+}
+
+// Select block shape bz: geometry, staged capacity and the grids of the block kernels.
+void apply_shape(bbmd_sim* sim, int bz) {
+    DevSim& D = sim->d;
+    shape_geometry(sim, bz, D);
+    D.grid_cell = block_grid(sim, D, force_blocks_per_sm(D));
+    D.grid_list = (int32_t)std::max<int64_t>(
+        1, std::min<int64_t>((int64_t)sim->nsm * list_blocks_per_sm(D), D.nblocks));
+    // the FP64 energy passes: their own occupancy (as many CTAs as the force kernel's would
+    // leave a last wave of a few).  Without stored lists any shape serves them, and 2 x 2 x 2
+    // runs two CTAs per SM where the larger shapes run one: 2.05 M in cell mode 4.4 ms against
+    // 6.5 (2 x 2 x 4) and 6.9 (4 x 4 x 2)
+    sim->sums_shape = bz;
+    if (D.nbr_mode != BBMD_NBR_VERLET && bz > 2 && shape_fits(sim, 2)) sim->sums_shape = 2;
+    DevSim S = D;
+    shape_geometry(sim, sim->sums_shape, S);
+    D.grid_sums = block_grid(sim, S, energies_blocks_per_sm(S));
+}
+
+// The system as the FP64 energy passes see it.
+DevSim sums_sim(const bbmd_sim* sim) {
+    DevSim S = sim->d;
+    if (sim->sums_shape != S.block_z) shape_geometry(sim, sim->sums_shape, S);
+    return S;
 }
 
 bbmd_status rebuild_now(bbmd_sim* sim);
 bbmd_status refresh_forces_and_K(bbmd_sim* sim);
 void finish_velocities(bbmd_sim* sim);
+
+// Forces of the current positions and, with energies, u_i.
+void launch_forces_and_energies(bbmd_sim* sim, bool energies) {
+    const bool fp64 = sim->d.precision == BBMD_PREC_FP64;
+    launch_force(sim->d, sim->st, energies && fp64, false);
+    if (energies && !fp64) launch_energies(sums_sim(sim), sim->st, true);
+}
+
 void free_graphs(bbmd_sim* sim);
 
 // A list build cut some lists at the capacity (Verlet mode).  The steps since then took
@@ -465,19 +496,29 @@ void begin_call(bbmd_sim* sim, int64_t nsteps, double dt, const bbmd_thermostat*
 //   - steepest descent (whose launches are not a captured graph) up to kGridRelaxMax particles:
 //     79 -> 25 at 4000, 99 -> 30 at 32 000, 222 -> 118 at 256 000, 314 -> 223 at 500 000.
 constexpr int64_t kGridRelaxMax = 500000;
+// Largest system whose captured step runs the rebuild trigger and the sort chain as one
+// cooperative launch (k_trigger_sort): it saves the skipped launches, and its rebuilds are
+// slower than full grids'.  Microseconds a step at T = 2, 11 launches -> one: 256 000 particles
+// 139 -> 133, 500 000 219 -> 212, 1.0 M 396 -> 395, 2.0 M 724 -> 730, 6.9 M 2413 -> 2469.
+constexpr int64_t kTriggerSortMax = 1000000;
 constexpr int64_t kGridSteps = 1024;  // steps per launch
+
+// Whether the handle's device runs cooperative launches.
+bool cooperative(const bbmd_sim* sim) {
+    int coop = 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, sim->device) != cudaSuccess) {
+        cudaGetLastError();
+        coop = 0;
+    }
+    return coop != 0;
+}
 
 // CTAs of the one-launch kernels for this handle's shape (0 where they do not run), and
 // whether every block has one.
 int grid_step_grid(bbmd_sim* sim, bool* one_wave) {
     if (sim->d.precision != BBMD_PREC_MIXED) return 0;
     if (sim->grid_shape != sim->d.block_z) {
-        int coop = 0;
-        if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, sim->device) != cudaSuccess) {
-            cudaGetLastError();
-            coop = 0;
-        }
-        sim->grid_ctas = coop ? grid_step_ctas(sim->d, sim->nsm) : 0;
+        sim->grid_ctas = cooperative(sim) ? grid_step_ctas(sim->d, sim->nsm) : 0;
         sim->grid_shape = sim->d.block_z;
     }
     *one_wave = sim->grid_ctas >= sim->d.nblocks;
@@ -495,8 +536,13 @@ bbmd_status build_graph(bbmd_sim* sim, int nh) {
     cudaGraph_t g;
     CK(cudaStreamBeginCapture(sim->st, cudaStreamCaptureModeThreadLocal));
     launch_integrate(sim->d, sim->st);
-    launch_check(sim->d, sim->st);
-    enqueue_rebuild(sim);
+    const int grid = sim->d.n <= kTriggerSortMax ? trigger_sort_ctas(sim->d, sim->nsm) : 0;
+    if (grid > 0 && cooperative(sim) && launch_trigger_sort(sim->d, grid, sim->st) == cudaSuccess) {
+        launch_list_build(sim->d, sim->st);
+    } else {
+        launch_check(sim->d, sim->st);
+        enqueue_rebuild(sim);
+    }
     launch_force(sim->d, sim->st, false, nh != 0);
     launch_finalize(sim->d, sim->st, nh != 0);
     cudaError_t e = cudaStreamEndCapture(sim->st, &g);
@@ -824,7 +870,7 @@ bbmd_status bbmd_observe(bbmd_sim* sim, uint32_t mask, const bbmd_obs_args* args
     // kinetic energy and momentum
     const bool energy = (mask & (BBMD_OBS_ENERGY | BBMD_OBS_VIRIAL)) != 0;
     launch_state_sums(D, sim->st);
-    if (energy) launch_energy_sums(D, sim->st);
+    if (energy) launch_energies(sums_sim(sim), sim->st, false);
     launch_observe_sums(D, sim->st, energy, sim->dout);
     const int origin = args ? args->origin : 0;
     if (origin < 0 || origin >= BBMD_MAX_ORIGINS)
@@ -1015,7 +1061,7 @@ bbmd_status bbmd_get_forces_ids(bbmd_sim* sim, const int64_t* ids, int64_t m, do
     for (int64_t t = 0; t < m; ++t)
         if (ids[t] < 0 || ids[t] >= n) return fail(sim, BBMD_ERR_ARG, "ids must be in [0, n)");
     if (m == 0) return BBMD_OK;
-    launch_force(sim->d, sim->st, u != nullptr, false);
+    launch_forces_and_energies(sim, u != nullptr);
     int32_t* slot_of = (int32_t*)dev_alloc(sim, (size_t)n * 4);
     int64_t* dids = (int64_t*)dev_alloc(sim, (size_t)m * 8);
     double* tf = (double*)dev_alloc(sim, (size_t)m * 24);
@@ -1046,7 +1092,7 @@ bbmd_status bbmd_get_forces(bbmd_sim* sim, double* F, double* u) {
     if (!sim || !F) return BBMD_ERR_ARG;
     DeviceGuard dg(sim->device);
     const int64_t n = sim->d.n;
-    launch_force(sim->d, sim->st, u != nullptr, false);
+    launch_forces_and_energies(sim, u != nullptr);
     double* const tf = stage_pos(sim);
     double* const tu = u ? stage_vel(sim) : nullptr;
     launch_unpack_forces(sim->d, sim->st, tf, tu);

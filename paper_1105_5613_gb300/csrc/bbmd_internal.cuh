@@ -127,6 +127,7 @@ struct alignas(16) DevSim {
     int32_t grid_part;       // grid of per-particle grid-stride kernels
     int32_t grid_cell;       // grid of the force kernel (kBlockWarps warps per CTA)
     int32_t grid_list;       // grid of the list-build kernel
+    int32_t grid_sums;       // grid of the FP64 energy passes
 };
 
 // ---------------------------------------------------------------- conversions ----
@@ -267,12 +268,17 @@ __device__ __forceinline__ void load_replica(const ManySims& m, DevSim& sh, int&
 
 // sort / rebuild chain (gated on sc->rebuild unless noted)
 void launch_rebuild_chain(const DevSim& s, cudaStream_t st);
+// rebuild trigger and sort chain in one cooperative launch of trigger_sort_ctas CTAs (0: no
+// such launch); the barrier words must be zero (k_begin, k_finalize)
+int trigger_sort_ctas(const DevSim& s, int nsm);
+cudaError_t launch_trigger_sort(const DevSim& s, int grid, cudaStream_t st);
 // Per block shape (namespace z1, z2, z4, z8; defined in k_force.cu compiled per shape):
 //   prepare_force_kernels  one-time kernel attributes (call before any stream capture)
 //   force/list_blocks_per_sm  resident CTAs per SM for this handle's shared memory
-//   launch_force   forces; energy: also per-particle energy and virial partials (not with
-//                  ke); ke: NH kinetic partials
-//   launch_energy_sums  energy and virial partials only
+//   launch_force   forces; energy: also per-particle energies (the FP64 form, not with ke);
+//                  ke: NH kinetic partials
+//   launch_energies  energy and virial partials of grid_sums CTAs; each: also per-particle
+//                  energies
 //   launch_list_build  Verlet list build (gated)
 //   launch_grid_step   many whole steps of a small mixed-precision system in one cooperative
 //                  launch of grid_step_ctas CTAs (0: no such launch); launch_grid_relax the
@@ -288,7 +294,8 @@ void launch_rebuild_chain(const DevSim& s, cudaStream_t st);
     int list_blocks_per_sm(const DevSim& s);                                           \
     int block_threads();                                                               \
     void launch_force(const DevSim& s, cudaStream_t st, bool energy, bool ke);         \
-    void launch_energy_sums(const DevSim& s, cudaStream_t st);                         \
+    void launch_energies(const DevSim& s, cudaStream_t st, bool each);                 \
+    int energies_blocks_per_sm(const DevSim& s);                                       \
     void launch_list_build(const DevSim& s, cudaStream_t st);                          \
     int grid_step_ctas(const DevSim& s, int nsm);                                      \
     cudaError_t launch_grid_step(const DevSim& s, int grid, int nsteps, bool ke, cudaStream_t st); \
@@ -352,8 +359,11 @@ inline int list_blocks_per_sm(const DevSim& s) { BBMD_SHAPE_DISPATCH(s.block_z, 
 inline void launch_force(const DevSim& s, cudaStream_t st, bool energy, bool ke) {
     BBMD_SHAPE_DISPATCH(s.block_z, launch_force(s, st, energy, ke))
 }
-inline void launch_energy_sums(const DevSim& s, cudaStream_t st) {
-    BBMD_SHAPE_DISPATCH(s.block_z, launch_energy_sums(s, st))
+inline void launch_energies(const DevSim& s, cudaStream_t st, bool each) {
+    BBMD_SHAPE_DISPATCH(s.block_z, launch_energies(s, st, each))
+}
+inline int energies_blocks_per_sm(const DevSim& s) {
+    BBMD_SHAPE_DISPATCH(s.block_z, energies_blocks_per_sm(s))
 }
 inline int grid_step_ctas(const DevSim& s, int nsm) {
     BBMD_SHAPE_DISPATCH(s.block_z, grid_step_ctas(s, nsm))

@@ -1,0 +1,103 @@
+// Grid-wide barrier of the cooperative kernels, and the rebuild trigger and sort chain run
+// phase after phase inside one launch.  Included inside an anonymous namespace, after
+// sort_bodies.cuh and step_bodies.cuh.
+#pragma once
+
+__device__ __forceinline__ unsigned long long globaltimer_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
+constexpr unsigned long long kGridWaitNs = 2000000000ull;  // a barrier wait gives up after it
+
+// Barrier over the CTAs of the launch; gen counts the barriers passed.  With `last` set, the
+// last CTA to arrive runs on_last before the others go on.  Every CTA is resident
+// (cooperative launch), so a wait ends; should one not end within kGridWaitNs, the CTA
+// raises the abort flag and ST_TIMEOUT, and every CTA leaves (false) at its next barrier.
+template <class OnLast>
+__device__ __forceinline__ bool grid_barrier(const DevSim& s, unsigned& gen, bool last, OnLast on_last) {
+    __shared__ int verdict;  // 0: abort, 1: go on, 2: this CTA arrived last
+    volatile uint32_t* const w = s.gsync;
+    ++gen;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const unsigned target = gen * gridDim.x;
+        const bool mine = atomicAdd(&s.gsync[kSyncArrive * kSyncStride], 1u) + 1u == target;
+        int v = 1;
+        if (last && mine) {
+            v = 2;
+        } else {
+            const int word = (last ? kSyncRelease : kSyncArrive) * kSyncStride;
+            const unsigned want = last ? gen : target;
+            unsigned long long t0 = 0;
+            for (unsigned it = 0; w[word] < want; ++it) {
+                if ((it & 63u) != 63u) continue;
+                if (t0 == 0) t0 = globaltimer_ns();
+                if (w[kSyncAbort * kSyncStride] != 0u || globaltimer_ns() - t0 > kGridWaitNs) {
+                    w[kSyncAbort * kSyncStride] = 1u;
+                    set_status(s, ST_TIMEOUT);
+                    v = 0;
+                    break;
+                }
+            }
+        }
+        __threadfence();
+        verdict = v;
+    }
+    __syncthreads();
+    const int v = verdict;
+    if (v == 2) {
+        on_last();
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            __threadfence();
+            w[kSyncRelease * kSyncStride] = gen;
+        }
+    }
+    __syncthreads();  // (verdict is written again at the next barrier)
+    // data of earlier phases, written by other CTAs, is read by bulk copies (the async
+    // proxy) as well as by ordinary loads
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    return v != 0;
+}
+
+__device__ __forceinline__ bool grid_barrier(const DevSim& s, unsigned& gen) {
+    return grid_barrier(s, gen, false, [] {});
+}
+
+// Rebuild trigger after the integrate phase (whose flags the caller has put behind a barrier):
+// due, the same on every thread, tells whether a rebuild is due; the cell counts are then
+// zero.  False after an abort.
+__device__ __forceinline__ bool grid_trigger(const DevSim& s, unsigned& gen, bool& due) {
+    const int lb = (int)blockIdx.x, lg = (int)gridDim.x;
+    due = false;
+    if (!*(volatile int*)&s.sc->near) return true;
+    celltop_body(s, lb, lg);
+    zero_counts(s, lb, lg);
+    if (!grid_barrier(s, gen)) return false;
+    check_body(s, lb, lg);
+    if (!grid_barrier(s, gen)) return false;
+    due = *(volatile int*)&s.sc->rebuild != 0;
+    return true;
+}
+
+// Sort chain of a rebuild whose flag is up and whose cell counts are zero (no barrier after
+// the last phase).
+__device__ __forceinline__ bool grid_sort(const DevSim& s, unsigned& gen) {
+    const int lb = (int)blockIdx.x, lg = (int)gridDim.x;
+    clear_list_flags(s, lb);
+    bin_body(s, lb, lg);
+    if (!grid_barrier(s, gen)) return false;
+    scan_cta_body(s, lb, lg);
+    if (!grid_barrier(s, gen)) return false;
+    scatter_body(s, lb, lg);
+    if (!grid_barrier(s, gen)) return false;
+    cellsort_body(s, lb, lg);
+    if (!grid_barrier(s, gen)) return false;
+    gather_body(s, lb, lg);
+    if (!grid_barrier(s, gen)) return false;
+    copyback_body(s, lb, lg);
+    return true;
+}

@@ -1378,95 +1378,21 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
 // of 70 (its list build 45).
 #include "sort_bodies.cuh"
 #include "step_bodies.cuh"
-
-__device__ __forceinline__ unsigned long long globaltimer_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
-constexpr unsigned long long kGridWaitNs = 2000000000ull;  // a barrier wait gives up after it
+#include "grid_bodies.cuh"
 
 #ifndef BBMD_GRID_MIN_BLOCKS
 #define BBMD_GRID_MIN_BLOCKS (BBMD_BLOCK_Z == 1 ? 4 : 2)
 #endif
 
-// Barrier over the CTAs of the launch; gen counts the barriers passed.  With `last` set, the
-// last CTA to arrive runs on_last before the others go on.  Every CTA is resident
-// (cooperative launch), so a wait ends; should one not end within kGridWaitNs, the CTA
-// raises the abort flag and ST_TIMEOUT, and every CTA leaves (false) at its next barrier.
-template <class OnLast>
-__device__ __forceinline__ bool grid_barrier(const DevSim& s, unsigned& gen, bool last, OnLast on_last) {
-    __shared__ int verdict;  // 0: abort, 1: go on, 2: this CTA arrived last
-    volatile uint32_t* const w = s.gsync;
-    ++gen;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        const unsigned target = gen * gridDim.x;
-        const bool mine = atomicAdd(&s.gsync[kSyncArrive * kSyncStride], 1u) + 1u == target;
-        int v = 1;
-        if (last && mine) {
-            v = 2;
-        } else {
-            const int word = (last ? kSyncRelease : kSyncArrive) * kSyncStride;
-            const unsigned want = last ? gen : target;
-            unsigned long long t0 = 0;
-            for (unsigned it = 0; w[word] < want; ++it) {
-                if ((it & 63u) != 63u) continue;
-                if (t0 == 0) t0 = globaltimer_ns();
-                if (w[kSyncAbort * kSyncStride] != 0u || globaltimer_ns() - t0 > kGridWaitNs) {
-                    w[kSyncAbort * kSyncStride] = 1u;
-                    set_status(s, ST_TIMEOUT);
-                    v = 0;
-                    break;
-                }
-            }
-        }
-        __threadfence();
-        verdict = v;
-    }
-    __syncthreads();
-    const int v = verdict;
-    if (v == 2) {
-        on_last();
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            __threadfence();
-            w[kSyncRelease * kSyncStride] = gen;
-        }
-    }
-    __syncthreads();  // (verdict is written again at the next barrier)
-    // data of earlier phases, written by other CTAs, is read by bulk copies (the async
-    // proxy) as well as by ordinary loads
-    asm volatile("fence.proxy.async.global;" ::: "memory");
-    return v != 0;
-}
-
-__device__ __forceinline__ bool grid_barrier(const DevSim& s, unsigned& gen) {
-    return grid_barrier(s, gen, false, [] {});
-}
-
 // The rebuild after its flag is up and the cell counts are zero: sort chain and list build.
 // on_last runs once at the end.
 template <class OnLast>
 __device__ __forceinline__ bool grid_rebuild(const DevSim& s, unsigned& gen, OnLast on_last) {
-    const int lb = (int)blockIdx.x, lg = (int)gridDim.x;
-    clear_list_flags(s, lb);
-    bin_body(s, lb, lg);
-    if (!grid_barrier(s, gen)) return false;
-    scan_cta_body(s, lb, lg);
-    if (!grid_barrier(s, gen)) return false;
-    scatter_body(s, lb, lg);
-    if (!grid_barrier(s, gen)) return false;
-    cellsort_body(s, lb, lg);
-    if (!grid_barrier(s, gen)) return false;
-    gather_body(s, lb, lg);
-    if (!grid_barrier(s, gen)) return false;
-    copyback_body(s, lb, lg);
+    if (!grid_sort(s, gen)) return false;
     if (s.nbr_mode == BBMD_NBR_VERLET) {
         if (!grid_barrier(s, gen)) return false;
-        for (int b = lb; b < s.grid_list; b += lg) list_build_body<true>(s, b, s.grid_list);
+        for (int b = (int)blockIdx.x; b < s.grid_list; b += (int)gridDim.x)
+            list_build_body<true>(s, b, s.grid_list);
     }
     return grid_barrier(s, gen, true, on_last);
 }
@@ -1487,15 +1413,9 @@ __global__ void __launch_bounds__(kBW * 32, BBMD_GRID_MIN_BLOCKS) k_step_grid(De
     for (int step = 0; step < nsteps; ++step) {
         integrate_body<false>(s, lb, lg);
         if (!grid_barrier(s, gen)) return;
-        if (*(volatile int*)&s.sc->near) {
-            celltop_body(s, lb, lg);
-            zero_counts(s, lb, lg);
-            if (!grid_barrier(s, gen)) return;
-            check_body(s, lb, lg);
-            if (!grid_barrier(s, gen)) return;
-            if (*(volatile int*)&s.sc->rebuild)
-                if (!grid_rebuild(s, gen, [] {})) return;
-        }
+        bool due;
+        if (!grid_trigger(s, gen, due)) return;
+        if (due && !grid_rebuild(s, gen, [] {})) return;
         grid_force<KE, FSHIFT>(s);
         if (!grid_barrier(s, gen, true, [&] { finalize_body(s, KE ? 1 : 0); })) return;
     }
@@ -1658,15 +1578,17 @@ __global__ void __launch_bounds__(kBW * 32, 2) k_step_persistent(PersistentStep 
 //   - each lane queues its interacting candidates (shared memory) and the warp drains the
 //     queues together, so a slot of the loop computes a pair on nearly every lane, instead
 //     of once per candidate that any of the 32 lanes interacts with;
-//   - r^2 stays in integer units (the scale is folded into sigma^2), 1/r^2 and 1/r come
+//   - r^2 stays in integer units (the scale is folded into the constants), 1/r^2 and 1/r come
 //     from the hardware's approximation and one third-order step, and energies and virial
-//     come from the sums of s^12 and s^6;
+//     come from the sums of r^-12 and r^-6 by species pair: 17 operations a pair for forces,
+//     13 for the sums;
 //   - sums over the system (energy, virial) take each pair from one side only.
 // Measured against the form that ran the FP64 arithmetic for every candidate some lane of
 // the warp interacts with: energy and virial sums at 16.4 M particles (lists, skin 0.4)
-// 132 -> 24 ms, at 4 M in cell mode 121 -> 13.6 ms; forces of the FP64 form at 108 000
-// 0.868 -> 0.383 ms.  (17 to 19 FP64 instructions a pair at 0.63e12 lanes a second put the
-// floor of the three at 14, 3.5 and 0.21 ms.)
+// 132 -> 23 ms, at 4 M in cell mode 121 -> 8.6 ms; forces of the FP64 form at 108 000
+// 0.868 -> 0.347 ms.  (At 0.63e12 lanes a second the pairs' operations take 11, 2.7 and 0.19 ms.
+// Every shape measures the same at 2 M; converting the integers with two additions instead of
+// a conversion instruction was 15 % slower.)
 
 // Staged record t: hi[t] = upper words of x, y, z and (global index << 1 | species), lo[t] =
 // lower words.
@@ -1742,11 +1664,13 @@ __device__ __forceinline__ uint16_t* warp_queue64(int w) {
 // energy and virial alone.
 enum : int { k64Force = 1, k64Energy = 2, k64Sums = 4 };
 
-// One lane's pair constants and accumulators, in units of 2^-k (r^2 and forces).
+// One lane's pair constants and accumulators; r^2 and forces in units of 2^-k, so the constants
+// of r^-6 carry 2^6k.
 struct Lane64 {
-    double sig20, sig21, e40, e41, dc0, dc1;  // sigma^2 2^2k, 4 eps, dV/dr(rc) 2^-k
-    double fx, fy, fz;                        // sum of f d, integer units
-    double s12, s6, sr;                       // sums of 4 eps s^12, 4 eps s^6, dV/dr(rc) r
+    double a0, a1, b0, b1;                    // 48 eps sigma^12 2^6k, 24 eps sigma^6 (0: soft)
+    double dc0, dc1;                          // dV/dr(rc) 2^-7k
+    double fx, fy, fz;                        // sum of f d
+    double t0, t1, u0, u1, q0, q1;            // sums of r^-12, r^-6, r by species of j
     int n0, n1;                               // interacting pairs by species of j
 };
 
@@ -1776,24 +1700,31 @@ __device__ __forceinline__ void pair_fp64(const DevSim& s, int si, long long mx,
     } else {
         ir2 = rcp64(r2);
     }
-    const double s2 = (b ? A.sig21 : A.sig20) * ir2;
-    const double s6 = s2 * s2 * s2;
-    const double w6 = (b ? A.e41 : A.e40) * s6;  // 4 eps s^6
-    const bool lj = s.pt.potential == BBMD_POT_LJ;
+    const double ir4 = ir2 * ir2;
+    const double ir6 = ir4 * ir2;
     if (WHAT & k64Force) {
-        // f / 12 = 4 eps s^6 (s^6 - 1/2) / r^2 (+ dV/dr(rc) / (12 r)); the 12 is applied
-        // to the finished sum
-        double f = fma(w6, s6, lj ? -0.5 * w6 : 0.0) * ir2;
-        if (FSHIFT) f = fma(b ? A.dc1 : A.dc0, ir * (1.0 / 12.0), f);
+        // f = (48 eps sigma^12 r^-6 - 24 eps sigma^6) r^-8 (+ dV/dr(rc) / r): the units of
+        // r^-8 and d, 2^7k, are applied to the finished sum
+        double f = fma(b ? A.a1 : A.a0, ir6, b ? A.b1 : A.b0) * (ir4 * ir4);
+        if (FSHIFT) f = fma(b ? A.dc1 : A.dc0, ir, f);
         A.fx = fma(f, dx, A.fx);
         A.fy = fma(f, dy, A.fy);
         A.fz = fma(f, dz, A.fz);
     }
     if (WHAT & (k64Energy | k64Sums)) {
-        A.s12 = fma(w6, s6, A.s12);
-        A.s6 += w6;
-        if (FSHIFT) A.sr = fma(b ? A.dc1 : A.dc0, r, A.sr);
-        if (b) ++A.n1; else ++A.n0;
+        // (selects, not branches: a divergent branch would take the FP64 pipe twice)
+        const double tn = fma(ir6, ir6, b ? A.t1 : A.t0), un = (b ? A.u1 : A.u0) + ir6;
+        A.t0 = b ? A.t0 : tn;
+        A.t1 = b ? tn : A.t1;
+        A.u0 = b ? A.u0 : un;
+        A.u1 = b ? un : A.u1;
+        if (FSHIFT) {
+            const double qn = (b ? A.q1 : A.q0) + r;
+            A.q0 = b ? A.q0 : qn;
+            A.q1 = b ? qn : A.q1;
+        }
+        A.n0 += b ? 0 : 1;
+        A.n1 += b ? 1 : 0;
     }
 }
 
@@ -1836,17 +1767,22 @@ __device__ __forceinline__ void force64_body(const DevSim& s, int lb, int lg) {
                 in2[b] = lo > 0.f ? lo * lo : 0.f;
                 out2[b] = hi * hi;
             }
+            const int kp = si * 2;
             Lane64 A;
-            A.sig20 = ldexp(s.pt.dsig2[si * 2], 2 * s.kexp);
-            A.sig21 = ldexp(s.pt.dsig2[si * 2 + 1], 2 * s.kexp);
-            A.e40 = s.pt.deps4[si * 2];
-            A.e41 = s.pt.deps4[si * 2 + 1];
-            A.dc0 = A.dc1 = 0.0;
-            if (FSHIFT) {
-                A.dc0 = s.pt.dfcut[si * 2] * s.sxd;
-                A.dc1 = s.pt.dfcut[si * 2 + 1] * s.sxd;
+            {
+                const double c0 = s.pt.dsig2[kp] * s.pt.dsig2[kp] * s.pt.dsig2[kp];  // sigma^6
+                const double c1 = s.pt.dsig2[kp + 1] * s.pt.dsig2[kp + 1] * s.pt.dsig2[kp + 1];
+                A.a0 = ldexp(s.pt.deps48[kp] * c0 * c0, 6 * s.kexp);
+                A.a1 = ldexp(s.pt.deps48[kp + 1] * c1 * c1, 6 * s.kexp);
+                A.b0 = lj ? -0.5 * s.pt.deps48[kp] * c0 : 0.0;
+                A.b1 = lj ? -0.5 * s.pt.deps48[kp + 1] * c1 : 0.0;
+                A.dc0 = A.dc1 = 0.0;
+                if (FSHIFT) {
+                    A.dc0 = ldexp(s.pt.dfcut[kp], -7 * s.kexp);
+                    A.dc1 = ldexp(s.pt.dfcut[kp + 1], -7 * s.kexp);
+                }
             }
-            A.fx = A.fy = A.fz = A.s12 = A.s6 = A.sr = 0.0;
+            A.fx = A.fy = A.fz = A.t0 = A.t1 = A.u0 = A.u1 = A.q0 = A.q1 = 0.0;
             A.n0 = A.n1 = 0;
             int cnt = 0;
             // classify candidate t; queue it unless it is beyond the cutoff
@@ -1925,7 +1861,7 @@ __device__ __forceinline__ void force64_body(const DevSim& s, int lb, int lg) {
             drain(0);
             double Fx = 0.0, Fy = 0.0, Fz = 0.0;
             if (WHAT & k64Force) {
-                const double c = -12.0 / s.sxd;  // (a power of two: exact)
+                const double c = -ldexp(1.0, 7 * s.kexp);
                 Fx = A.fx * c;
                 Fy = A.fy * c;
                 Fz = A.fz * c;
@@ -1947,15 +1883,20 @@ __device__ __forceinline__ void force64_body(const DevSim& s, int lb, int lg) {
             if ((WHAT & (k64Energy | k64Sums)) && act) {
                 // V = 4 eps (s^12 - s^6) - V(rc) - (r - rc) dV/dr(rc), summed; virial
                 // f r^2 = 12 (4 eps s^12) - 6 (4 eps s^6) + r dV/dr(rc) (soft sphere: no s^6)
-                const int k = si * 2;
-                double c0 = s.pt.dvshift[k], c1 = s.pt.dvshift[k + 1];
-                if (FSHIFT) {
-                    c0 -= s.pt.drc[k] * s.pt.dfcut[k];
-                    c1 -= s.pt.drc[k + 1] * s.pt.dfcut[k + 1];
+                double u = 0.0, wv = 0.0;
+#pragma unroll
+                for (int b = 0; b < 2; ++b) {
+                    const double sg6 = s.pt.dsig2[kp + b] * s.pt.dsig2[kp + b] * s.pt.dsig2[kp + b];
+                    const double e6 = s.pt.deps4[kp + b] * sg6;
+                    // (the units of the sums, 2^12k and 2^6k, in two steps within range)
+                    const double s12 = ldexp(ldexp(b ? A.t1 : A.t0, 6 * s.kexp) * sg6, 6 * s.kexp) * e6;
+                    const double s6 = lj ? ldexp(b ? A.u1 : A.u0, 6 * s.kexp) * e6 : 0.0;
+                    const double dc = FSHIFT ? s.pt.dfcut[kp + b] : 0.0;
+                    const double sr = FSHIFT ? (b ? A.q1 : A.q0) * s.sxd * dc : 0.0;
+                    const double cut = s.pt.dvshift[kp + b] - s.pt.drc[kp + b] * dc;
+                    u += ((s12 - s6) - sr) - (double)(b ? A.n1 : A.n0) * cut;
+                    wv += fma(12.0, s12, fma(-6.0, s6, sr));
                 }
-                const double s6 = lj ? A.s6 : 0.0;
-                const double u = ((A.s12 - s6) - A.sr) - ((double)A.n0 * c0 + (double)A.n1 * c1);
-                const double wv = fma(12.0, A.s12, fma(-6.0, s6, A.sr));
                 const double half = WHAT & k64Sums ? 1.0 : 0.5;
                 if (WHAT & k64Energy) s.ud[gi] = half * u;
                 acc_u += half * u;
@@ -2042,9 +1983,7 @@ void set_smem(K kernel) {
 // Dynamic shared memory of the FP64 kernels: upper and lower words of every staged record.
 static size_t smem64(int smax) { return (size_t)(smax + 1) * 32; }
 
-// Mixed precision: FP32 forces; an energy pass (E) adds the FP64 energy kernel, which
-// writes the per-particle energies and the energy and virial partials from exact integer
-// positions (FP32 coordinates would limit u_i to about 1e-4) and leaves the forces alone.
+// E: with per-particle energies (the FP64 form only; mixed precision has launch_energies).
 template <int MODE, bool E, bool KE, bool FS>
 void run_force(const DevSim& s, cudaStream_t st) {
     if (s.precision == BBMD_PREC_FP64) {
@@ -2053,7 +1992,6 @@ void run_force(const DevSim& s, cudaStream_t st) {
     } else {
         size_t bytes = kStageBuffers * (size_t)(s.smax + 1) * sizeof(float4);
         k_force<MODE, KE, FS><<<s.grid_cell, kBW * 32, bytes, st>>>(s);
-        if (E) k_force64<MODE, k64Energy, false, FS><<<s.grid_cell, kBW * 32, smem64(s.smax), st>>>(s);
     }
 }
 
@@ -2082,10 +2020,10 @@ void run_force_mode(const DevSim& s, cudaStream_t st, bool energy, bool ke, bool
     else run_force_fs<MODE, false>(s, st, energy, ke);
 }
 
-template <int MODE>
-void run_energy_sums(const DevSim& s, cudaStream_t st, bool fs) {
-    if (fs) k_force64<MODE, k64Sums, false, true><<<s.grid_cell, kBW * 32, smem64(s.smax), st>>>(s);
-    else k_force64<MODE, k64Sums, false, false><<<s.grid_cell, kBW * 32, smem64(s.smax), st>>>(s);
+template <int MODE, int WHAT>
+void run_energies(const DevSim& s, cudaStream_t st, bool fs) {
+    if (fs) k_force64<MODE, WHAT, false, true><<<s.grid_sums, kBW * 32, smem64(s.smax), st>>>(s);
+    else k_force64<MODE, WHAT, false, false><<<s.grid_sums, kBW * 32, smem64(s.smax), st>>>(s);
 }
 
 template <int MODE, bool FS>
@@ -2156,11 +2094,28 @@ void launch_force(const DevSim& s, cudaStream_t st, bool energy, bool ke) {
     run_force_mode<1>(s, st, energy, ke, fs);
 }
 
-// Energy and virial partials of the current positions alone, both precisions.
-void launch_energy_sums(const DevSim& s, cudaStream_t st) {
+// FP64 energies of the current positions from exact integer positions (FP32 coordinates would
+// limit u_i to about 1e-4), either precision; the forces are left alone.  each: per-particle
+// energies; else the energy and virial sums alone (partials of grid_sums CTAs, either way).
+void launch_energies(const DevSim& s, cudaStream_t st, bool each) {
     const bool fs = s.pt.shift == BBMD_SHIFT_FORCE;
-    if (s.nbr_mode == BBMD_NBR_VERLET) run_energy_sums<0>(s, st, fs);
-    run_energy_sums<1>(s, st, fs);
+    if (s.nbr_mode == BBMD_NBR_VERLET) {
+        if (each) run_energies<0, k64Energy>(s, st, fs);
+        else run_energies<0, k64Sums>(s, st, fs);
+    }
+    if (each) run_energies<1, k64Energy>(s, st, fs);
+    else run_energies<1, k64Sums>(s, st, fs);
+}
+
+int energies_blocks_per_sm(const DevSim& s) {
+    int nb = 0;
+    if (s.nbr_mode == BBMD_NBR_VERLET)
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_force64<0, k64Sums, false, false>, kBW * 32,
+                                                      smem64(s.smax));
+    else
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_force64<1, k64Sums, false, false>, kBW * 32,
+                                                      smem64(s.smax));
+    return nb > 0 ? nb : 1;
 }
 
 void launch_force_many(const ManySims& m, int total, bool fp64, bool cell, bool ke, bool fshift,

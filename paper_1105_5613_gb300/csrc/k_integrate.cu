@@ -86,7 +86,10 @@ __global__ void __launch_bounds__(kThreads, 4) k_integrate_many(ManySims m) {
     integrate_body<FP64>(sh, lb, lg);
 }
 
-__global__ void __launch_bounds__(256) k_finalize(DevSim s, int ke) { finalize_body(s, ke); }
+__global__ void __launch_bounds__(256) k_finalize(DevSim s, int ke) {
+    finalize_body(s, ke);
+    if (threadIdx.x == 32) clear_grid_sync(s);  // for the next step's trigger and sort
+}
 
 __global__ void __launch_bounds__(256) k_finalize_many(ManySims m, int ke) {
     __shared__ DevSim sh;
@@ -194,7 +197,7 @@ __global__ void __launch_bounds__(256) k_observe_sums(DevSim s, int energy, doub
     static_assert(sizeof(DevScalars) % 8 == 0 && sizeof(DevScalars) <= (64 - kOutScalars) * 8, "dout");
     __shared__ double r[6];
     sum_partials(s, s.grid_part, 4, r);
-    if (energy) sum_partials(s, s.grid_cell, 2, r + 4, kEnergyPartial);
+    if (energy) sum_partials(s, s.grid_sums, 2, r + 4, kEnergyPartial);
     if (threadIdx.x < 4) out[threadIdx.x] = r[threadIdx.x];
     if (energy && threadIdx.x < 2) out[9 + threadIdx.x] = r[4 + threadIdx.x];
     if (threadIdx.x < sizeof(DevScalars) / 8)

@@ -17,6 +17,8 @@ namespace {
 
 constexpr int kThreads = 256;
 #include "sort_bodies.cuh"
+#include "step_bodies.cuh"
+#include "grid_bodies.cuh"
 
 BBMD_ONE_AND_MANY(kThreads, k_zero, zero_body)
 BBMD_ONE_AND_MANY(kThreads, k_bin, bin_body)
@@ -28,7 +30,32 @@ BBMD_ONE_AND_MANY(kThreads, k_cellsort, cellsort_body)
 BBMD_ONE_AND_MANY(kThreads, k_gather, gather_body)
 BBMD_ONE_AND_MANY(kThreads, k_copyback, copyback_body)
 
+// Rebuild trigger and sort chain in one cooperative launch, behind the integrate kernel: 11
+// launches of a captured step become one, which returns at once in a step in which no
+// displacement came near the threshold.  (The four-CTA bound: the phases are bound by memory.)
+__global__ void __launch_bounds__(kThreads, 4) k_trigger_sort(DevSim s) {
+    unsigned gen = 0;
+    bool due;
+    if (!grid_trigger(s, gen, due)) return;
+    if (due) grid_sort(s, gen);
+}
+
 }  // namespace
+
+int trigger_sort_ctas(const DevSim& s, int nsm) {
+    int nb = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_trigger_sort, kThreads, 0) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    return s.grid_part < nb * nsm ? s.grid_part : nb * nsm;
+}
+
+cudaError_t launch_trigger_sort(const DevSim& s, int grid, cudaStream_t st) {
+    DevSim a = s;
+    void* params[] = {&a};
+    return cudaLaunchCooperativeKernel((const void*)k_trigger_sort, grid, kThreads, params, 0, st);
+}
 
 int scan_grid(const DevSim& s) {
     const int nchunks = scan_chunks(s);

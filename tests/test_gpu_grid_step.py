@@ -49,6 +49,23 @@ def test_step_equals_phase_launches(ncell, shape, thermo, shift, mode):
     b.close()
 
 
+@pytest.mark.parametrize("ncell,shape,kw", [(36, 1, {}), (36, 4, {"mode": 1}),
+                                            (10, 2, {"precision": bbmd.PREC_FP64}),
+                                            (14, 8, {"precision": bbmd.PREC_FP64, "mode": 1})])
+def test_captured_step_equals_phase_launches(ncell, shape, kw):
+    # past one wave of blocks, and the FP64 form: one launch per phase, trigger and sort chain
+    # as one
+    a, b = make(ncell, shape, **kw), make(ncell, shape, **kw)
+    a.step(24, 0.005, (bbmd.THERMO_NH, 2.0, 1.5, 0.5))
+    b.step_profiled(24, 0.005, (bbmd.THERMO_NH, 2.0, 1.5, 0.5))
+    for x, y in zip(a.get_state(), b.get_state()):
+        assert np.array_equal(x, y)
+    oa, ob = a.observe(0), b.observe(0)
+    assert oa["n_rebuilds"] == ob["n_rebuilds"] > 1 and oa["xi"] == ob["xi"]
+    a.close()
+    b.close()
+
+
 def test_cut_lists_fall_back_and_grow():
     # lists that hold the lattice but not the liquid: forces come from the stencil until the
     # next synchronising call grows them
