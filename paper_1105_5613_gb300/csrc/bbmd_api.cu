@@ -42,6 +42,7 @@ struct bbmd_sim {
     std::vector<int> shapes;         // block shapes that fit (candidates of the autotuner)
     int sums_shape = 0;              // block shape of the FP64 energy passes
     int grid_shape = -1, grid_ctas = 0;  // one-launch step: block shape it was sized for, CTAs
+    bool grid_wide = false;          // ... and whether with eight warps a CTA (shape 1)
     float shape_ms[4][2] = {};       // autotuner: per kShapes entry, force and list-build ms
 };
 
@@ -519,6 +520,13 @@ int grid_step_grid(bbmd_sim* sim, bool* one_wave) {
     if (sim->d.precision != BBMD_PREC_MIXED) return 0;
     if (sim->grid_shape != sim->d.block_z) {
         sim->grid_ctas = cooperative(sim) ? grid_step_ctas(sim->d, sim->nsm) : 0;
+        // eight warps a block of four cells where a block has an SM to itself (forces are then
+        // one round of chunks, the list build one of cells): 864 particles 38 -> 34 us a step,
+        // 4000 41 -> 38, 8000 43 -> 39; two such CTAs on an SM gain nothing (steepest descent
+        // at 32 000 28 -> 31)
+        sim->grid_wide = sim->grid_ctas > 0 && sim->d.block_z == 1 && sim->d.nblocks <= sim->nsm &&
+                         z1w::grid_step_ctas(sim->d, sim->nsm) >= sim->d.nblocks;
+        if (sim->grid_wide) sim->grid_ctas = z1w::grid_step_ctas(sim->d, sim->nsm);
         sim->grid_shape = sim->d.block_z;
     }
     *one_wave = sim->grid_ctas >= sim->d.nblocks;
@@ -845,7 +853,7 @@ bbmd_status bbmd_step(bbmd_sim* sim, int64_t nsteps, double dt, const bbmd_therm
         LAUNCHED("begin");
         for (int64_t k = 0; k < nsteps; k += kGridSteps) {
             if (k > 0) launch_clear_grid_sync(sim->d, sim->st);
-            CK(launch_grid_step(sim->d, grid, (int)std::min(kGridSteps, nsteps - k), nh != 0, sim->st));
+            CK(launch_grid_step(sim->d, grid, sim->grid_wide, (int)std::min(kGridSteps, nsteps - k), nh != 0, sim->st));
         }
         return BBMD_OK;
     }
@@ -981,7 +989,7 @@ bbmd_status bbmd_minimize(bbmd_sim* sim, int64_t nsteps, double hmax, double dma
         int64_t k = 0;
         do {
             launch_clear_grid_sync(sim->d, sim->st);
-            CK(launch_grid_relax(sim->d, grid, (int)std::min(kGridSteps, nsteps - k), hmax, dmax, sim->st));
+            CK(launch_grid_relax(sim->d, grid, sim->grid_wide, (int)std::min(kGridSteps, nsteps - k), hmax, dmax, sim->st));
             k += kGridSteps;
         } while (k < nsteps);
         LAUNCHED("minimize");

@@ -307,6 +307,14 @@ BBMD_SHAPE_API(z2)
 BBMD_SHAPE_API(z4)
 BBMD_SHAPE_API(z8)
 #undef BBMD_SHAPE_API
+// The one-launch kernels of shape 1 with eight warps a CTA (k_force.cu, BBMD_WIDE)
+namespace z1w {
+bool prepare_force_kernels();
+int grid_step_ctas(const DevSim& s, int nsm);
+cudaError_t launch_grid_step(const DevSim& s, int grid, int nsteps, bool ke, cudaStream_t st);
+cudaError_t launch_grid_relax(const DevSim& s, int grid, int nsteps, double hmax, double dmax,
+                              cudaStream_t st);
+}  // namespace z1w
 
 // Block shape of the persistent batch step (k_force.cu compiled for it holds the kernel).
 #ifndef BBMD_PERSIST_Z
@@ -352,7 +360,7 @@ cudaError_t launch_persistent_step(const PersistentStep& a, int grid, int smax_m
     }
 inline bool prepare_force_kernels() {
     return z1::prepare_force_kernels() && z2::prepare_force_kernels() &&
-           z4::prepare_force_kernels() && z8::prepare_force_kernels();
+           z4::prepare_force_kernels() && z8::prepare_force_kernels() && z1w::prepare_force_kernels();
 }
 inline int force_blocks_per_sm(const DevSim& s) { BBMD_SHAPE_DISPATCH(s.block_z, force_blocks_per_sm(s)) }
 inline int list_blocks_per_sm(const DevSim& s) { BBMD_SHAPE_DISPATCH(s.block_z, list_blocks_per_sm(s)) }
@@ -368,11 +376,14 @@ inline int energies_blocks_per_sm(const DevSim& s) {
 inline int grid_step_ctas(const DevSim& s, int nsm) {
     BBMD_SHAPE_DISPATCH(s.block_z, grid_step_ctas(s, nsm))
 }
-inline cudaError_t launch_grid_step(const DevSim& s, int grid, int nsteps, bool ke, cudaStream_t st) {
+inline cudaError_t launch_grid_step(const DevSim& s, int grid, bool wide, int nsteps, bool ke,
+                                    cudaStream_t st) {
+    if (wide) return z1w::launch_grid_step(s, grid, nsteps, ke, st);
     BBMD_SHAPE_DISPATCH(s.block_z, launch_grid_step(s, grid, nsteps, ke, st))
 }
-inline cudaError_t launch_grid_relax(const DevSim& s, int grid, int nsteps, double hmax, double dmax,
-                                     cudaStream_t st) {
+inline cudaError_t launch_grid_relax(const DevSim& s, int grid, bool wide, int nsteps, double hmax,
+                                     double dmax, cudaStream_t st) {
+    if (wide) return z1w::launch_grid_relax(s, grid, nsteps, hmax, dmax, st);
     BBMD_SHAPE_DISPATCH(s.block_z, launch_grid_relax(s, grid, nsteps, hmax, dmax, st))
 }
 inline void launch_list_build(const DevSim& s, cudaStream_t st) {

@@ -51,8 +51,13 @@
 #else
 #error "BBMD_BLOCK_Z must be 1, 2, 4 or 8"
 #endif
+// BBMD_WIDE (with shape 1): only the one-launch kernels, with eight warps a CTA, in namespace
+// z1w -- for systems so small that a block has an SM to itself
+#ifndef BBMD_WIDE
+#define BBMD_WIDE 0
+#endif
 #ifndef BBMD_BLOCK_WARPS
-#define BBMD_BLOCK_WARPS BBMD_SHAPE_WARPS
+#define BBMD_BLOCK_WARPS (BBMD_WIDE ? 8 : BBMD_SHAPE_WARPS)
 #endif
 #ifndef BBMD_FORCE_MIN_BLOCKS
 #define BBMD_FORCE_MIN_BLOCKS BBMD_SHAPE_FORCE_MIN
@@ -69,7 +74,11 @@
 #define BBMD_CAT(a, b) BBMD_CAT2(a, b)
 
 namespace bbmd {
+#if BBMD_WIDE
+namespace z1w {
+#else
 namespace BBMD_CAT(z, BBMD_BLOCK_Z) {
+#endif
 
 namespace {
 
@@ -1183,12 +1192,16 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
         const int par = blk_it & 1;
         if (threadIdx.x == 0) ss.next_cell[par ^ 1] = 0;  // for the next block
         ++blk_it;
-        for (int cw = take_cell(ss, par, lane); cw < kCells; cw = take_cell(ss, par, lane)) {
-            const WarpCell wc = warp_cell(s, bp, cw);
+        // (a cell's first 32 particles are an item, the others another: a warp that had both
+        // would be the last of its block)
+        for (int item = take_cell(ss, par, lane); item < 2 * kCells; item = take_cell(ss, par, lane)) {
+            const int first = item < kCells ? 1 : 0;
+            const WarpCell wc = warp_cell(s, bp, first ? item : item - kCells);
             const int i0 = wc.valid ? Rc.start[wc.rq] : 0;
-            const int cnt = wc.valid ? staged_count(Rc, wc.rq) : 0;
+            const int all = wc.valid ? staged_count(Rc, wc.rq) : 0;
+            const int cnt = first ? min(all, 32) : all;
             const int self0 = Rc.off[wc.rq];
-            for (int ch = 0; ch * 32 < cnt; ++ch) {
+            for (int ch = 1 - first; ch * 32 < cnt; ++ch) {
                 const int li = ch * 32 + lane;
                 const bool act = li < cnt;
                 const int64_t gi = (int64_t)i0 + li;
@@ -1373,15 +1386,15 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
 // the phases are kept apart by a grid-wide barrier (about 1.3 us) only where one is needed:
 // two in a step in which nothing came near the rebuild trigger, two more for the trigger,
 // seven more for a rebuild.  Where it is used and what it measured: grid_step_grid
-// (bbmd_api.cu).  At 4000 particles (2 x 2 x 1 blocks, one per SM) a step's 41 us are forces 14
-// (two rounds of chunks on four warps), barriers 6, finalize 6, integrate 2, and 0.2 rebuilds
-// of 70 (its list build 45).
+// (bbmd_api.cu).  At 4000 particles (2 x 2 x 1 blocks, one per SM, four warps) a step's 41 us
+// were forces 14 (two rounds of chunks), barriers 6, finalize 6, integrate 2, and 0.2 rebuilds
+// of 70 (its list build 45, two rounds for a cell of more than 32).
 #include "sort_bodies.cuh"
 #include "step_bodies.cuh"
 #include "grid_bodies.cuh"
 
 #ifndef BBMD_GRID_MIN_BLOCKS
-#define BBMD_GRID_MIN_BLOCKS (BBMD_BLOCK_Z == 1 ? 4 : 2)
+#define BBMD_GRID_MIN_BLOCKS (BBMD_BLOCK_Z == 1 && !BBMD_WIDE ? 4 : 2)
 #endif
 
 // The rebuild after its flag is up and the cell counts are zero: sort chain and list build.
@@ -1914,6 +1927,7 @@ __device__ __forceinline__ void force64_body(const DevSim& s, int lb, int lg) {
     }
 }
 
+#if !BBMD_WIDE
 // ------------------------------------------------------------------ kernels ----
 // Each body runs for one system (DevSim by value) or, in the _many form, for the replica of
 // a batch that owns the CTA.
@@ -1959,6 +1973,8 @@ __global__ void __launch_bounds__(kBW * 32) k_force64_many(ManySims m) {
     force64_body<MODE, k64Force, KE, FSHIFT>(sh, lb, lg);
 }
 
+#endif  // !BBMD_WIDE
+
 // Opt every kernel with dynamic shared memory into the largest size the device allows
 // next to the kernel's static shared memory (done at create, outside any stream capture);
 // each launch then requests only what it needs.
@@ -1980,6 +1996,7 @@ void set_smem(K kernel) {
         g_smem_ok = false;
 }
 
+#if !BBMD_WIDE
 // Dynamic shared memory of the FP64 kernels: upper and lower words of every staged record.
 static size_t smem64(int smax) { return (size_t)(smax + 1) * 32; }
 
@@ -2047,8 +2064,27 @@ void prep_mode() {
     prep_mode_fs<MODE, true>();
 }
 
+#endif  // !BBMD_WIDE
+
 }  // namespace
 
+// Attributes of the one-launch kernels.
+static void prep_grid() {
+    set_smem(k_step_grid<false, false>);
+    set_smem(k_step_grid<true, false>);
+    set_smem(k_step_grid<false, true>);
+    set_smem(k_step_grid<true, true>);
+    set_smem(k_relax_grid<false>);
+    set_smem(k_relax_grid<true>);
+}
+
+#if BBMD_WIDE
+bool prepare_force_kernels() {
+    g_smem_ok = true;
+    prep_grid();
+    return g_smem_ok;
+}
+#else
 int block_threads() { return kBW * 32; }
 
 bool prepare_force_kernels() {
@@ -2057,12 +2093,7 @@ bool prepare_force_kernels() {
     prep_mode<1>();
     set_smem(k_list_build);
     set_smem(k_list_build_many);
-    set_smem(k_step_grid<false, false>);
-    set_smem(k_step_grid<true, false>);
-    set_smem(k_step_grid<false, true>);
-    set_smem(k_step_grid<true, true>);
-    set_smem(k_relax_grid<false>);
-    set_smem(k_relax_grid<true>);
+    prep_grid();
     return g_smem_ok;
 }
 
@@ -2161,6 +2192,8 @@ void launch_list_build(const DevSim& s, cudaStream_t st) {
     size_t bytes = kStageBuffers * (size_t)(s.smax + 1) * sizeof(float4);
     k_list_build<<<s.grid_list, kBW * 32, bytes, st>>>(s);
 }
+
+#endif  // BBMD_WIDE
 
 // CTAs of the one-launch step: enough for every block and for 256 particles a CTA, at most
 // what is resident at once.
