@@ -445,7 +445,10 @@ bbmd_status autotune_shape(bbmd_sim* sim, float rebuild_rate = 0.25f) {
             continue;
         }
         const float cost = tf + (verlet ? rebuild_rate * tl : 0.f);
-        if (best < 0 || cost < best_cost) {
+        // (a larger block has to be 2 % cheaper: shapes within the timings' noise of each other
+        // would otherwise take turns from one creation to the next, and with them the
+        // summation order)
+        if (best < 0 || cost < 0.98f * best_cost) {
             best = bz;
             best_cost = cost;
         }
@@ -716,10 +719,9 @@ bbmd_status bbmd_create(const bbmd_params* params, int64_t n, const double box[3
     if (params->precision == BBMD_PREC_FP64) D.Fd = (double*)A(3 * np * 8);
     D.ud = (double*)A(np * 8);
     D.key = (int32_t*)A(np * 4);
+    D.rank = (int32_t*)A(np * 4);
     D.perm = (int32_t*)A(np * 4);
-    D.perm_tmp = (int32_t*)A(np * 4);
     D.count = (int32_t*)A((ncell + 1) * 4);
-    D.cursor = (int32_t*)A((ncell + 1) * 4);
     D.cell_start = (int32_t*)A((ncell + 1) * 4);
     D.scan_part = (int32_t*)A(((ncell + 8191) / 8192 + 1) * 4);
     if (params->nbr_mode == BBMD_NBR_VERLET) D.list = (uint16_t*)A((size_t)D.lcap8 * np * 16);

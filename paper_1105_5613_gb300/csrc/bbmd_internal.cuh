@@ -118,7 +118,7 @@ struct alignas(16) DevSim {
     float4 *rel, *relb, *F;
     double* Fd;
     double* ud;              // per-particle FP64 energy (energy passes)
-    int32_t *key, *cell_start, *count, *cursor, *perm, *perm_tmp, *scan_part;
+    int32_t *key, *cell_start, *count, *rank, *perm, *scan_part;
     uint16_t* list;
     uint16_t* rows;          // per particle: rows (8 entries each) of its Verlet list
     double* partials;        // [kMaxPartials][4]
@@ -326,8 +326,8 @@ constexpr int kPersistZ = BBMD_PERSIST_Z;
 // index, CTA count) come from one queue, step-major and phase-major within a step; an
 // item starts once its replica's previous non-empty phase has finished.
 enum {
-    kPhIntegrate = 0, kPhCelltop, kPhCheck, kPhZero, kPhBin, kPhScan, kPhScatter, kPhCellsort,
-    kPhGather, kPhCopyback, kPhList, kPhForce, kPhFinalize, kPhases
+    kPhIntegrate = 0, kPhCelltop, kPhCheck, kPhZero, kPhBin, kPhScan, kPhScatter, kPhSortGather,
+    kPhCopyback, kPhList, kPhForce, kPhFinalize, kPhases
 };
 struct PersistentStep {
     const DevSim* sims;       // nrep replica systems (device copies)

@@ -94,9 +94,7 @@ __device__ __forceinline__ bool grid_sort(const DevSim& s, unsigned& gen) {
     if (!grid_barrier(s, gen)) return false;
     scatter_body(s, lb, lg);
     if (!grid_barrier(s, gen)) return false;
-    cellsort_body(s, lb, lg);
-    if (!grid_barrier(s, gen)) return false;
-    gather_body(s, lb, lg);
+    sortgather_body(s, lb, lg);
     if (!grid_barrier(s, gen)) return false;
     copyback_body(s, lb, lg);
     return true;

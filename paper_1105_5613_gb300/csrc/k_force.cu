@@ -1467,7 +1467,7 @@ __global__ void __launch_bounds__(kBW * 32, BBMD_GRID_MIN_BLOCKS)
 
 // ------------------------------------------------------- persistent batch step ----
 // One cooperative launch advances every replica of a batch by many steps.  The step of
-// each replica is a chain of phases (integrate, the two trigger passes, the seven sort
+// each replica is a chain of phases (integrate, the two trigger passes, the six sort
 // passes, the list build, forces, finalize); each phase of each replica is cut into work
 // items with the same (CTA index, CTA count) as the kernels launched for one system, so a
 // replica advances bit for bit as it would alone.  The items of all replicas are handed
@@ -1495,8 +1495,7 @@ __device__ __forceinline__ void run_phase(int phase, const DevSim& s, int lb, in
         case kPhBin: bin_body(s, lb, lg); break;
         case kPhScan: scan_cta_body(s, lb, lg); break;
         case kPhScatter: scatter_body(s, lb, lg); break;
-        case kPhCellsort: cellsort_body(s, lb, lg); break;
-        case kPhGather: gather_body(s, lb, lg); break;
+        case kPhSortGather: sortgather_body(s, lb, lg); break;
         case kPhCopyback: copyback_body(s, lb, lg); break;
         case kPhList: list_build_body<true>(s, lb, lg); break;
         case kPhForce:

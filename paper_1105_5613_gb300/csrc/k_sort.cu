@@ -6,9 +6,10 @@
 // use fixed grid-stride grids (a few blocks per SM) so that a skipped rebuild costs only
 // a handful of empty launches.
 //
-// Chain: zero counts -> bin (key + histogram) -> exclusive scan -> scatter -> order each
-// cell by id (canonical order: the sorted state depends only on positions and ids) ->
-// gather into the alternate buffers (+ frame-relative FP32 copies) -> copy back.
+// Chain: zero counts -> bin (key + histogram, and each particle's place in its cell) ->
+// exclusive scan -> scatter -> per cell, order by species and id (canonical order: the sorted
+// state depends only on positions, species and ids) and gather into the alternate buffers (+
+// frame-relative FP32 copies) -> copy back.
 #include "bbmd_internal.cuh"
 
 namespace bbmd {
@@ -26,11 +27,10 @@ BBMD_ONE_AND_MANY(kScanThreads, k_scan_reduce, scan_reduce_body)
 BBMD_ONE_AND_MANY(kScanThreads, k_scan_top, scan_top_body)
 BBMD_ONE_AND_MANY(kScanThreads, k_scan_down, scan_down_body)
 BBMD_ONE_AND_MANY(kThreads, k_scatter, scatter_body)
-BBMD_ONE_AND_MANY(kThreads, k_cellsort, cellsort_body)
-BBMD_ONE_AND_MANY(kThreads, k_gather, gather_body)
+BBMD_ONE_AND_MANY(kThreads, k_sortgather, sortgather_body)
 BBMD_ONE_AND_MANY(kThreads, k_copyback, copyback_body)
 
-// Rebuild trigger and sort chain in one cooperative launch, behind the integrate kernel: 11
+// Rebuild trigger and sort chain in one cooperative launch, behind the integrate kernel: 10
 // launches of a captured step become one, which returns at once in a step in which no
 // displacement came near the threshold.  (The four-CTA bound: the phases are bound by memory.)
 __global__ void __launch_bounds__(kThreads, 4) k_trigger_sort(DevSim s) {
@@ -70,8 +70,7 @@ void launch_rebuild_chain(const DevSim& s, cudaStream_t st) {
     k_scan_top<<<1, kScanThreads, 0, st>>>(s);
     k_scan_down<<<gscan, kScanThreads, 0, st>>>(s);
     k_scatter<<<s.grid_part, kThreads, 0, st>>>(s);
-    k_cellsort<<<s.grid_part, kThreads, 0, st>>>(s);
-    k_gather<<<s.grid_part, kThreads, 0, st>>>(s);
+    k_sortgather<<<s.grid_part, kThreads, 0, st>>>(s);
     k_copyback<<<s.grid_part, kThreads, 0, st>>>(s);
 }
 
@@ -83,8 +82,7 @@ void launch_rebuild_chain_many(const ManySims& part, const ManySims& scan, const
     k_scan_top_many<<<nrep, kScanThreads, 0, st>>>(one);
     k_scan_down_many<<<total_scan, kScanThreads, 0, st>>>(scan);
     k_scatter_many<<<total_part, kThreads, 0, st>>>(part);
-    k_cellsort_many<<<total_part, kThreads, 0, st>>>(part);
-    k_gather_many<<<total_part, kThreads, 0, st>>>(part);
+    k_sortgather_many<<<total_part, kThreads, 0, st>>>(part);
     k_copyback_many<<<total_part, kThreads, 0, st>>>(part);
 }
 

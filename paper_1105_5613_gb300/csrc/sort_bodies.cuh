@@ -26,7 +26,6 @@ __device__ __forceinline__ void zero_counts(const DevSim& s, int lb, int lg) {
     for (int64_t c = lb * (int64_t)blockDim.x + threadIdx.x; c <= s.ncell;
          c += (int64_t)lg * blockDim.x) {
         s.count[c] = 0;
-        s.cursor[c] = 0;
     }
 }
 
@@ -45,7 +44,7 @@ __device__ __forceinline__ void bin_body(const DevSim& s, int lb, int lg) {
         int az = cell_axis((long long)s.x[2 * s.npad + i], s.D[2], s.nc[2]);
         int c = (az * s.nc[1] + ay) * s.nc[0] + ax;
         s.key[i] = c;
-        atomicAdd(&s.count[c], 1);
+        s.rank[i] = atomicAdd(&s.count[c], 1);  // its place among the cell's (in any order)
     }
 }
 
@@ -190,9 +189,7 @@ __device__ __forceinline__ void scatter_body(const DevSim& s, int lb, int lg) {
     if (!s.sc->rebuild) return;
     for (int64_t i = lb * (int64_t)blockDim.x + threadIdx.x; i < s.n;
          i += (int64_t)lg * blockDim.x) {
-        int c = s.key[i];
-        int slot = s.cell_start[c] + atomicAdd(&s.cursor[c], 1);
-        s.perm_tmp[slot] = (int32_t)i;
+        s.perm[s.cell_start[s.key[i]] + s.rank[i]] = (int32_t)i;
     }
 }
 
@@ -203,69 +200,69 @@ __device__ __forceinline__ long long cell_key(const DevSim& s, int p) {
     return ((long long)s.sp[p] << 32) | (long long)(unsigned)s.id[p];
 }
 
-__device__ __forceinline__ void cellsort_body(const DevSim& s, int lb, int lg) {
+// Particle p of cell c (cell coordinates a3) to slot k of the alternate buffers, with its
+// frame-relative FP32 copies.
+__device__ __forceinline__ void move_particle(const DevSim& s, int64_t p, int64_t k, int c,
+                                              const int a3[3], long long key) {
+    // all loads of the particle first (the stores could alias them for the compiler)
+    uint64_t xv[3];
+    int64_t vv[3];
+    int32_t iv[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        xv[d] = s.x[d * s.npad + p];
+        vv[d] = s.v[d * s.npad + p];
+        iv[d] = s.img[d * s.npad + p];
+    }
+    float r[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        s.x2[d * s.npad + k] = xv[d];
+        s.v2[d * s.npad + k] = vv[d];
+        s.img2[d * s.npad + k] = iv[d];
+        const long long rel = (long long)xv[d] - frame_axis(a3[d], s.D[d]);
+        r[d] = i64_to_f32(rel) * s.sx;
+    }
+    const int spc = (int)(key >> 32);
+    s.id2[k] = (int32_t)key;
+    s.sp2[k] = (uint8_t)spc;
+    s.relb[k] = make_float4(r[0], r[1], r[2], __int_as_float((c << 1) | spc));
+    s.rel[k] = make_float4(r[0], r[1], r[2], (float)spc);
+}
+
+// A warp per cell: its particles go, in canonical order, to the alternate buffers.  (One pass
+// for what was two, ordering and gathering: the particles' ids and species are read once and
+// no ordered permutation is written.  With the places in the cells taken from the binning's
+// counts instead of a second round of atomics, the chain of 16.4 M particles takes 1.42 ms
+// for 1.73.)
+__device__ __forceinline__ void sortgather_body(const DevSim& s, int lb, int lg) {
     if (!s.sc->rebuild) return;
     const int lane = threadIdx.x & 31;
     const int64_t nwarps = (int64_t)lg * (blockDim.x >> 5);
     for (int64_t c = (lb * (int64_t)blockDim.x + threadIdx.x) >> 5; c < s.ncell;
          c += nwarps) {
-        int start = s.cell_start[c];
-        int cnt = s.cell_start[c + 1] - start;
+        const int start = s.cell_start[c];
+        const int cnt = s.cell_start[c + 1] - start;
+        int a3[3];
+        cell_coords((int)c, s.nc, a3[0], a3[1], a3[2]);
         if (cnt <= 32) {
-            int pe = lane < cnt ? s.perm_tmp[start + lane] : 0;
-            long long key = lane < cnt ? cell_key(s, pe) : 0x7fffffffffffffffll;
+            const int pe = lane < cnt ? s.perm[start + lane] : 0;
+            const long long key = lane < cnt ? cell_key(s, pe) : 0x7fffffffffffffffll;
             int rank = 0;
             for (int f = 0; f < cnt; ++f) {
-                long long other = __shfl_sync(0xffffffffu, key, f);
+                const long long other = __shfl_sync(0xffffffffu, key, f);
                 rank += other < key;
             }
-            if (lane < cnt) s.perm[start + rank] = pe;
+            if (lane < cnt) move_particle(s, pe, start + rank, (int)c, a3, key);
         } else {
             for (int e = lane; e < cnt; e += 32) {
-                int pe = s.perm_tmp[start + e];
-                long long key = cell_key(s, pe);
+                const int pe = s.perm[start + e];
+                const long long key = cell_key(s, pe);
                 int rank = 0;
-                for (int f = 0; f < cnt; ++f) rank += cell_key(s, s.perm_tmp[start + f]) < key;
-                s.perm[start + rank] = pe;
+                for (int f = 0; f < cnt; ++f) rank += cell_key(s, s.perm[start + f]) < key;
+                move_particle(s, pe, start + rank, (int)c, a3, key);
             }
         }
-    }
-}
-
-__device__ __forceinline__ void gather_body(const DevSim& s, int lb, int lg) {
-    if (!s.sc->rebuild) return;
-    for (int64_t k = lb * (int64_t)blockDim.x + threadIdx.x; k < s.n;
-         k += (int64_t)lg * blockDim.x) {
-        int64_t o = s.perm[k];
-        // all loads of the particle first (the stores could alias them for the compiler)
-        const int c = s.key[o];
-        uint64_t xv[3];
-        int64_t vv[3];
-        int32_t iv[3];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            xv[d] = s.x[d * s.npad + o];
-            vv[d] = s.v[d * s.npad + o];
-            iv[d] = s.img[d * s.npad + o];
-        }
-        const int32_t idv = s.id[o];
-        const uint8_t spc = s.sp[o];
-        int ax, ay, az;
-        cell_coords(c, s.nc, ax, ay, az);
-        int a3[3] = {ax, ay, az};
-        float r[3];
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            s.x2[d * s.npad + k] = xv[d];
-            s.v2[d * s.npad + k] = vv[d];
-            s.img2[d * s.npad + k] = iv[d];
-            long long rel = (long long)xv[d] - frame_axis(a3[d], s.D[d]);
-            r[d] = i64_to_f32(rel) * s.sx;
-        }
-        s.id2[k] = idv;
-        s.sp2[k] = spc;
-        s.relb[k] = make_float4(r[0], r[1], r[2], __int_as_float((c << 1) | spc));
-        s.rel[k] = make_float4(r[0], r[1], r[2], (float)spc);
     }
 }
 
