@@ -723,7 +723,8 @@ bbmd_status bbmd_create(const bbmd_params* params, int64_t n, const double box[3
     D.perm = (int32_t*)A(np * 4);
     D.count = (int32_t*)A((ncell + 1) * 4);
     D.cell_start = (int32_t*)A((ncell + 1) * 4);
-    D.scan_part = (int32_t*)A(((ncell + 8191) / 8192 + 1) * 4);
+    // (chunk sums of either scan: one per 8192 cells, or at most 256)
+    D.scan_part = (int32_t*)A(std::max<int64_t>((ncell + 8191) / 8192 + 1, 256) * 4);
     if (params->nbr_mode == BBMD_NBR_VERLET) D.list = (uint16_t*)A((size_t)D.lcap8 * np * 16);
     D.rows = (uint16_t*)A(np * 2);
     D.partials = (double*)A((size_t)8 * kMaxPartials * 8);

@@ -90,7 +90,17 @@ __device__ __forceinline__ bool grid_sort(const DevSim& s, unsigned& gen) {
     clear_list_flags(s, lb);
     bin_body(s, lb, lg);
     if (!grid_barrier(s, gen)) return false;
-    scan_cta_body(s, lb, lg);
+    // cell starts: one CTA's scan where it holds all cells at once; else every CTA sums its
+    // chunk, and adds the sums of the chunks before to its scan
+    const int per = (int)blockDim.x * kScanItems;
+    const int chunks = (s.ncell + per - 1) / per;
+    if (chunks == 1 || chunks > lg || chunks > kScanParts) {
+        scan_cta_body(s, lb, lg);
+    } else {
+        if (lb < chunks) scan_chunk_sum(s, lb);
+        if (!grid_barrier(s, gen)) return false;
+        if (lb < chunks) scan_chunk_down(s, lb, chunks);
+    }
     if (!grid_barrier(s, gen)) return false;
     scatter_body(s, lb, lg);
     if (!grid_barrier(s, gen)) return false;

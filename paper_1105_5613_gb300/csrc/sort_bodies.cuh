@@ -185,6 +185,55 @@ __device__ __forceinline__ void scan_cta_body(const DevSim& s, int lb, int lg) {
     if (threadIdx.x == 0) s.cell_start[s.ncell] = (int32_t)s.n;
 }
 
+// The same scan in two phases over chunks of kScanItems cells per thread, one CTA each, with a
+// grid-wide barrier between (at most kScanParts chunks): the chunk's sum, then its scan from
+// the sum of the chunks before it.
+constexpr int kScanParts = 256;
+
+__device__ __forceinline__ void scan_chunk_sum(const DevSim& s, int ch) {
+    __shared__ int red[kScanThreads / 32];
+    const int64_t base = ((int64_t)ch * blockDim.x + threadIdx.x) * kScanItems;
+    int acc = 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k)
+        if (base + k < s.ncell) acc += s.count[base + k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += red[k];
+        s.scan_part[ch] = t;
+    }
+}
+
+__device__ __forceinline__ void scan_chunk_down(const DevSim& s, int ch, int chunks) {
+    __shared__ int before, tot;
+    if (threadIdx.x < 32) {
+        int t = 0;
+        for (int k = threadIdx.x; k < ch; k += 32) t += s.scan_part[k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (threadIdx.x == 0) before = t;
+    }
+    const int64_t base = ((int64_t)ch * blockDim.x + threadIdx.x) * kScanItems;
+    int vals[kScanItems];
+    int acc = 0;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        vals[k] = base + k < s.ncell ? s.count[base + k] : 0;
+        acc += vals[k];
+    }
+    int ex = block_scan_excl(acc, tot) + before;  // (it synchronises: `before` is there)
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+        if (base + k < s.ncell) s.cell_start[base + k] = ex;
+        ex += vals[k];
+    }
+    if (ch + 1 == chunks && threadIdx.x == 0) s.cell_start[s.ncell] = (int32_t)s.n;
+}
+
 __device__ __forceinline__ void scatter_body(const DevSim& s, int lb, int lg) {
     if (!s.sc->rebuild) return;
     for (int64_t i = lb * (int64_t)blockDim.x + threadIdx.x; i < s.n;
