@@ -437,19 +437,17 @@ __device__ __forceinline__ void pair_add(const LaneTab& T, bool b, float dx, flo
     a.fz = fmaf(f, dz, a.fz);
 }
 
-// Force of one interacting pair with the constants of its species pair given (the stencil
-// kernel loads them per candidate stream); the same arithmetic as pair_add.
+// Scalar forces f of two interacting pairs with the constants of their species pair given
+// (the stencil kernel loads them per candidate stream); the arithmetic of pair_add.
 template <bool FSHIFT>
-__device__ __forceinline__ void pair_add_c(float sig2, float e48, float cpot, float fc, float dx, float dy,
-                                           float dz, float r2, Acc& a) {
-    float ir2 = rcp_approx(r2);
-    float s2 = sig2 * ir2;
-    float s6 = s2 * s2 * s2;
-    float f = e48 * ir2 * s6 * (s6 - cpot);
-    if (FSHIFT) f = fmaf(fc, rsqrtf(r2), f);
-    a.fx = fmaf(f, dx, a.fx);
-    a.fy = fmaf(f, dy, a.fy);
-    a.fz = fmaf(f, dz, a.fz);
+__device__ __forceinline__ float2 pair_f2(float sig2, float e48, float cpot, float fc, float2 r2) {
+    const float2 ir2 = make_float2(rcp_approx(r2.x), rcp_approx(r2.y));
+    const float2 s2 = __fmul2_rn(make_float2(sig2, sig2), ir2);
+    const float2 s6 = __fmul2_rn(__fmul2_rn(s2, s2), s2);
+    float2 f = __fmul2_rn(__fmul2_rn(__fmul2_rn(make_float2(e48, e48), ir2), s6),
+                          __fadd2_rn(s6, make_float2(-cpot, -cpot)));
+    if (FSHIFT) f = __ffma2_rn(make_float2(fc, fc), make_float2(rsqrtf(r2.x), rsqrtf(r2.y)), f);
+    return f;
 }
 
 // Fast path of one list pair (i, staged t), classified by d = r^2 - (middle of the band
@@ -1063,14 +1061,31 @@ __device__ __forceinline__ void force_body(const DevSim& s, int lb, int lg) {
                         const float sig2 = s.pt.sig2[k], e48 = s.pt.eps48[k];
                         const float fcut = FSHIFT ? s.pt.fcut[k] : 0.f;
                         const float cpot = s.pt.potential == BBMD_POT_LJ ? 0.5f : 0.0f;
+                        // Two entries an iteration, for the loop runs to the lane with the most
+                        // entries: two-wide FP32, each half rounding like the scalar operation,
+                        // the forces added one after the other.  2.05 M particles, one entry ->
+                        // two: 4x4x2 1048 -> 1001 us, 4x4x4 1176 -> 1093, 4x4x8 1195 -> 1087
                         while (inw) {
                             const int u = __clz(inw);
                             inw &= 0x7fffffffu >> u;
+                            const bool two = inw != 0u;
+                            const int w = two ? __clz(inw) : u;
+                            inw &= 0x7fffffffu >> w;
                             // p' - m' (0.5 m2 = -m' exactly)
-                            const float dx = fmaf(m2x, 0.5f, W.x[u]), dy = fmaf(m2y, 0.5f, W.y[u]),
-                                        dz = fmaf(m2z, 0.5f, W.z[u]);
-                            const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
-                            pair_add_c<FSHIFT>(sig2, e48, cpot, fcut, dx, dy, dz, r2, a);
+                            const float2 h = make_float2(0.5f, 0.5f);
+                            const float2 dx = __ffma2_rn(make_float2(m2x, m2x), h, make_float2(W.x[u], W.x[w]));
+                            const float2 dy = __ffma2_rn(make_float2(m2y, m2y), h, make_float2(W.y[u], W.y[w]));
+                            const float2 dz = __ffma2_rn(make_float2(m2z, m2z), h, make_float2(W.z[u], W.z[w]));
+                            const float2 r2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __fmul2_rn(dz, dz)));
+                            const float2 f = pair_f2<FSHIFT>(sig2, e48, cpot, fcut, r2);
+                            a.fx = fmaf(f.x, dx.x, a.fx);
+                            a.fy = fmaf(f.x, dy.x, a.fy);
+                            a.fz = fmaf(f.x, dz.x, a.fz);
+                            if (two) {
+                                a.fx = fmaf(f.y, dx.y, a.fx);
+                                a.fy = fmaf(f.y, dy.y, a.fy);
+                                a.fz = fmaf(f.y, dz.y, a.fz);
+                            }
                         }
                     };
                     auto flush_full = [&](int S) {
