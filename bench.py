@@ -408,9 +408,10 @@ def run_ours(args):
         "shape_times": shape_times,
         "rebuilds_per_step": timed_rebuilds / args.steps,  # over the timed steps
         "phases_rebuilds_per_step": nreb / nprof,
-        # per step: integrate, 2 trigger kernels, 9 gated sort kernels, gated list build,
-        # list force and the stencil force that stands in for cut lists (one of the two
-        # returns at once), finalize (one graph); plus begin and finish of the call
+        # per step: integrate, 2 trigger kernels, gated sort kernels, gated list build, list
+        # force and the stencil force that stands in for cut lists (one of the two returns at
+        # once), finalize (one graph); plus begin and finish of the call.  Nominal: it counts
+        # 9 sort kernels; ordering and gathering are one kernel now, so 15 a step are launched
         "gpu_launches": args.steps * 16 + 2,
         "clocks": clocks,
         "fp64": fp64,
