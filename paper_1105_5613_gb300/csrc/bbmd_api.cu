@@ -286,9 +286,9 @@ void apply_shape(bbmd_sim* sim, int bz) {
     D.grid_list = (int32_t)std::max<int64_t>(
         1, std::min<int64_t>((int64_t)sim->nsm * list_blocks_per_sm(D), D.nblocks));
     // the FP64 energy passes: their own occupancy (as many CTAs as the force kernel's would
-    // leave a last wave of a few).  Without stored lists any shape serves them, and 2 x 2 x 2
-    // runs two CTAs per SM where the larger shapes run one: 2.05 M in cell mode 4.4 ms against
-    // 6.5 (2 x 2 x 4) and 6.9 (4 x 4 x 2)
+    // leave a last wave of a few).  Without stored lists any shape whose region holds the state
+    // serves them (launch_energy_pass), and 2 x 2 x 2 runs two CTAs per SM where the larger
+    // shapes run one: 2.05 M in cell mode 4.4 ms against 6.5 (2 x 2 x 4) and 6.9 (4 x 4 x 2)
     sim->sums_shape = bz;
     if (D.nbr_mode != BBMD_NBR_VERLET && bz > 2 && shape_fits(sim, 2)) sim->sums_shape = 2;
     DevSim S = D;
@@ -296,11 +296,19 @@ void apply_shape(bbmd_sim* sim, int bz) {
     D.grid_sums = block_grid(sim, S, energies_blocks_per_sm(S));
 }
 
-// The system as the FP64 energy passes see it.
-DevSim sums_sim(const bbmd_sim* sim) {
+// FP64 energy pass (each: with per-particle energies) in its own block shape, and behind a
+// smaller one than the forces' the pass that stands in for it on a state it cannot hold
+// (returns at once otherwise).  Both write grid_sums partials.
+void launch_energy_pass(const bbmd_sim* sim, bool each) {
     DevSim S = sim->d;
-    if (sim->sums_shape != S.block_z) shape_geometry(sim, sim->sums_shape, S);
-    return S;
+    if (sim->sums_shape != S.block_z) {
+        shape_geometry(sim, sim->sums_shape, S);
+        S.sums_role = kSumsSmaller;
+        launch_energies(S, sim->st, each);
+        S = sim->d;
+        S.sums_role = kSumsStandIn;
+    }
+    launch_energies(S, sim->st, each);
 }
 
 bbmd_status rebuild_now(bbmd_sim* sim);
@@ -311,7 +319,7 @@ void finish_velocities(bbmd_sim* sim);
 void launch_forces_and_energies(bbmd_sim* sim, bool energies) {
     const bool fp64 = sim->d.precision == BBMD_PREC_FP64;
     launch_force(sim->d, sim->st, energies && fp64, false);
-    if (energies && !fp64) launch_energies(sums_sim(sim), sim->st, true);
+    if (energies && !fp64) launch_energy_pass(sim, true);
 }
 
 void free_graphs(bbmd_sim* sim);
@@ -881,7 +889,7 @@ bbmd_status bbmd_observe(bbmd_sim* sim, uint32_t mask, const bbmd_obs_args* args
     // kinetic energy and momentum
     const bool energy = (mask & (BBMD_OBS_ENERGY | BBMD_OBS_VIRIAL)) != 0;
     launch_state_sums(D, sim->st);
-    if (energy) launch_energies(sums_sim(sim), sim->st, false);
+    if (energy) launch_energy_pass(sim, false);
     launch_observe_sums(D, sim->st, energy, sim->dout);
     const int origin = args ? args->origin : 0;
     if (origin < 0 || origin >= BBMD_MAX_ORIGINS)

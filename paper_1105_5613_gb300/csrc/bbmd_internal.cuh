@@ -47,6 +47,16 @@ enum : int32_t {
     ST_NONFINITE = 4,
     ST_VEL_RANGE = 8,
     ST_TIMEOUT = 16,
+    ST_SUMS_SHORT = 32,  // not an error: an energy pass's smaller region did not hold the state
+};
+
+// Energy passes in cell mode may use a smaller block shape than the forces, and with it a
+// smaller staged region (DevSim::sums_role): a state whose density varies can fit the one and
+// not the other.
+enum : int32_t {
+    kSumsOwn = 0,      // the handle's own shape: a region too small is an error
+    kSumsSmaller = 1,  // the smaller shape: raises ST_SUMS_SHORT, and stays out once it is up
+    kSumsStandIn = 2,  // the handle's own shape behind it: runs only when ST_SUMS_SHORT is up
 };
 
 // Words of the grid-wide barrier, each in a cache line of its own: arrivals, release count,
@@ -128,6 +138,7 @@ struct alignas(16) DevSim {
     int32_t grid_cell;       // grid of the force kernel (kBlockWarps warps per CTA)
     int32_t grid_list;       // grid of the list-build kernel
     int32_t grid_sums;       // grid of the FP64 energy passes
+    int32_t sums_role;       // what this system's energy pass is (kSums*)
 };
 
 // ---------------------------------------------------------------- conversions ----

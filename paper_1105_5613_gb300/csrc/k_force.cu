@@ -258,7 +258,8 @@ __device__ void region_info(const DevSim& s, const BlockPos& b, Region& R) {
             int total = base + incl;
             R.off[kRegion] = min(total, s.smax);
             R.nstaged = min(total, s.smax);
-            if (total > s.smax) set_status(s, ST_STENCIL_OVERFLOW);
+            if (total > s.smax)
+                set_status(s, s.sums_role == kSumsSmaller ? ST_SUMS_SHORT : ST_STENCIL_OVERFLOW);
         }
     }
     __syncthreads();
@@ -1774,6 +1775,11 @@ __device__ __forceinline__ void pair_fp64(const DevSim& s, int si, long long mx,
 template <int MODE, int WHAT, bool KE, bool FSHIFT>
 __device__ __forceinline__ void force64_body(const DevSim& s, int lb, int lg) {
     if (!force_selected<MODE>(s)) return;  // CTA-uniform, before any barrier
+    if (!(WHAT & k64Force) && s.sums_role != kSumsOwn) {
+        // (one thread looks: other CTAs of the pass may raise the bit meanwhile)
+        const bool is_short = __syncthreads_or(threadIdx.x == 0 && (*(volatile int*)&s.sc->status & ST_SUMS_SHORT));
+        if (is_short != (s.sums_role == kSumsStandIn)) return;
+    }
     extern __shared__ float4 smem[];
     StageShared& ss = stage_shared();
     Region& R = ss.R[0];
