@@ -27,6 +27,7 @@
 #include <cstddef>
 
 #include "bbmd_internal.cuh"
+#include "stage_loop.cuh"
 
 #ifndef BBMD_BLOCK_Z
 #error "k_force.cu is compiled once per block shape: define BBMD_BLOCK_Z (code 1, 2, 4 or 8)"
@@ -135,6 +136,11 @@ __device__ __forceinline__ void mbar_init(uint64_t* mbar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(mbar)), "r"(count)
                  : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+// (the memory may then be initialised again, or used for something else)
+__device__ __forceinline__ void mbar_inval(uint64_t* mbar) {
+    asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(smem_u32(mbar)) : "memory");
 }
 
 __device__ __forceinline__ void fence_proxy_async_smem() {
@@ -311,38 +317,45 @@ __device__ bool finish_block(const DevSim& s, const Region& R, float4* sm, uint6
 #endif
 constexpr int kStageBuffers = BBMD_STAGE_BUFFERS;
 
-// Blocks of this CTA in order (grid-stride).  With two staging buffers the copies of block
-// i+1 are in flight while block i is computed; with one, each block is staged then
-// computed.  body(pos, R, sm) computes one staged block and must not synchronise the CTA.
+struct StageOps {
+    float4* smem;
+    int stride;  // records of a buffer
+    Region* R;
+    uint64_t* mbar;
+
+    __device__ __forceinline__ void open() {
+        if (threadIdx.x == 0)
+            for (int k = 0; k < kStageBuffers; ++k) mbar_init(&mbar[k], 1);
+        __syncthreads();
+    }
+    __device__ __forceinline__ BlockPos position(const DevSim& s, int64_t blk) { return block_pos(s, blk); }
+    __device__ __forceinline__ void issue(const DevSim& s, const BlockPos& pos, int b) {
+        issue_block(s, pos, R[b], smem + b * stride, &mbar[b]);
+    }
+    __device__ __forceinline__ bool finish(const DevSim& s, int b, uint32_t parity) {
+        return finish_block(s, R[b], smem + b * stride, &mbar[b], parity);
+    }
+    template <class Body>
+    __device__ __forceinline__ void compute(const BlockPos& pos, int b, Body& body) {
+        body(pos, R[b], smem + b * stride, b);
+    }
+    __device__ __forceinline__ void drain(const DevSim& s, int b, uint32_t parity) {
+        mbar_wait_bounded(s, &mbar[b], parity);
+    }
+    __device__ __forceinline__ void sync() { __syncthreads(); }
+    __device__ __forceinline__ void close() {
+        if (threadIdx.x == 0)
+            for (int k = 0; k < kStageBuffers; ++k) mbar_inval(&mbar[k]);
+    }
+};
+
+// Blocks of this CTA in order (grid-stride): body(pos, R, sm, b) computes one staged block,
+// from buffer b, and must not synchronise the CTA.  False (on every thread) if a staging wait
+// gave up (see staged_blocks).
 template <class Body>
-__device__ void for_each_block(const DevSim& s, int lb, int lg, float4* smem, int buf_stride, Region* R,
-                               uint64_t* mbar, Body body) {
-    int64_t blk = lb;
-    if (kStageBuffers == 1) {
-        for (int it = 0; blk < s.nblocks; ++it, blk += lg) {
-            const BlockPos bp = block_pos(s, blk);
-            issue_block(s, bp, R[0], smem, &mbar[0]);
-            if (!finish_block(s, R[0], smem, &mbar[0], (uint32_t)(it & 1))) return;
-            body(bp, R[0], smem);
-            __syncthreads();
-        }
-        return;
-    }
-    float4* buf[2] = {smem, smem + buf_stride};
-    if (blk < s.nblocks) issue_block(s, block_pos(s, blk), R[0], buf[0], &mbar[0]);
-    for (int it = 0; blk < s.nblocks; ++it, blk += lg) {
-        const int cur = it & 1;
-        const int64_t nb = blk + lg;
-        if (nb < s.nblocks) issue_block(s, block_pos(s, nb), R[cur ^ 1], buf[cur ^ 1], &mbar[cur ^ 1]);
-        if (!finish_block(s, R[cur], buf[cur], &mbar[cur], (uint32_t)((it >> 1) & 1))) {
-            // let the copies already issued for the next block land before leaving
-            if (nb < s.nblocks)
-                mbar_wait_bounded(s, &mbar[cur ^ 1], (uint32_t)(((it + 1) >> 1) & 1));
-            return;
-        }
-        body(block_pos(s, blk), R[cur], buf[cur]);
-        __syncthreads();  // buf[cur] and R[cur] are refilled two iterations later
-    }
+__device__ __forceinline__ bool for_each_block(const DevSim& s, int lb, int lg, float4* smem, int stride,
+                                               Region* R, uint64_t* mbar, Body body) {
+    return staged_blocks<kStageBuffers>(s, StageOps{smem, stride, R, mbar}, lb, lg, body);
 }
 
 // Particles of region cell q that were staged: all of them unless the region overflowed
@@ -877,11 +890,9 @@ __device__ __forceinline__ void force_body(const DevSim& s, int lb, int lg) {
     uint64_t* const mbar = ss.mbar;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (threadIdx.x == 0) {
-        for (int k = 0; k < kStageBuffers; ++k) mbar_init(&mbar[k], 1);
         ss.next_cell[0] = ss.next_cell[1] = 0;
         ss.ke_fix = 0ull;
     }
-    __syncthreads();
     int blk_it = 0;  // blocks of this CTA so far (the parity selects the counter)
     float hdt0 = 0.f, hdt1 = 0.f;
     if (KE) {
@@ -895,8 +906,7 @@ __device__ __forceinline__ void force_body(const DevSim& s, int lb, int lg) {
     StreamRings* SRp = nullptr;  // candidate streams of the stencil mode
     if constexpr (MODE == 1) SRp = &warp_streams(w);
     for_each_block(s, lb, lg, smem, s.smax + 1, R, mbar,
-                   [&](const BlockPos& bp, const Region& Rc,
-                                                      const float4* sm) {
+                   [&](const BlockPos& bp, const Region& Rc, const float4* sm, int) {
         const int par = blk_it & 1;
         if (threadIdx.x == 0) ss.next_cell[par ^ 1] = 0;  // for the next block
         ++blk_it;
@@ -1209,15 +1219,11 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
     StreamRings& SR = warp_streams(w);
     uint16_t* buf = nullptr;
     if constexpr (BUFFER) buf = entry_buffer(ss, w, lane);
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < kStageBuffers; ++k) mbar_init(&mbar[k], 1);
-        ss.next_cell[0] = ss.next_cell[1] = 0;
-    }
-    __syncthreads();
+    if (threadIdx.x == 0) ss.next_cell[0] = ss.next_cell[1] = 0;
     int blk_it = 0;  // blocks of this CTA so far (the parity selects the cell counter)
     const float far = kFar;
-    for_each_block(s, lb, lg, smem, s.smax + 1, R, mbar, [&](const BlockPos& bp, const Region& Rc,
-                                                           const float4* sm) {
+    for_each_block(s, lb, lg, smem, s.smax + 1, R, mbar,
+                   [&](const BlockPos& bp, const Region& Rc, const float4* sm, int) {
         const int par = blk_it & 1;
         if (threadIdx.x == 0) ss.next_cell[par ^ 1] = 0;  // for the next block
         ++blk_it;
