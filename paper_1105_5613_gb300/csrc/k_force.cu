@@ -239,7 +239,7 @@ __device__ void region_info(const DevSim& s, const BlockPos& b, Region& R) {
         }
         const int nb = (a[2] * s.nc[1] + a[1]) * s.nc[0] + a[0];
         const int st = s.cell_start[nb];
-        cnt = s.cell_start[nb + 1] - st;
+        cnt = cell_count(st, s.cell_start[nb + 1], s.smax);
         R.start[tid] = st;
         R.cnt[tid] = cnt;
     }

@@ -735,6 +735,8 @@ void launch_unpack_cells(const DevSim& s, cudaStream_t st, int64_t* cell) {
 }
 
 void launch_slot_of(const DevSim& s, cudaStream_t st, int32_t* slot_of) {
+    // (ids left half reordered by a launch that was given up do not cover every entry)
+    cudaMemsetAsync(slot_of, 0, (size_t)s.n * sizeof(int32_t), st);
     k_slot_of<<<s.grid_part, kThreads, 0, st>>>(s, slot_of);
 }
 

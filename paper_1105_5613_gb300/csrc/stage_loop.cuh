@@ -1,6 +1,7 @@
-// Order of the staging of one CTA's blocks: which buffer, which barrier phase, and what
-// happens when a wait gives up.  Plain control flow over an Ops object, so that it compiles
-// for the host as well (tests/host_stage_loop.cpp drives it with a model of the barriers).
+// Staging of one CTA's blocks: the particles a cell contributes, and the order in which the
+// blocks go through the buffers -- which buffer, which barrier phase, and what happens when a
+// wait gives up.  Plain arithmetic, and control flow over an Ops object, so that it compiles for
+// the host as well (tests/host_stage_loop.cpp drives it with a model of the barriers).
 #pragma once
 
 #include <cstdint>
@@ -12,6 +13,15 @@
 #endif
 
 namespace bbmd {
+
+// Particles of a cell whose entries of the cell table are first and next, at most smax + 1 (the
+// region overflows all the same, and a region's sum fits an int).  A launch that was given up
+// half way through a sort leaves old and new entries side by side, each of them in [0, n]: the
+// count is then never negative, and first + count never beyond the larger of the two.
+BBMD_STAGE_FN int cell_count(int first, int next, int smax) {
+    const int c = next > first ? next - first : 0;
+    return c > smax ? smax + 1 : c;
+}
 
 // Blocks lb, lb + lg, ... of system s (below s.nblocks).  With two buffers the copies of the next block are
 // in flight while a block is computed; with one, each block is staged, then computed.

@@ -1,6 +1,8 @@
 // The staging loop (stage_loop.cuh) on the host, over a model of the barriers and buffers that
 // records every use the hardware leaves undefined.  Usage: host_stage_loop <buffers> <blocks>
-// <bodies> <block whose wait gives up, or -1>; prints "ok" or the first misuse.
+// <bodies> <block whose wait gives up, or -1>; prints "ok" or the first misuse.  With the single
+// argument "cells": the counts taken from a cell table of which a sort wrote only a part.
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <string>
@@ -98,7 +100,38 @@ static int run(int64_t blocks, int bodies, int64_t fail_at) {
     return 0;
 }
 
+// Tables of n particles in `cells` cells, every entry from one or the other of two sorts.
+static int torn_cells() {
+    const int n = 2000000000, cells = 144, smax = 65000;
+    uint64_t x = 1;
+    auto draw = [&](uint64_t m) { return (x = x * 6364136223846793005ull + 1442695040888963407ull, (x >> 33) % m); };
+    for (int trial = 0; trial < 1000; ++trial) {
+        std::vector<std::vector<int>> sorted(2, std::vector<int>(cells + 1));
+        for (auto& s : sorted) {
+            for (int& v : s) v = (int)draw((uint64_t)n + 1);
+            std::sort(s.begin(), s.end());
+            s[0] = 0;
+            s[cells] = n;
+        }
+        std::vector<int> torn(cells + 1);
+        for (int c = 0; c <= cells; ++c) torn[(size_t)c] = sorted[draw(2)][(size_t)c];
+        int sum = 0;
+        for (int c = 0; c < cells; ++c) {
+            const int first = torn[(size_t)c], k = bbmd::cell_count(first, torn[(size_t)c + 1], smax);
+            if (k < 0 || k > n - first || k > smax + 1 || __builtin_add_overflow(sum, k, &sum))
+                return std::puts("a count out of range"), 0;
+        }
+        for (int c = 0; c < cells; ++c) {  // a whole table: the counts themselves
+            const int k = sorted[0][(size_t)c + 1] - sorted[0][(size_t)c];
+            if (bbmd::cell_count(sorted[0][(size_t)c], sorted[0][(size_t)c + 1], smax) != std::min(k, smax + 1))
+                return std::puts("a count of a whole table changed"), 0;
+        }
+    }
+    return std::puts("ok"), 0;
+}
+
 int main(int argc, char** argv) {
+    if (argc == 2) return torn_cells();
     if (argc != 5) return 2;
     const int64_t blocks = std::atoll(argv[2]), fail_at = std::atoll(argv[4]);
     const int bodies = std::atoi(argv[3]);

@@ -1,7 +1,7 @@
 """The order in which a CTA stages its blocks, compiled for the host over a model of the
 mbarriers: kernels that run several bodies never initialise a live barrier, no buffer is
 refilled while in use or in flight, and a wait that gives up is reported with no copy left
-in flight."""
+in flight.  Counts from a cell table that a launch left half sorted stay in range."""
 import os
 import subprocess
 
@@ -30,3 +30,7 @@ def test_bodies_one_after_the_other(loop, buffers, blocks, bodies):
 @pytest.mark.parametrize("fail_at", [1, 4, 7, 19])
 def test_a_wait_that_gives_up(loop, buffers, fail_at):
     assert loop(buffers, 20, 2, fail_at) == "ok"
+
+
+def test_cells_of_a_table_half_sorted(loop):
+    assert loop("cells") == "ok"
