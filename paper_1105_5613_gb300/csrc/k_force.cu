@@ -365,15 +365,9 @@ __device__ __forceinline__ int staged_count(const Region& R, int q) {
     return min(R.cnt[q], R.off[q + 1] - R.off[q]);
 }
 
-// Global index of staged entry t (rare path): binary search of the region prefix.
-__device__ __forceinline__ int64_t staged_global(const Region& R, int t) {
-    int lo = 0, hi = kRegion - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (R.off[mid] <= t) lo = mid;
-        else hi = mid - 1;
-    }
-    return (int64_t)R.start[lo] + (t - R.off[lo]);
+// Global index of staged entry t (rare path).
+__device__ __forceinline__ int64_t staged_global(const DevSim& s, const Region& R, int t) {
+    return staged_particle(R.start, R.off, kRegion, t, s.n);
 }
 
 // The warp's own cell: its region index and whether it exists (odd nc leaves some warps of
@@ -502,7 +496,7 @@ __device__ __forceinline__ void pair_band(const DevSim& s, const Region& R, cons
     const bool b = p.w != 0.f;
     if (!valid || !(fabsf(r2 - (b ? T.rm1 : T.rm0)) < T.hw)) return;
     if (!min_image_copy(s, dx, dy, dz)) return;
-    int64_t gj = staged_global(R, t);
+    int64_t gj = staged_global(s, R, t);
     if (r2_exact(s, gi, gj) < s.pt.rc2[T.si * 2 + (b ? 1 : 0)])
         pair_add<FSHIFT>(T, b, dx, dy, dz, r2, true, a);
 }
@@ -1057,7 +1051,7 @@ __device__ __forceinline__ void force_body(const DevSim& s, int lb, int lg) {
                                                     fmaf(m2z, 0.5f, W.z[u])))
                                     continue;
                                 const int t = (int)SR.idx[S][(cq + u) & (kSRing - 1)];
-                                const int64_t gj = staged_global(Rc, t);
+                                const int64_t gj = staged_global(s, Rc, t);
                                 if (r2_exact(s, gi, gj) < s.pt.rc2[si * 2 + S]) inw |= bit;
                             }
                         }
@@ -1294,7 +1288,7 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
                                                 fmaf(m2z, 0.5f, W.z[u])))
                                 continue;
                             const int t = (int)SR.idx[S][(cq + u) & (kSRing - 1)];
-                            const int64_t gj = staged_global(Rc, t);
+                            const int64_t gj = staged_global(s, Rc, t);
                             if (r2_exact(s, gi, gj) < s.pt.R2[si * 2 + S]) inw |= bit;
                         }
                     }

@@ -102,10 +102,11 @@ static int run(int64_t blocks, int bodies, int64_t fail_at) {
 
 // Tables of n particles in `cells` cells, every entry from one or the other of two sorts.
 static int torn_cells() {
-    const int n = 2000000000, cells = 144, smax = 65000;
+    const int cells = 144, smax = 65000;
     uint64_t x = 1;
     auto draw = [&](uint64_t m) { return (x = x * 6364136223846793005ull + 1442695040888963407ull, (x >> 33) % m); };
     for (int trial = 0; trial < 1000; ++trial) {
+        const int n = trial % 2 ? 2000000000 : 20000;  // (a region overflows, or holds them all)
         std::vector<std::vector<int>> sorted(2, std::vector<int>(cells + 1));
         for (auto& s : sorted) {
             for (int& v : s) v = (int)draw((uint64_t)n + 1);
@@ -121,9 +122,20 @@ static int torn_cells() {
             if (k < 0 || k > n - first || k > smax + 1 || __builtin_add_overflow(sum, k, &sum))
                 return std::puts("a count out of range"), 0;
         }
+        // the region's prefix, cut at smax; entries up to the sentinel's may stand in a list
+        std::vector<int> off(cells + 1, 0);
+        for (int c = 0, t = 0; c < cells; ++c) {
+            t += bbmd::cell_count(torn[(size_t)c], torn[(size_t)c + 1], smax);
+            off[(size_t)c + 1] = std::min(t, smax);
+        }
+        for (int t = 0; t <= smax; t += 97) {
+            const int64_t i = bbmd::staged_particle(torn.data(), off.data(), cells, t, n);
+            if (i < 0 || i >= n) return std::puts("a staged entry out of range"), 0;
+        }
+        const std::vector<int>& s0 = sorted[0];
         for (int c = 0; c < cells; ++c) {  // a whole table: the counts themselves
-            const int k = sorted[0][(size_t)c + 1] - sorted[0][(size_t)c];
-            if (bbmd::cell_count(sorted[0][(size_t)c], sorted[0][(size_t)c + 1], smax) != std::min(k, smax + 1))
+            const int k = s0[(size_t)c + 1] - s0[(size_t)c];
+            if (bbmd::cell_count(s0[(size_t)c], s0[(size_t)c + 1], smax) != std::min(k, smax + 1))
                 return std::puts("a count of a whole table changed"), 0;
         }
     }
