@@ -394,6 +394,18 @@ const char* bbmd_batch_last_error(const bbmd_batch* b);
  * Synchronising. */
 bbmd_status bbmd_gr_counts_noalloc(bbmd_sim* sim, int32_t nbins, double rmax, uint64_t* counts);
 
+/* Limits of the device's waits in the launches of this handle.  barrier_ns (default 2e9, at
+ * least 1, else BBMD_ERR_ARG): a wait at the grid-wide barrier of the launches that run several
+ * phases (the steps and descents of small systems, the rebuild trigger and sort).
+ * staging_tries (default 2^18): looks for the copies of a block into shared memory; with 0 the
+ * first wait gives up at once (its copies are still waited for).  A wait that runs out ends its
+ * launch, later launches of several phases return at once, and every synchronising call from
+ * then on returns BBMD_ERR_TIMEOUT.  The state is then that of a step half done (destroy the
+ * handle); the device context stays usable.  The waits between the phases of a replica batch
+ * have their own limit (bbmd_batch_set_wait_limit).  Takes effect at the next call.  The paper
+ * has no counterpart (failure detection of this design). */
+bbmd_status bbmd_set_wait_limits(bbmd_sim* sim, uint64_t barrier_ns, uint32_t staging_tries);
+
 /* Message of the last failed call on this handle ("" if none). */
 const char* bbmd_last_error(const bbmd_sim* sim);
 

@@ -364,6 +364,9 @@ bbmd_status read_status(bbmd_sim* sim, int known = -1) {
         CK(cudaMemcpyAsync(&st, &sim->d.sc->status, sizeof(int), cudaMemcpyDeviceToHost, sim->st));
         CK(cudaStreamSynchronize(sim->st));
     }
+    sim->sticky |= st & ST_TIMEOUT;
+    if (sim->sticky & ST_TIMEOUT)  // (first: the rest of the word is that of a state half advanced)
+        return fail(sim, BBMD_ERR_TIMEOUT, "a bounded device wait gave up");
     if (st & ST_LIST_OVERFLOW) {
         bbmd_status g = grow_lists(sim);
         if (g != BBMD_OK) return g;
@@ -377,7 +380,6 @@ bbmd_status read_status(bbmd_sim* sim, int known = -1) {
                     "stencil_capacity)");
     if (sim->sticky & (ST_NONFINITE | ST_VEL_RANGE))
         return fail(sim, BBMD_ERR_NUMERIC, "non-finite force or velocity beyond the fixed-point range");
-    if (sim->sticky & ST_TIMEOUT) return fail(sim, BBMD_ERR_TIMEOUT, "a bounded device wait gave up");
     return BBMD_OK;
 }
 
@@ -652,6 +654,8 @@ bbmd_status bbmd_create(const bbmd_params* params, int64_t n, const double box[3
     D.ncell = (int32_t)ncell;
     D.nbr_mode = params->nbr_mode;
     D.precision = params->precision;
+    D.wait_ns = kBarrierWaitNs;
+    D.stage_tries = kStageTries;
     fill_pair_table(*params, D.pt);
     for (int k = 0; k < 4; ++k)
         D.pt.rcfix[k] = (long long)std::ceil(std::ldexp(D.pt.drc[k], D.kexp));
@@ -1237,6 +1241,16 @@ bbmd_status bbmd_rebuild(bbmd_sim* sim) {
     launch_force(sim->d, sim->st, false, false);
     LAUNCHED("rebuild forces");
     return read_status(sim);
+}
+
+bbmd_status bbmd_set_wait_limits(bbmd_sim* sim, uint64_t barrier_ns, uint32_t staging_tries) {
+    if (!sim) return BBMD_ERR_ARG;
+    if (barrier_ns == 0) return fail(sim, BBMD_ERR_ARG, "barrier_ns must be at least 1");
+    DeviceGuard dg(sim->device);
+    sim->d.wait_ns = barrier_ns;
+    sim->d.stage_tries = staging_tries;
+    free_graphs(sim);  // the captured launches carry the previous limits
+    return BBMD_OK;
 }
 
 bbmd_status bbmd_get_info(const bbmd_sim* sim, bbmd_info* info) {

@@ -64,6 +64,11 @@ enum : int32_t {
 enum { kSyncArrive = 0, kSyncRelease, kSyncAbort, kSyncMax0, kSyncMax1, kSyncWords };
 constexpr int kSyncStride = 32;
 
+// Limits of the device's waits (bbmd_set_wait_limits): a wait at the grid-wide barrier in ns,
+// tries of a wait for staged copies.
+constexpr uint64_t kBarrierWaitNs = 2000000000ull;
+constexpr uint32_t kStageTries = 1u << 18;
+
 struct DevScalars {
     double xi, eta;          // Nose-Hoover friction and its time integral
     double K;                // kinetic energy of the stored (full-step) velocities
@@ -134,6 +139,8 @@ struct alignas(16) DevSim {
     double* partials;        // [kMaxPartials][4]
     DevScalars* sc;
     uint32_t* gsync;         // grid-wide barrier of the one-launch step (kSyncWords words)
+    uint64_t wait_ns;        // limit of a wait at it
+    uint32_t stage_tries;    // tries of a wait for staged copies
     int32_t grid_part;       // grid of per-particle grid-stride kernels
     int32_t grid_cell;       // grid of the force kernel (kBlockWarps warps per CTA)
     int32_t grid_list;       // grid of the list-build kernel
@@ -226,6 +233,12 @@ __device__ __forceinline__ double r2_exact(const DevSim& s, int64_t i, int64_t j
 
 __device__ __forceinline__ void set_status(const DevSim& s, int bits) {
     atomicOr(&s.sc->status, bits);
+}
+
+// Whether a launch of the system was given up (the same on every thread of the CTA, which
+// synchronises): its state is then that of a phase half done, and no phase is run on it.
+__device__ __forceinline__ bool given_up(const DevSim& s) {
+    return __syncthreads_or(threadIdx.x == 0 && (*(volatile int*)&s.sc->status & ST_TIMEOUT));
 }
 
 // ------------------------------------------------------------------ replica batches ----

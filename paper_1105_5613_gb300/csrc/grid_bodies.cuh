@@ -9,12 +9,11 @@ __device__ __forceinline__ unsigned long long globaltimer_ns() {
     return t;
 }
 
-constexpr unsigned long long kGridWaitNs = 2000000000ull;  // a barrier wait gives up after it
-
 // Barrier over the CTAs of the launch; gen counts the barriers passed.  With `last` set, the
 // last CTA to arrive runs on_last before the others go on.  Every CTA is resident
-// (cooperative launch), so a wait ends; should one not end within kGridWaitNs, the CTA
+// (cooperative launch), so a wait ends; should one not end within s.wait_ns, the CTA
 // raises the abort flag and ST_TIMEOUT, and every CTA leaves (false) at its next barrier.
+// The clock is read at every 64th look, or at every one where the limit is below a millisecond.
 template <class OnLast>
 __device__ __forceinline__ bool grid_barrier(const DevSim& s, unsigned& gen, bool last, OnLast on_last) {
     __shared__ int verdict;  // 0: abort, 1: go on, 2: this CTA arrived last
@@ -31,11 +30,12 @@ __device__ __forceinline__ bool grid_barrier(const DevSim& s, unsigned& gen, boo
         } else {
             const int word = (last ? kSyncRelease : kSyncArrive) * kSyncStride;
             const unsigned want = last ? gen : target;
+            const unsigned skip = s.wait_ns < 1000000ull ? 0u : 63u;
             unsigned long long t0 = 0;
             for (unsigned it = 0; w[word] < want; ++it) {
-                if ((it & 63u) != 63u) continue;
+                if ((it & skip) != skip) continue;
                 if (t0 == 0) t0 = globaltimer_ns();
-                if (w[kSyncAbort * kSyncStride] != 0u || globaltimer_ns() - t0 > kGridWaitNs) {
+                if (w[kSyncAbort * kSyncStride] != 0u || globaltimer_ns() - t0 > s.wait_ns) {
                     w[kSyncAbort * kSyncStride] = 1u;
                     set_status(s, ST_TIMEOUT);
                     v = 0;

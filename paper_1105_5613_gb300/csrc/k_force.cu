@@ -175,15 +175,13 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* mbar, uint32_t parity) {
     return ok != 0;
 }
 
-// Wait for the current phase with an iteration limit.  On expiry raise ST_TIMEOUT, wait
+// Wait for the current phase, s.stage_tries tries at most.  On expiry raise ST_TIMEOUT, wait
 // once more (again bounded) for the copies still in flight, and return false.
-constexpr int kWaitLimit = 1 << 18;
-
 __device__ __forceinline__ bool mbar_wait_bounded(const DevSim& s, uint64_t* mbar, uint32_t parity) {
-    for (int it = 0; it < kWaitLimit; ++it)
+    for (uint32_t it = 0; it < s.stage_tries; ++it)
         if (mbar_try_wait(mbar, parity)) return true;
     set_status(s, ST_TIMEOUT);
-    for (int it = 0; it < kWaitLimit; ++it)
+    for (uint32_t it = 0; it < kStageTries; ++it)
         if (mbar_try_wait(mbar, parity)) break;
     return false;
 }
@@ -1450,6 +1448,7 @@ __device__ __forceinline__ void grid_force(const DevSim& s) {
 
 template <bool KE, bool FSHIFT>
 __global__ void __launch_bounds__(kBW * 32, BBMD_GRID_MIN_BLOCKS) k_step_grid(DevSim s, int nsteps) {
+    if (given_up(s)) return;
     const int lb = (int)blockIdx.x, lg = (int)gridDim.x;
     unsigned gen = 0;
     for (int step = 0; step < nsteps; ++step) {
@@ -1467,6 +1466,7 @@ __global__ void __launch_bounds__(kBW * 32, BBMD_GRID_MIN_BLOCKS) k_step_grid(De
 template <bool FSHIFT>
 __global__ void __launch_bounds__(kBW * 32, BBMD_GRID_MIN_BLOCKS)
     k_relax_grid(DevSim s, int nsteps, double hmax, double dmax) {
+    if (given_up(s)) return;
     const int lb = (int)blockIdx.x, lg = (int)gridDim.x;
     unsigned gen = 0;
     for (int step = 0; step < nsteps; ++step) {

@@ -34,6 +34,7 @@ BBMD_ONE_AND_MANY(kThreads, k_copyback, copyback_body)
 // launches of a captured step become one, which returns at once in a step in which no
 // displacement came near the threshold.  (The four-CTA bound: the phases are bound by memory.)
 __global__ void __launch_bounds__(kThreads, 4) k_trigger_sort(DevSim s) {
+    if (!s.sc->near || given_up(s)) return;
     unsigned gen = 0;
     bool due;
     if (!grid_trigger(s, gen, due)) return;
