@@ -67,6 +67,12 @@ __device__ __forceinline__ bool grid_barrier(const DevSim& s, unsigned& gen) {
     return grid_barrier(s, gen, false, [] {});
 }
 
+// Ends the launch for a CTA that cannot go on: the others leave at their next barrier.
+__device__ __forceinline__ bool grid_abort(const DevSim& s) {
+    if (threadIdx.x == 0) *(volatile uint32_t*)&s.gsync[kSyncAbort * kSyncStride] = 1u;
+    return false;
+}
+
 // Rebuild trigger after the integrate phase (whose flags the caller has put behind a barrier):
 // due, the same on every thread, tells whether a rebuild is due; the cell counts are then
 // zero.  False after an abort.

@@ -872,10 +872,11 @@ __device__ __forceinline__ bool force_selected(const DevSim& s) {
 }
 
 // MODE 0: Verlet list.  MODE 1: every particle of the 27-cell stencil (no stored list).
-// BAND_INL: the band fix-up inline (else called out of line).
+// BAND_INL: the band fix-up inline (else called out of line).  False (on every thread of the
+// CTA) if a staging wait gave up: the CTA must not stage again (staged_blocks).
 template <int MODE, bool KE, bool FSHIFT, bool BAND_INL = kBandInline>
-__device__ __forceinline__ void force_body(const DevSim& s, int lb, int lg) {
-    if (!force_selected<MODE>(s)) return;  // CTA-uniform, before any barrier
+__device__ __forceinline__ bool force_body(const DevSim& s, int lb, int lg) {
+    if (!force_selected<MODE>(s)) return true;  // CTA-uniform, before any barrier
     extern __shared__ float4 smem[];
     StageShared& ss = stage_shared();
     Region* const R = ss.R;
@@ -897,8 +898,8 @@ __device__ __forceinline__ void force_body(const DevSim& s, int lb, int lg) {
     const uint4 sent = make_uint4(sv, sv, sv, sv);
     StreamRings* SRp = nullptr;  // candidate streams of the stencil mode
     if constexpr (MODE == 1) SRp = &warp_streams(w);
-    for_each_block(s, lb, lg, smem, s.smax + 1, R, mbar,
-                   [&](const BlockPos& bp, const Region& Rc, const float4* sm, int) {
+    const bool staged = for_each_block(s, lb, lg, smem, s.smax + 1, R, mbar,
+                                       [&](const BlockPos& bp, const Region& Rc, const float4* sm, int) {
         const int par = blk_it & 1;
         if (threadIdx.x == 0) ss.next_cell[par ^ 1] = 0;  // for the next block
         ++blk_it;
@@ -1146,11 +1147,13 @@ __device__ __forceinline__ void force_body(const DevSim& s, int lb, int lg) {
             }
         }
     });
+    if (!staged) return false;
     if (KE) {
         // every warp has passed the last block's closing barrier
         const double acc_ke = threadIdx.x == 0 ? __ull2double_rn(ss.ke_fix) * 0x1p-32 : 0.0;
         block_partials(s, lb, &acc_ke, 0, 1);
     }
+    return true;
 }
 
 // ------------------------------------------------------------------ list build ----
@@ -1198,9 +1201,10 @@ __device__ __forceinline__ uint16_t* entry_buffer(StageShared& ss, int w, int la
     return more[w - kFree][lane];
 }
 
+// False as force_body.
 template <bool BUFFER>
-__device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg) {
-    if (!s.sc->rebuild) return;
+__device__ __forceinline__ bool list_build_body(const DevSim& s, int lb, int lg) {
+    if (!s.sc->rebuild) return true;
     extern __shared__ float4 smem[];
     StageShared& ss = stage_shared();
     Region* const R = ss.R;
@@ -1214,8 +1218,8 @@ __device__ __forceinline__ void list_build_body(const DevSim& s, int lb, int lg)
     if (threadIdx.x == 0) ss.next_cell[0] = ss.next_cell[1] = 0;
     int blk_it = 0;  // blocks of this CTA so far (the parity selects the cell counter)
     const float far = kFar;
-    for_each_block(s, lb, lg, smem, s.smax + 1, R, mbar,
-                   [&](const BlockPos& bp, const Region& Rc, const float4* sm, int) {
+    return for_each_block(s, lb, lg, smem, s.smax + 1, R, mbar,
+                          [&](const BlockPos& bp, const Region& Rc, const float4* sm, int) {
         const int par = blk_it & 1;
         if (threadIdx.x == 0) ss.next_cell[par ^ 1] = 0;  // for the next block
         ++blk_it;
@@ -1432,18 +1436,20 @@ __device__ __forceinline__ bool grid_rebuild(const DevSim& s, unsigned& gen, OnL
     if (s.nbr_mode == BBMD_NBR_VERLET) {
         if (!grid_barrier(s, gen)) return false;
         for (int b = (int)blockIdx.x; b < s.grid_list; b += (int)gridDim.x)
-            list_build_body<true>(s, b, s.grid_list);
+            if (!list_build_body<true>(s, b, s.grid_list)) return grid_abort(s);
     }
     return grid_barrier(s, gen, true, on_last);
 }
 
-// Forces with the CTA index and count of the force kernel's own launch.
+// Forces with the CTA index and count of the force kernel's own launch.  False after a staging
+// wait that gave up.
 template <bool KE, bool FSHIFT>
-__device__ __forceinline__ void grid_force(const DevSim& s) {
-    for (int b = (int)blockIdx.x; b < s.grid_cell; b += (int)gridDim.x) {
-        force_body<0, KE, FSHIFT, false>(s, b, s.grid_cell);
-        force_body<1, KE, FSHIFT, false>(s, b, s.grid_cell);
-    }
+__device__ __forceinline__ bool grid_force(const DevSim& s) {
+    for (int b = (int)blockIdx.x; b < s.grid_cell; b += (int)gridDim.x)
+        if (!force_body<0, KE, FSHIFT, false>(s, b, s.grid_cell) ||
+            !force_body<1, KE, FSHIFT, false>(s, b, s.grid_cell))
+            return grid_abort(s);
+    return true;
 }
 
 template <bool KE, bool FSHIFT>
@@ -1457,7 +1463,7 @@ __global__ void __launch_bounds__(kBW * 32, BBMD_GRID_MIN_BLOCKS) k_step_grid(De
         bool due;
         if (!grid_trigger(s, gen, due)) return;
         if (due && !grid_rebuild(s, gen, [] {})) return;
-        grid_force<KE, FSHIFT>(s);
+        if (!grid_force<KE, FSHIFT>(s)) return;
         if (!grid_barrier(s, gen, true, [&] { finalize_body(s, KE ? 1 : 0); })) return;
     }
 }
@@ -1472,7 +1478,7 @@ __global__ void __launch_bounds__(kBW * 32, BBMD_GRID_MIN_BLOCKS)
     for (int step = 0; step < nsteps; ++step) {
         // (squares of FP32 forces are not negative: their bits order like the values)
         uint32_t* const slot = &s.gsync[(kSyncMax0 + (step & 1)) * kSyncStride];
-        grid_force<false, FSHIFT>(s);
+        if (!grid_force<false, FSHIFT>(s)) return;
         if (!grid_barrier(s, gen)) return;
         const float m = maxf_body(s, lb, lg);
         if ((threadIdx.x & 31) == 0) atomicMax(slot, __float_as_uint(m));
@@ -1508,14 +1514,15 @@ __global__ void __launch_bounds__(kBW * 32, BBMD_GRID_MIN_BLOCKS)
 // overlap; an item waits only on items handed out before it, and every CTA is resident,
 // so the queue always advances.
 #if BBMD_BLOCK_Z == BBMD_PERSIST_Z
-// Raise the abort flag and ST_TIMEOUT on every replica.
+// Raise the abort flag and ST_TIMEOUT on every replica (one thread).
 __device__ __forceinline__ void persistent_abort(const PersistentStep& a) {
     if (atomicExch(a.abort, 1) == 0)
         for (int r = 0; r < a.nrep; ++r) atomicOr(&a.sims[r].sc->status, ST_TIMEOUT);
 }
 
+// False (on every thread) if a staging wait gave up.
 template <bool KE, bool FSHIFT>
-__device__ __forceinline__ void run_phase(int phase, const DevSim& s, int lb, int lg) {
+__device__ __forceinline__ bool run_phase(int phase, const DevSim& s, int lb, int lg) {
     switch (phase) {
         case kPhIntegrate: integrate_body<false>(s, lb, lg); break;
         case kPhCelltop: celltop_body(s, lb, lg); break;
@@ -1526,15 +1533,14 @@ __device__ __forceinline__ void run_phase(int phase, const DevSim& s, int lb, in
         case kPhScatter: scatter_body(s, lb, lg); break;
         case kPhSortGather: sortgather_body(s, lb, lg); break;
         case kPhCopyback: copyback_body(s, lb, lg); break;
-        case kPhList: list_build_body<true>(s, lb, lg); break;
+        case kPhList: return list_build_body<true>(s, lb, lg);
         case kPhForce:
             // the list body, or for a replica whose lists are cut (and in cell mode) the
             // stencil body: each returns at once when not selected
-            force_body<0, KE, FSHIFT, false>(s, lb, lg);
-            force_body<1, KE, FSHIFT, false>(s, lb, lg);
-            break;
+            return force_body<0, KE, FSHIFT, false>(s, lb, lg) && force_body<1, KE, FSHIFT, false>(s, lb, lg);
         default: finalize_body(s, KE ? 1 : 0); break;
     }
+    return true;
 }
 
 template <bool KE, bool FSHIFT>
@@ -1592,7 +1598,10 @@ __global__ void __launch_bounds__(kBW * 32, 2) k_step_persistent(PersistentStep 
             int4* dst4 = reinterpret_cast<int4*>(&sh);
             for (int k = threadIdx.x; k < (int)(sizeof(DevSim) / 16); k += blockDim.x) dst4[k] = src4[k];
             __syncthreads();
-            run_phase<KE, FSHIFT>(d.x, sh, d.z, d.w);
+            if (!run_phase<KE, FSHIFT>(d.x, sh, d.z, d.w)) {
+                if (threadIdx.x == 0) persistent_abort(a);
+                return;
+            }
         }
         __syncthreads();
         if (threadIdx.x == 0) {

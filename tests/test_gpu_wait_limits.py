@@ -87,3 +87,69 @@ def test_a_barrier_wait_of_a_descent_that_runs_out(ncell, shape):
     assert e.value.code == 7
     every_call_times_out(sim)
     sim.close()
+
+
+def moved_at_most(sim, pos, L, dist):
+    """The positions on the device (get_state fills its arrays whatever status it returns)."""
+    now = np.empty_like(pos)
+    dp = bbmd.C.POINTER(bbmd.C.c_double)
+    rc = bbmd.load().bbmd_get_state(sim.h, now.ctypes.data_as(dp), None, None)
+    assert rc == 7  # BBMD_ERR_TIMEOUT
+    d = now - pos
+    d -= L * np.round(d / L)
+    return np.abs(d).max() <= dist
+
+
+# a staging wait that gives up ends the launch of many steps: none is taken on old forces
+@pytest.mark.parametrize("ncell,shape,kw", [(10, 1, {}), (16, 4, {}), (16, 2, {"nbr_mode": bbmd.NBR_CELL})])
+def test_a_staging_wait_that_gives_up(ncell, shape, kw):
+    ref = make(ncell, shape, **kw)
+    ref.step(30, 0.005, NH)
+    want = ref.get_state()
+    ref.close()
+    sim = make(ncell, shape, **kw)
+    pos, vel, _ = sim.get_state()
+    L = mixture(ncell)[1]
+    mode = kw.get("nbr_mode", bbmd.NBR_VERLET)
+    sim.set_wait_limits(staging_tries=0)
+    sim.step(400, 0.005)
+    assert moved_at_most(sim, pos, L, 2 * 0.005 * 2 * np.abs(vel).max())
+    every_call_times_out(sim, mode)
+    sim.close()
+    sim = make(ncell, shape, **kw)
+    sim.set_wait_limits(staging_tries=0)
+    with pytest.raises(bbmd.BBMDError) as e:
+        sim.minimize(400, 1e-3, 0.05)
+    assert e.value.code == 7
+    assert moved_at_most(sim, pos, L, 2 * 0.05)
+    sim.close()
+    still_works(ncell, shape, want, **kw)
+
+
+def test_a_staging_wait_of_a_captured_step_that_gives_up():
+    sim = make(36, 1)
+    sim.set_wait_limits(staging_tries=0)
+    sim.step(5, 0.005)
+    every_call_times_out(sim)
+    sim.close()
+
+
+def test_a_staging_wait_of_a_replica_that_gives_up():
+    sys = [mixture(m, shake=0.1) for m in (8, 9, 10)]
+    ns, boxes, pos, vel, sp = zip(*sys)
+    b = bbmd.Batch(bbmd.ka_params(), ns, boxes, sp, pos, vel)
+    assert b.uses_persistent()
+    b.step(3, 0.005)
+    b.replica(1).set_wait_limits(staging_tries=0)
+    b.step(400, 0.005)
+    for r in range(3):
+        with pytest.raises(bbmd.BBMDError) as e:
+            b.replica(r).observe(0)
+        assert e.value.code == 7, r
+    v = np.abs(vel[1]).max()
+    start = bbmd.Sim(bbmd.ka_params(block_z=4), ns[1], boxes[1], sp[1], pos[1], vel[1])
+    start.step(3, 0.005)
+    p3, _, _ = start.get_state()
+    start.close()
+    assert moved_at_most(b.replica(1), p3, boxes[1], 2 * 0.005 * 2 * v)
+    b.close()
