@@ -1191,13 +1191,14 @@ __device__ __forceinline__ void push_entries(unsigned& top, unsigned e, unsigned
 }
 
 // The lane's entry buffer: 16 entries, 16-byte aligned.  One KB per warp, in the part of the
-// region's description that is free once the block is staged (as many warps as fit), and
-// beside it for the others.
-__device__ __forceinline__ uint16_t* entry_buffer(StageShared& ss, int w, int lane) {
+// description of the region being computed, buffer b's, that is free once its block is staged
+// (as many warps as fit; with two staging buffers the other one describes the next block
+// meanwhile), and beside it for the others.
+__device__ __forceinline__ uint16_t* entry_buffer(StageShared& ss, int b, int w, int lane) {
     constexpr int kFree = (int)(sizeof(Region) - offsetof(Region, hi)) / 1024;  // warps
     constexpr int kMore = kBW > kFree ? kBW - kFree : 1;
     __shared__ __align__(16) uint16_t more[kMore][32][16];
-    if (w < kFree) return reinterpret_cast<uint16_t*>(&ss.R[0].hi[0][0]) + (w * 32 + lane) * 16;
+    if (w < kFree) return reinterpret_cast<uint16_t*>(&ss.R[b].hi[0][0]) + (w * 32 + lane) * 16;
     return more[w - kFree][lane];
 }
 
@@ -1213,13 +1214,13 @@ __device__ __forceinline__ bool list_build_body(const DevSim& s, int lb, int lg)
     const int lcap = s.lcap8 * 8;
     const int lcap2 = lcap >> 1;  // pair slots per particle
     StreamRings& SR = warp_streams(w);
-    uint16_t* buf = nullptr;
-    if constexpr (BUFFER) buf = entry_buffer(ss, w, lane);
     if (threadIdx.x == 0) ss.next_cell[0] = ss.next_cell[1] = 0;
     int blk_it = 0;  // blocks of this CTA so far (the parity selects the cell counter)
     const float far = kFar;
     return for_each_block(s, lb, lg, smem, s.smax + 1, R, mbar,
-                          [&](const BlockPos& bp, const Region& Rc, const float4* sm, int) {
+                          [&](const BlockPos& bp, const Region& Rc, const float4* sm, int b) {
+        uint16_t* buf = nullptr;
+        if constexpr (BUFFER) buf = entry_buffer(ss, b, w, lane);
         const int par = blk_it & 1;
         if (threadIdx.x == 0) ss.next_cell[par ^ 1] = 0;  // for the next block
         ++blk_it;
