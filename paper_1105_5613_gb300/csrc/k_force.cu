@@ -1745,8 +1745,11 @@ __device__ __forceinline__ void pair_fp64(const DevSim& s, int si, long long mx,
     const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
     double ir2, r = 0.0, ir = 0.0;
     if (FSHIFT) {
+        // (the square of the rounded 1/r carries its error and a rounding of its own: one
+        // Newton step makes it the reciprocal of r^2 to its last rounding, as rcp64 is)
         ir = rsqrt64(r2);
-        ir2 = ir * ir;
+        const double sq = ir * ir;
+        ir2 = fma(fma(-r2, sq, 1.0), sq, sq);
         r = r2 * ir;
     } else {
         ir2 = rcp64(r2);
