@@ -1630,9 +1630,9 @@ __global__ void __launch_bounds__(kBW * 32, 2) k_step_persistent(PersistentStep 
 //     queues together, so a slot of the loop computes a pair on nearly every lane, instead
 //     of once per candidate that any of the 32 lanes interacts with;
 //   - r^2 stays in integer units (the scale is folded into the constants), 1/r^2 and 1/r come
-//     from the hardware's approximation and one third-order step, and energies and virial
-//     come from the sums of r^-12 and r^-6 by species pair: 17 operations a pair for forces,
-//     13 for the sums;
+//     from the hardware's approximation and one third-order step, and the virial comes from the
+//     energies and the sum of their attractions: 17 operations a pair for forces, 14 for the
+//     sums (22 and 20 with the force shift, which needs 1/r);
 //   - sums over the system (energy, virial) take each pair from one side only.
 // Measured against the form that ran the FP64 arithmetic for every candidate some lane of
 // the warp interacts with: energy and virial sums at 16.4 M particles (lists, skin 0.4)
@@ -1685,9 +1685,12 @@ __device__ __forceinline__ long long join64(int hi, unsigned lo) {
     return (long long)(((unsigned long long)(unsigned)hi << 32) | lo);
 }
 
-// 1/x and 1/sqrt(x) in FP64: the hardware's approximation y (relative error e below 2^-18)
-// and one third-order step, y (1 + e + e^2 [+ ...]) with e = 1 - x y or 1 - x y^2, whose
-// own error is of order e^3 < 2^-54.
+// 1/x, and 1/sqrt(x) with 1/x, in FP64: the hardware's approximation y (relative error e
+// below 2^-18) and one third-order step, y (1 + e + e^2 [+ ...]) with e = 1 - x y or 1 - x y^2,
+// whose own error is of order e^3 < 2^-54.  Either way 1/x has one rounding and little more: with
+// the square root it comes from the rounded y^2 that e was taken of, for the square of the
+// rounded 1/sqrt(x) would carry that one's error (forces of a liquid with the force shift were
+// off by 1.85e-15 of their rms that way, by 1.15e-15 this way).
 __device__ __forceinline__ double rcp64(double x) {
     double y;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -1695,11 +1698,13 @@ __device__ __forceinline__ double rcp64(double x) {
     return fma(y, fma(e, e, e), y);
 }
 
-__device__ __forceinline__ double rsqrt64(double x) {
+__device__ __forceinline__ void rsqrt64(double x, double& r, double& r2) {
     double y;
     asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double e = fma(-x * y, y, 1.0);
-    return fma(fma(e, 0.375, 0.5), e * y, y);
+    const double y2 = y * y;
+    const double e = fma(-x, y2, 1.0);
+    r = fma(fma(e, 0.375, 0.5), e * y, y);
+    r2 = fma(fma(e, e, e), y2, y2);
 }
 
 // Queue entries per lane: full rows of 8 candidates are added while at most kQ64 - 8 wait.
@@ -1716,12 +1721,18 @@ __device__ __forceinline__ uint16_t* warp_queue64(int w) {
 enum : int { k64Force = 1, k64Energy = 2, k64Sums = 4 };
 
 // One lane's pair constants and accumulators; r^2 and forces in units of 2^-k, so the constants
-// of r^-6 carry 2^6k.
+// of r^-6 carry 2^6k.  The energies are summed pair by pair (sums of r^-12 and r^-6 apart are
+// larger than their difference, and so are their roundings: u_i of a liquid of LJ pairs was off
+// by 4.0e-15 rms that way, by 1.7e-15 this way); the sum of the attractions completes the virial.
 struct Lane64 {
     double a0, a1, b0, b1;                    // 48 eps sigma^12 2^6k, 24 eps sigma^6 (0: soft)
     double dc0, dc1;                          // dV/dr(rc) 2^-7k
+    double e0, e1, g0, g1;                    // 4 eps sigma^12 2^6k, -4 eps sigma^6 (0: soft)
     double fx, fy, fz;                        // sum of f d
-    double t0, t1, u0, u1, q0, q1;            // sums of r^-12, r^-6, r by species of j
+    double rc;                                // cutoff with species A 2^k
+    double t0, t1;                            // sums of 4 eps ((sigma/r)^12 - (sigma/r)^6) by
+                                              // species of j
+    double at, q;                             // sums of -4 eps (sigma/r)^6 and (r - rc) dV/dr(rc)
     int n0, n1;                               // interacting pairs by species of j
 };
 
@@ -1743,14 +1754,9 @@ __device__ __forceinline__ void pair_fp64(const DevSim& s, int si, long long mx,
         if (!(e2 * s.sxd * s.sxd < s.pt.rc2[si * 2 + (b ? 1 : 0)])) return;
     }
     const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-    double ir2, r = 0.0, ir = 0.0;
+    double ir2, ir = 0.0;
     if (FSHIFT) {
-        // (the square of the rounded 1/r carries its error and a rounding of its own: one
-        // Newton step makes it the reciprocal of r^2 to its last rounding, as rcp64 is)
-        ir = rsqrt64(r2);
-        const double sq = ir * ir;
-        ir2 = fma(fma(-r2, sq, 1.0), sq, sq);
-        r = r2 * ir;
+        rsqrt64(r2, ir, ir2);
     } else {
         ir2 = rcp64(r2);
     }
@@ -1767,16 +1773,12 @@ __device__ __forceinline__ void pair_fp64(const DevSim& s, int si, long long mx,
     }
     if (WHAT & (k64Energy | k64Sums)) {
         // (selects, not branches: a divergent branch would take the FP64 pipe twice)
-        const double tn = fma(ir6, ir6, b ? A.t1 : A.t0), un = (b ? A.u1 : A.u0) + ir6;
+        const double gb = b ? A.g1 : A.g0;
+        const double tn = fma(fma(b ? A.e1 : A.e0, ir6, gb), ir6, b ? A.t1 : A.t0);
+        A.at = fma(gb, ir6, A.at);
         A.t0 = b ? A.t0 : tn;
         A.t1 = b ? tn : A.t1;
-        A.u0 = b ? A.u0 : un;
-        A.u1 = b ? un : A.u1;
-        if (FSHIFT) {
-            const double qn = (b ? A.q1 : A.q0) + r;
-            A.q0 = b ? A.q0 : qn;
-            A.q1 = b ? qn : A.q1;
-        }
+        if (FSHIFT) A.q = fma(b ? A.dc1 : A.dc0, fma(r2, ir, -A.rc), A.q);
         A.n0 += b ? 0 : 1;
         A.n1 += b ? 1 : 0;
     }
@@ -1825,6 +1827,10 @@ __device__ __forceinline__ void force64_body(const DevSim& s, int lb, int lg) {
                 const float lo = rc * (1.0f - 2e-6f) - 2.0f, hi = rc * (1.0f + 2e-6f) + 2.0f;
                 in2[b] = lo > 0.f ? lo * lo : 0.f;
                 out2[b] = hi * hi;
+                // (kept in registers: computed anew for every candidate they cost FP64 operations
+                // in the classification -- with the constants below so too, the sums of shifted
+                // forces at 2.05 M in cell mode took 24 ms for 5)
+                asm volatile("" : "+f"(in2[b]), "+f"(out2[b]));
             }
             const int kp = si * 2;
             Lane64 A;
@@ -1835,13 +1841,24 @@ __device__ __forceinline__ void force64_body(const DevSim& s, int lb, int lg) {
                 A.a1 = ldexp(s.pt.deps48[kp + 1] * c1 * c1, 6 * s.kexp);
                 A.b0 = lj ? -0.5 * s.pt.deps48[kp] * c0 : 0.0;
                 A.b1 = lj ? -0.5 * s.pt.deps48[kp + 1] * c1 : 0.0;
-                A.dc0 = A.dc1 = 0.0;
+                A.e0 = ldexp(s.pt.deps4[kp] * c0 * c0, 6 * s.kexp);
+                A.e1 = ldexp(s.pt.deps4[kp + 1] * c1 * c1, 6 * s.kexp);
+                A.g0 = lj ? -s.pt.deps4[kp] * c0 : 0.0;
+                A.g1 = lj ? -s.pt.deps4[kp + 1] * c1 : 0.0;
+                A.dc0 = A.dc1 = A.rc = 0.0;
                 if (FSHIFT) {
+                    A.rc = ldexp(s.pt.drc[kp], s.kexp);
                     A.dc0 = ldexp(s.pt.dfcut[kp], -7 * s.kexp);
                     A.dc1 = ldexp(s.pt.dfcut[kp + 1], -7 * s.kexp);
                 }
+                // (kept in registers, or the compiler computes them anew for every pair, ldexp and
+                // all: forces with the shift at 256 000 in cell mode 2.46 -> 1.80 ms)
+                if (WHAT & k64Force) asm volatile("" : "+d"(A.a0), "+d"(A.a1));
+                if (WHAT & (k64Energy | k64Sums)) asm volatile("" : "+d"(A.e0), "+d"(A.e1));
+                if (FSHIFT) asm volatile("" : "+d"(A.dc0), "+d"(A.dc1));
+                if (FSHIFT && (WHAT & (k64Energy | k64Sums))) asm volatile("" : "+d"(A.rc));
             }
-            A.fx = A.fy = A.fz = A.t0 = A.t1 = A.u0 = A.u1 = A.q0 = A.q1 = 0.0;
+            A.fx = A.fy = A.fz = A.t0 = A.t1 = A.at = A.q = 0.0;
             A.n0 = A.n1 = 0;
             int cnt = 0;
             // classify candidate t; queue it unless it is beyond the cutoff
@@ -1941,20 +1958,16 @@ __device__ __forceinline__ void force64_body(const DevSim& s, int lb, int lg) {
             }
             if ((WHAT & (k64Energy | k64Sums)) && act) {
                 // V = 4 eps (s^12 - s^6) - V(rc) - (r - rc) dV/dr(rc), summed; virial
-                // f r^2 = 12 (4 eps s^12) - 6 (4 eps s^6) + r dV/dr(rc) (soft sphere: no s^6)
-                double u = 0.0, wv = 0.0;
+                // f r^2 = 12 (4 eps (s^12 - s^6)) + 6 (4 eps s^6) + r dV/dr(rc) (soft: no s^6).
+                // (The units of the sums, 2^6k, and of q, 2^-6k: powers of two within range.)
+                const double q = FSHIFT ? ldexp(A.q, 6 * s.kexp) : 0.0;
+                const double v = ldexp(A.t0 + A.t1, 6 * s.kexp);
+                double u = v - q, wv = fma(12.0, v, q) - 6.0 * ldexp(A.at, 6 * s.kexp);
 #pragma unroll
                 for (int b = 0; b < 2; ++b) {
-                    const double sg6 = s.pt.dsig2[kp + b] * s.pt.dsig2[kp + b] * s.pt.dsig2[kp + b];
-                    const double e6 = s.pt.deps4[kp + b] * sg6;
-                    // (the units of the sums, 2^12k and 2^6k, in two steps within range)
-                    const double s12 = ldexp(ldexp(b ? A.t1 : A.t0, 6 * s.kexp) * sg6, 6 * s.kexp) * e6;
-                    const double s6 = lj ? ldexp(b ? A.u1 : A.u0, 6 * s.kexp) * e6 : 0.0;
-                    const double dc = FSHIFT ? s.pt.dfcut[kp + b] : 0.0;
-                    const double sr = FSHIFT ? (b ? A.q1 : A.q0) * s.sxd * dc : 0.0;
-                    const double cut = s.pt.dvshift[kp + b] - s.pt.drc[kp + b] * dc;
-                    u += ((s12 - s6) - sr) - (double)(b ? A.n1 : A.n0) * cut;
-                    wv += fma(12.0, s12, fma(-6.0, s6, sr));
+                    const double np = (double)(b ? A.n1 : A.n0), dc = FSHIFT ? s.pt.dfcut[kp + b] : 0.0;
+                    u -= np * (s.pt.dvshift[kp + b] + (s.pt.drc[kp] - s.pt.drc[kp + b]) * dc);
+                    wv += np * (s.pt.drc[kp] * dc);
                 }
                 const double half = WHAT & k64Sums ? 1.0 : 0.5;
                 if (WHAT & k64Energy) s.ud[gi] = half * u;

@@ -29,8 +29,8 @@ def _lib():
     bbmd.load()
 
 
-def system():
-    n, L, pos, vel, sp = mixture(NCELL, seed=3, shake=0.13)
+def system(shake=0.13):
+    n, L, pos, vel, sp = mixture(NCELL, seed=3, shake=shake)
     return n, L, pos, sp
 
 
@@ -94,4 +94,20 @@ def test_forces_round_like_plain_fp64(pot, shift, mode):
     p = bbmd.ka_params(precision=bbmd.PREC_FP64, potential=pot, shift=shift, nbr_mode=mode)
     sim = bbmd.Sim(p, n, L, sp, pos, np.zeros_like(pos))
     assert rms(sim.get_forces(), wide) <= 1.15 * rms(plain, wide)
+    sim.close()
+
+
+@pytest.mark.parametrize("pot", [bbmd.POT_LJ, bbmd.POT_SOFT])
+@pytest.mark.parametrize("shift", [bbmd.SHIFT_NONE, bbmd.SHIFT_ENERGY, bbmd.SHIFT_FORCE])
+@pytest.mark.parametrize("prec,mode", [(bbmd.PREC_FP64, bbmd.NBR_VERLET), (bbmd.PREC_MIXED, bbmd.NBR_VERLET),
+                                       (bbmd.PREC_MIXED, bbmd.NBR_CELL)])
+def test_energies_round_like_plain_fp64(pot, shift, prec, mode):
+    # (a small shake: attraction and repulsion of the order of their sum, as in a liquid)
+    n, L, pos, sp = system(0.05)
+    _, wide = evaluate(np.longdouble, pos, sp, L, pot, shift)
+    _, plain = evaluate(np.float64, pos, sp, L, pot, shift)
+    p = bbmd.ka_params(precision=prec, potential=pot, shift=shift, nbr_mode=mode)
+    sim = bbmd.Sim(p, n, L, sp, pos, np.zeros_like(pos))
+    _, u = sim.get_forces(energies=True)
+    assert rms(u, wide) <= 1.15 * rms(plain, wide)
     sim.close()
