@@ -511,12 +511,14 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
-// Sum of the lanes' kinetic energies k in units of 2^-32, rounded once.  Below 2^18 each (any
-// sane state): the lanes' values in units of 2^-40 (exact from 2^-17 up), summed as three limbs
-// by the warp's integer reduction -- the sum in FP64, which stands for the rest, takes the
-// FP64 pipe 8 x 16 clocks a chunk (forces at 16.4 M particles, 4 x 4 x 2: 2.95 -> 2.90 ms).
+// Sum of the lanes' kinetic energies k in units of 2^-32, rounded once.  Where every lane's is
+// zero or in [2^-17, 2^18): the lanes' values in units of 2^-40, which hold them exactly, summed
+// as three limbs by the warp's integer reduction.  Else (a system far colder than any liquid, or
+// flying apart) the sum in FP64, which takes the FP64 pipe 8 x 16 clocks a chunk (forces at
+// 16.4 M particles, 4 x 4 x 2: 2.95 -> 2.90 ms without it).
 __device__ __forceinline__ unsigned long long chunk_energy(float k) {
-    if (!__all_sync(FULL, k < 0x1p18f)) return __double2ull_rn(warp_sum_d((double)k) * 0x1p32);
+    const bool exact = k < 0x1p18f && (k >= 0x1p-17f || k == 0.f);
+    if (!__all_sync(FULL, exact)) return __double2ull_rn(warp_sum_d((double)k) * 0x1p32);
     const unsigned long long q = (unsigned long long)f32_to_i64(k * 0x1p40f);
     const unsigned s0 = __reduce_add_sync(FULL, (unsigned)q & 0x3ffffffu);
     const unsigned s1 = __reduce_add_sync(FULL, (unsigned)(q >> 26) & 0x3ffffffu);
