@@ -43,6 +43,7 @@ struct bbmd_sim {
     int sums_shape = 0;              // block shape of the FP64 energy passes
     int grid_shape = -1, grid_ctas = 0;  // one-launch step: block shape it was sized for, CTAs
     bool grid_wide = false;          // ... and whether with eight warps a CTA (shape 1)
+    bool no_trigger_sort = false;    // the device refused the captured step's cooperative node
     float shape_ms[4][2] = {};       // autotuner: per kShapes entry, force and list-build ms
 };
 
@@ -553,12 +554,26 @@ void finish_velocities(bbmd_sim* sim) {
     sim->pending = false;
 }
 
-bbmd_status build_graph(bbmd_sim* sim, int nh) {
-    cudaGraph_t g;
+// A cooperative launch can be refused where its CTAs are not resident at once (a device shared
+// by a limit on its SMs, say).  The launches per phase, which need no such thing, then take over,
+// for this call and those that follow on the handle.
+void keep_to_launches_per_phase(bbmd_sim* sim) {
+    cudaGetLastError();
+    sim->grid_ctas = 0;  // (until the next shape)
+}
+
+bool has_trigger_sort(const bbmd_sim* sim) {
+    return !sim->no_trigger_sort && sim->d.n <= kTriggerSortMax && cooperative(sim) &&
+           trigger_sort_ctas(sim->d, sim->nsm) > 0;
+}
+
+bbmd_status capture_step(bbmd_sim* sim, int nh, bool one_launch_sort) {
+    cudaGraph_t g = nullptr;
     CK(cudaStreamBeginCapture(sim->st, cudaStreamCaptureModeThreadLocal));
     launch_integrate(sim->d, sim->st);
-    const int grid = sim->d.n <= kTriggerSortMax ? trigger_sort_ctas(sim->d, sim->nsm) : 0;
-    if (grid > 0 && cooperative(sim) && launch_trigger_sort(sim->d, grid, sim->st) == cudaSuccess) {
+    cudaError_t refused = cudaSuccess;
+    if (one_launch_sort) {
+        refused = launch_trigger_sort(sim->d, trigger_sort_ctas(sim->d, sim->nsm), sim->st);
         launch_list_build(sim->d, sim->st);
     } else {
         launch_check(sim->d, sim->st);
@@ -567,10 +582,37 @@ bbmd_status build_graph(bbmd_sim* sim, int nh) {
     launch_force(sim->d, sim->st, false, nh != 0);
     launch_finalize(sim->d, sim->st, nh != 0);
     cudaError_t e = cudaStreamEndCapture(sim->st, &g);
+    if (refused != cudaSuccess) e = refused;
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&sim->graph[nh], g, 0);
+    if (e != cudaSuccess) sim->graph[nh] = nullptr;
+    if (g) cudaGraphDestroy(g);
     CK(e);
-    e = cudaGraphInstantiate(&sim->graph[nh], g, 0);
-    cudaGraphDestroy(g);
-    CK(e);
+    return BBMD_OK;
+}
+
+bbmd_status build_graph(bbmd_sim* sim, int nh) {
+    if (has_trigger_sort(sim)) {
+        if (capture_step(sim, nh, true) == BBMD_OK) return BBMD_OK;
+        cudaGetLastError();
+        sim->no_trigger_sort = true;
+    }
+    return capture_step(sim, nh, false);
+}
+
+// nsteps replays of the captured step.
+bbmd_status replay_steps(bbmd_sim* sim, int nh, int64_t nsteps) {
+    for (int64_t k = 0; k < nsteps; ++k) {
+        cudaError_t e = cudaGraphLaunch(sim->graph[nh], sim->st);
+        if (e != cudaSuccess && has_trigger_sort(sim)) {
+            cudaGetLastError();
+            sim->no_trigger_sort = true;
+            free_graphs(sim);
+            bbmd_status r = build_graph(sim, nh);
+            if (r != BBMD_OK) return r;
+            e = cudaGraphLaunch(sim->graph[nh], sim->st);
+        }
+        CK(e);
+    }
     return BBMD_OK;
 }
 
@@ -866,11 +908,20 @@ bbmd_status bbmd_step(bbmd_sim* sim, int64_t nsteps, double dt, const bbmd_therm
         if (cap != cudaStreamCaptureStatusNone) return fail(sim, BBMD_ERR_CUDA, "the stream is capturing");
         begin_call(sim, nsteps, dt, nh ? th : nullptr);
         LAUNCHED("begin");
-        for (int64_t k = 0; k < nsteps; k += kGridSteps) {
-            if (k > 0) launch_clear_grid_sync(sim->d, sim->st);
-            CK(launch_grid_step(sim->d, grid, sim->grid_wide, (int)std::min(kGridSteps, nsteps - k), nh != 0, sim->st));
+        int64_t done = 0;
+        for (; done < nsteps; done += kGridSteps) {
+            if (done > 0) launch_clear_grid_sync(sim->d, sim->st);
+            if (launch_grid_step(sim->d, grid, sim->grid_wide, (int)std::min(kGridSteps, nsteps - done), nh != 0,
+                                 sim->st) != cudaSuccess)
+                break;
         }
-        return BBMD_OK;
+        if (done >= nsteps) return BBMD_OK;
+        keep_to_launches_per_phase(sim);
+        if (!sim->graph[nh]) {
+            bbmd_status r = build_graph(sim, nh);
+            if (r != BBMD_OK) return r;
+        }
+        return replay_steps(sim, nh, nsteps - done);
     }
     if (!sim->graph[nh]) {
         bbmd_status r = build_graph(sim, nh);
@@ -878,8 +929,7 @@ bbmd_status bbmd_step(bbmd_sim* sim, int64_t nsteps, double dt, const bbmd_therm
     }
     begin_call(sim, nsteps, dt, nh ? th : nullptr);
     LAUNCHED("begin");
-    for (int64_t k = 0; k < nsteps; ++k) CK(cudaGraphLaunch(sim->graph[nh], sim->st));
-    return BBMD_OK;
+    return replay_steps(sim, nh, nsteps);
 }
 
 bbmd_status bbmd_observe(bbmd_sim* sim, uint32_t mask, const bbmd_obs_args* args, bbmd_obs* out) {
@@ -1000,17 +1050,21 @@ bbmd_status bbmd_minimize(bbmd_sim* sim, int64_t nsteps, double hmax, double dma
     finish_velocities(sim);
     bool one_wave = false;
     const int grid = sim->d.n <= kGridRelaxMax ? grid_step_grid(sim, &one_wave) : 0;
+    int64_t k = 0;
     if (grid > 0) {
-        int64_t k = 0;
+        cudaError_t e = cudaSuccess;
         do {
             launch_clear_grid_sync(sim->d, sim->st);
-            CK(launch_grid_relax(sim->d, grid, sim->grid_wide, (int)std::min(kGridSteps, nsteps - k), hmax, dmax, sim->st));
-            k += kGridSteps;
-        } while (k < nsteps);
-        LAUNCHED("minimize");
-        return read_status(sim);
+            e = launch_grid_relax(sim->d, grid, sim->grid_wide, (int)std::min(kGridSteps, nsteps - k), hmax, dmax, sim->st);
+            if (e == cudaSuccess) k += kGridSteps;
+        } while (e == cudaSuccess && k < nsteps);
+        if (e == cudaSuccess) {
+            LAUNCHED("minimize");
+            return read_status(sim);
+        }
+        keep_to_launches_per_phase(sim);
     }
-    for (int64_t k = 0; k < nsteps; ++k) {
+    for (; k < nsteps; ++k) {
         launch_force(sim->d, sim->st, false, false);
         launch_sd_step(sim->d, sim->st, hmax, dmax);
         enqueue_rebuild(sim);

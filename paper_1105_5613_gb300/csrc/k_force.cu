@@ -24,6 +24,7 @@
 // This file is compiled once per block shape, code BBMD_BLOCK_Z = 1, 2 or 4 (2 x 2 x Z
 // cells) or 8 (4 x 4 x 2 cells), into namespace bbmd::z<BBMD_BLOCK_Z>; the handle picks one
 // shape at creation.
+#include <climits>
 #include <cstddef>
 
 #include "bbmd_internal.cuh"
@@ -2259,12 +2260,19 @@ void launch_list_build(const DevSim& s, cudaStream_t st) {
 // CTAs of the one-launch step: enough for every block and for 256 particles a CTA, at most
 // what is resident at once.
 int grid_step_ctas(const DevSim& s, int nsm) {
-    int nb = 0;
     const size_t bytes = kStageBuffers * (size_t)(s.smax + 1) * sizeof(float4);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_step_grid<true, true>, kBW * 32, bytes) !=
-        cudaSuccess) {
-        cudaGetLastError();
-        return 0;
+    // (every form that may be launched with the grid: their static shared memory differs)
+    const void* forms[] = {(const void*)k_step_grid<false, false>, (const void*)k_step_grid<false, true>,
+                           (const void*)k_step_grid<true, false>, (const void*)k_step_grid<true, true>,
+                           (const void*)k_relax_grid<false>, (const void*)k_relax_grid<true>};
+    int nb = INT_MAX;
+    for (const void* f : forms) {
+        int one = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&one, f, kBW * 32, bytes) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        nb = one < nb ? one : nb;
     }
     int64_t want = (s.n + 255) / 256;
     if (want < s.nblocks) want = s.nblocks;
