@@ -716,7 +716,7 @@ bbmd_status bbmd_create(const bbmd_params* params, int64_t n, const double box[3
                      std::ldexp((double)D.D[2], -D.kexp);
     double mean = (double)n / V * cellvol;
     for (int d = 0; d < 3; ++d) D.halfL[d] = (float)(0.5 * box[d]);
-    if (!prepare_force_kernels()) {
+    if (!prepare_force_kernels() || !prepare_gr_kernels()) {
         cudaGetLastError();
         std::fprintf(stderr, "bbmd_create: could not configure kernel shared memory\n");
         bbmd_destroy(sim);
@@ -938,7 +938,7 @@ bbmd_status bbmd_observe(bbmd_sim* sim, uint32_t mask, const bbmd_obs_args* args
     int nbins = args && args->nbins > 0 ? args->nbins : 500;
     double rmax = args && args->rmax > 0.0 ? args->rmax : 5.0;
     double kv = args && args->k > 0.0 ? args->k : 7.25;
-    if (nbins > 4096) return fail(sim, BBMD_ERR_ARG, "nbins <= 4096");
+    if (nbins > kGrMaxBins) return fail(sim, BBMD_ERR_ARG, "nbins <= 4096");
     DevSim& D = sim->d;
     // kinetic energy and momentum
     const bool energy = (mask & (BBMD_OBS_ENERGY | BBMD_OBS_VIRIAL)) != 0;
@@ -1828,6 +1828,7 @@ namespace {
 
 constexpr int64_t kNoAllocInts = BBMD_NOALLOC_GR_SCRATCH_INTS;
 constexpr int kNoAllocBins = BBMD_NOALLOC_GR_MAX_BINS;
+static_assert(kNoAllocBins <= kGrMaxBins, "shared memory of the g(r) kernels");
 constexpr int kNoAllocDevices = 64;
 
 struct NoAllocSlot {

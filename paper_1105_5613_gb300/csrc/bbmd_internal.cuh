@@ -450,6 +450,9 @@ void launch_clear_grid_sync(const DevSim& s, cudaStream_t st);
 void launch_set_ref(const DevSim& s, cudaStream_t st, double* ref);
 void launch_msd_fs(const DevSim& s, cudaStream_t st, const double* ref, double kvec,
                    double* out_dev);
+constexpr int kGrMaxBins = 4096;  // bins of a g(r) call at most
+// one-time kernel attributes of launch_gr (at creation, outside any stream capture)
+bool prepare_gr_kernels();
 int launch_gr(const DevSim& s, cudaStream_t st, int nbins, double rmax,
               unsigned long long* counts_dev, int32_t* scratch_i32, float4* scratch_f4,
               int64_t scratch_n);

@@ -495,6 +495,23 @@ bool gr_rows(const DevSim& s, int nbins, double rmax, GrRows& g) {
 
 }  // namespace
 
+namespace {
+
+size_t gr_rows_bytes(int nbins) { return kRowWarps * sizeof(RowRing) + (size_t)3 * nbins * sizeof(unsigned); }
+size_t gr_bytes(int nbins) { return kChunk * sizeof(JEnt) + (size_t)4 * nbins * sizeof(unsigned); }
+
+}  // namespace
+
+// Every kernel is opted into the shared memory of the most bins once and for all: set to each
+// call's own need, the limit could be lowered by another thread's call between this one's set
+// and its launch.
+bool prepare_gr_kernels() {
+    const cudaFuncAttribute most = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    return cudaFuncSetAttribute(k_gr_rows, most, (int)gr_rows_bytes(kGrMaxBins)) == cudaSuccess &&
+           cudaFuncSetAttribute(k_gr_all, most, (int)gr_bytes(kGrMaxBins)) == cudaSuccess &&
+           cudaFuncSetAttribute(k_gr_cells, most, (int)gr_bytes(kGrMaxBins)) == cudaSuccess;
+}
+
 // scratch_i32: 2 n + 3 (ncells + 1) ints.  Returns 0, or -1 if scratch is too small.
 int launch_gr(const DevSim& s, cudaStream_t st, int nbins, double rmax,
               unsigned long long* counts_dev, int32_t* scratch_i32, float4* /*scratch_f4*/,
@@ -514,7 +531,7 @@ int launch_gr(const DevSim& s, cudaStream_t st, int nbins, double rmax,
         g.Dg[d] = s.Lfix[d] / g.ncg[d];
         g.ncells *= g.ncg[d];
     }
-    size_t smem = kChunk * sizeof(JEnt) + (size_t)4 * nbins * sizeof(unsigned);
+    const size_t smem = gr_bytes(nbins);
     cudaMemsetAsync(counts_dev, 0, sizeof(unsigned long long) * 4 * nbins, st);
     if (cells && scratch_n < 2 * s.n + 3 * ((int64_t)g.ncells + 1)) return -1;
     GrRows rows;
@@ -522,15 +539,12 @@ int launch_gr(const DevSim& s, cudaStream_t st, int nbins, double rmax,
         int dev = 0, nsm = 1;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        const size_t bytes = kRowWarps * sizeof(RowRing) + (size_t)3 * nbins * sizeof(unsigned);
-        cudaFuncSetAttribute(k_gr_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         const int64_t want = (rows.ntiles + kRowWarps - 1) / kRowWarps;
         const int grid = (int)(want < (int64_t)nsm * 3 ? want : (int64_t)nsm * 3);  // all resident
-        k_gr_rows<<<grid, kRowWarps * 32, bytes, st>>>(s, g, rows, counts_dev);
+        k_gr_rows<<<grid, kRowWarps * 32, gr_rows_bytes(nbins), st>>>(s, g, rows, counts_dev);
         return 0;
     }
     if (!cells) {
-        cudaFuncSetAttribute(k_gr_all, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         int nblk = (int)((s.n + kT - 1) / kT);
         k_gr_all<<<nblk, kT, smem, st>>>(s, g, counts_dev);
         return 0;
@@ -544,7 +558,6 @@ int launch_gr(const DevSim& s, cudaStream_t st, int nbins, double rmax,
     k_gr_key<<<s.grid_part, 256, 0, st>>>(s, g);
     k_gr_scan<<<1, 1024, 0, st>>>(g);
     k_gr_scatter<<<s.grid_part, 256, 0, st>>>(s, g);
-    cudaFuncSetAttribute(k_gr_cells, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int nblk = g.ncells < 65535 * 4 ? g.ncells : 65535 * 4;
     k_gr_cells<<<nblk, kT, smem, st>>>(s, g, counts_dev);
     return 0;
