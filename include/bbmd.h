@@ -380,11 +380,13 @@ const char* bbmd_batch_last_error(const bbmd_batch* b);
  * library variant of the g(r) observable for callers that must not allocate.
  *   nbins <= 0 -> 500, rmax <= 0 -> 5.0 (as bbmd_observe); nbins <= 4096.
  *   Scratch: one fixed device array inside the library, BBMD_NOALLOC_GR_SCRATCH_INTS int32
- *   entries plus 4*4096 counters.  When the box holds at least 3 cells of side rmax per
- *   axis, the coarse-grid search needs 2n + 3(ncg + 1) entries (ncg = number of those
- *   cells); a larger need is rejected with BBMD_ERR_ARG before anything is launched (use
- *   bbmd_observe then).  Smaller boxes take the all-pairs path, which needs no int32
- *   scratch.
+ *   entries plus 4*4096 counters.  Pairs are searched over the cells of the last rebuild where
+ *   these reach rmax (2 R + 1 of them fit each axis, R cells to each side), else on a coarse grid
+ *   where the box holds at least 3 cells of side rmax per axis, else by all pairs.  Only the
+ *   coarse grid takes int32 scratch, 2n + 3(ncg + 1) entries (ncg = number of its cells).  A box
+ *   with at least 3 cells of side rmax per axis whose coarse grid would need more than the array
+ *   is rejected with BBMD_ERR_ARG before anything is launched, whichever search would serve
+ *   it (use bbmd_observe then).
  *   Nothing has to start at zero: each call clears the counters and the coarse-cell counts
  *   it uses before filling them.
  *   The first call on a device looks up the array's address (cudaGetSymbolAddress); make

@@ -966,18 +966,13 @@ bbmd_status bbmd_observe(bbmd_sim* sim, uint32_t mask, const bbmd_obs_args* args
             sim->gr_counts = (unsigned long long*)dev_alloc(sim, (size_t)4 * nbins * 8);
             sim->gr_nbins = nbins;
         }
-        int64_t ncg = 1;
-        for (int d = 0; d < 3; ++d) {
-            int m = (int)std::floor(sim->box[d] / rmax);
-            ncg *= m < 1 ? 1 : m;
-        }
-        int64_t need = 2 * D.n + 3 * (ncg + 1);
+        const int64_t need = gr_scratch_ints(D, nbins, rmax);
         if (sim->gr_scratch_n < need) {
             dev_free(sim, sim->gr_scratch);
             sim->gr_scratch = (int32_t*)dev_alloc(sim, (size_t)need * 4);
             sim->gr_scratch_n = sim->gr_scratch ? need : 0;
         }
-        if (!sim->gr_counts || !sim->gr_scratch) return fail(sim, BBMD_ERR_OOM, "g(r) scratch");
+        if (!sim->gr_counts || sim->gr_scratch_n < need) return fail(sim, BBMD_ERR_OOM, "g(r) scratch");
         if (launch_gr(D, sim->st, nbins, rmax, sim->gr_counts, sim->gr_scratch, nullptr,
                       sim->gr_scratch_n) != 0)
             return fail(sim, BBMD_ERR_STATE, "g(r) scratch too small");
@@ -1859,7 +1854,7 @@ extern "C" bbmd_status bbmd_gr_counts_noalloc(bbmd_sim* sim, int32_t nbins, doub
     if (!(rmax > 0.0)) rmax = 5.0;
     if (nbins > kNoAllocBins) return fail(sim, BBMD_ERR_ARG, "nbins <= 4096");
     const DevSim& D = sim->d;
-    // the scratch the coarse-grid path of launch_gr will ask for (same rule as launch_gr)
+    // the scratch a coarse grid takes, asked for whichever search serves (bbmd.h)
     bool cells = true;
     int64_t ncg = 1;
     for (int d = 0; d < 3; ++d) {

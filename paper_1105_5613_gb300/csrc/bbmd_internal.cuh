@@ -453,6 +453,9 @@ void launch_msd_fs(const DevSim& s, cudaStream_t st, const double* ref, double k
 constexpr int kGrMaxBins = 4096;  // bins of a g(r) call at most
 // one-time kernel attributes of launch_gr (at creation, outside any stream capture)
 bool prepare_gr_kernels();
+// int32 scratch that the search of launch_gr takes for these bins: none over the build cells or by
+// all pairs
+int64_t gr_scratch_ints(const DevSim& s, int nbins, double rmax);
 int launch_gr(const DevSim& s, cudaStream_t st, int nbins, double rmax,
               unsigned long long* counts_dev, int32_t* scratch_i32, float4* scratch_f4,
               int64_t scratch_n);

@@ -512,7 +512,34 @@ bool prepare_gr_kernels() {
            cudaFuncSetAttribute(k_gr_cells, most, (int)gr_bytes(kGrMaxBins)) == cudaSuccess;
 }
 
-// scratch_i32: 2 n + 3 (ncells + 1) ints.  Returns 0, or -1 if scratch is too small.
+namespace {
+
+// Coarse cells of side >= rmax; false if the box holds fewer than three of them on an axis.
+bool gr_coarse(const DevSim& s, double rmax, GrArgs& g) {
+    bool cells = true;
+    int64_t n = 1;
+    for (int d = 0; d < 3; ++d) {
+        double L = ldexp((double)s.Lfix[d], -s.kexp);
+        int m = (int)floor(L / rmax);
+        if (m < 3) cells = false;
+        g.ncg[d] = m < 1 ? 1 : m;
+        g.Dg[d] = s.Lfix[d] / g.ncg[d];
+        n *= g.ncg[d];
+    }
+    g.ncells = (int)n;
+    return cells;
+}
+
+}  // namespace
+
+int64_t gr_scratch_ints(const DevSim& s, int nbins, double rmax) {
+    GrRows rows;
+    GrArgs g;
+    if (gr_rows(s, nbins, rmax, rows) || !gr_coarse(s, rmax, g)) return 0;
+    return 2 * s.n + 3 * ((int64_t)g.ncg[0] * g.ncg[1] * g.ncg[2] + 1);
+}
+
+// Returns 0, or -1 if scratch is too small (gr_scratch_ints).
 int launch_gr(const DevSim& s, cudaStream_t st, int nbins, double rmax,
               unsigned long long* counts_dev, int32_t* scratch_i32, float4* /*scratch_f4*/,
               int64_t scratch_n) {
@@ -521,19 +548,10 @@ int launch_gr(const DevSim& s, cudaStream_t st, int nbins, double rmax,
     g.dr = rmax / (double)nbins;
     g.inv_dr = (float)(1.0 / g.dr);
     g.rmax2_hi = (float)(rmax * rmax * 1.001);
-    bool cells = true;
-    g.ncells = 1;
-    for (int d = 0; d < 3; ++d) {
-        double L = ldexp((double)s.Lfix[d], -s.kexp);
-        int m = (int)floor(L / rmax);
-        if (m < 3) cells = false;
-        g.ncg[d] = m < 1 ? 1 : m;
-        g.Dg[d] = s.Lfix[d] / g.ncg[d];
-        g.ncells *= g.ncg[d];
-    }
+    const bool cells = gr_coarse(s, rmax, g);
+    if (scratch_n < gr_scratch_ints(s, nbins, rmax)) return -1;
     const size_t smem = gr_bytes(nbins);
     cudaMemsetAsync(counts_dev, 0, sizeof(unsigned long long) * 4 * nbins, st);
-    if (cells && scratch_n < 2 * s.n + 3 * ((int64_t)g.ncells + 1)) return -1;
     GrRows rows;
     if (gr_rows(s, nbins, rmax, rows)) {
         int dev = 0, nsm = 1;

@@ -29,6 +29,7 @@ void launch_finalize_many(const ManySims&, int, bool, cudaStream_t) {}
 void launch_finish(const DevSim&, cudaStream_t) {}
 void launch_forces_of_ids(const DevSim&, cudaStream_t, const int32_t*, const int64_t*, int64_t, double*, double*) {}
 bool prepare_gr_kernels() { return true; }
+int64_t gr_scratch_ints(const DevSim&, int, double) { return 0; }
 int launch_gr(const DevSim&, cudaStream_t, int, double, unsigned long long*, int32_t*, float4*, int64_t) { return 0; }
 void launch_init_fcc(const DevSim&, cudaStream_t, int, double, uint64_t) {}
 void launch_init_mb(const DevSim&, cudaStream_t, double, uint64_t, double*, double*) {}

@@ -6,8 +6,9 @@
 
 extern "C" int gr_prepare() { return bbmd::prepare_gr_kernels() ? 0 : 1; }
 
-// g(r) of a box of side L in nc cells a side; 0, or launch_gr's refusal.
-extern "C" int gr_call(double L, int nc, int nbins, double rmax) {
+// g(r) of a box of side L in nc cells a side, with scratch_n entries of scratch; 0, or launch_gr's
+// refusal.
+extern "C" int gr_call(double L, int nc, int nbins, double rmax, int64_t scratch_n) {
     bbmd::DevSim s = {};
     static int32_t scratch[1 << 20];
     static unsigned long long counts[4 * bbmd::kGrMaxBins];
@@ -21,5 +22,5 @@ extern "C" int gr_call(double L, int nc, int nbins, double rmax) {
     s.ncell = nc * nc * nc;
     s.disp_thr = s.disp_far = 0.3f;
     s.grid_part = 4;
-    return bbmd::launch_gr(s, nullptr, nbins, rmax, counts, scratch, nullptr, 1 << 20);
+    return bbmd::launch_gr(s, nullptr, nbins, rmax, counts, scratch, nullptr, scratch_n);
 }
