@@ -396,6 +396,11 @@ const char* bbmd_batch_last_error(const bbmd_batch* b);
  * Synchronising. */
 bbmd_status bbmd_gr_counts_noalloc(bbmd_sim* sim, int32_t nbins, double rmax, uint64_t* counts);
 
+/* Kernels that bbmd_step has launched on this handle since its creation (those of graph
+ * replays included; a gated kernel that returns at once counts).  The paper has no
+ * counterpart. */
+int64_t bbmd_step_launches(const bbmd_sim* sim);
+
 /* Limits of the device's waits in the launches of this handle.  barrier_ns (default 2e9, at
  * least 1, else BBMD_ERR_ARG): a wait at the grid-wide barrier of the launches that run several
  * phases (the steps and descents of small systems, the rebuild trigger and sort).

@@ -91,7 +91,7 @@ EXPORTS = ["bbmd_create", "bbmd_destroy", "bbmd_step", "bbmd_step_profiled", "bb
            "bbmd_get_neighbors", "bbmd_rebuild", "bbmd_get_info", "bbmd_last_error",
            "bbmd_gr_counts_noalloc", "bbmd_tune", "bbmd_get_forces_ids", "bbmd_create_batch", "bbmd_step_batch",
            "bbmd_batch_replica", "bbmd_batch_size", "bbmd_batch_set_branches",
-           "bbmd_batch_set_mode", "bbmd_batch_set_wait_limit", "bbmd_set_wait_limits",
+           "bbmd_batch_set_mode", "bbmd_batch_set_wait_limit", "bbmd_set_wait_limits", "bbmd_step_launches",
            "bbmd_batch_uses_persistent", "bbmd_destroy_batch",
            "bbmd_batch_last_error", "bbmd_fma_peak", "bbmd_smem_scatter_rate"]
 
@@ -156,6 +156,8 @@ def load(path: str | None = None):
     L.bbmd_batch_set_branches.restype = C.c_int
     L.bbmd_batch_set_mode.argtypes = [vp, C.c_int32]
     L.bbmd_batch_set_mode.restype = C.c_int
+    L.bbmd_step_launches.argtypes = [vp]
+    L.bbmd_step_launches.restype = i64
     L.bbmd_set_wait_limits.argtypes = [vp, C.c_uint64, C.c_uint32]
     L.bbmd_set_wait_limits.restype = C.c_int
     L.bbmd_batch_set_wait_limit.argtypes = [vp, C.c_uint64]
@@ -409,6 +411,10 @@ class Sim:
 
     def rebuild(self):
         _check(self.h, load().bbmd_rebuild(self.h))
+
+    def step_launches(self):
+        """Kernels launched by step() so far (bbmd_step_launches)."""
+        return int(load().bbmd_step_launches(self.h))
 
     def set_wait_limits(self, barrier_ns=2_000_000_000, staging_tries=1 << 18):
         """Limits of the device's waits: ns at a grid-wide barrier, looks for staged copies

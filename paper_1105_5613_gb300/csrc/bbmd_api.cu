@@ -43,6 +43,8 @@ struct bbmd_sim {
     int sums_shape = 0;              // block shape of the FP64 energy passes
     int grid_shape = -1, grid_ctas = 0;  // one-launch step: block shape it was sized for, CTAs
     bool grid_wide = false;          // ... and whether with eight warps a CTA (shape 1)
+    int64_t graph_kernels[2] = {0, 0};  // kernels of a replay of graph[]
+    int64_t launched = 0;            // kernels launched by bbmd_step
     bool no_trigger_sort = false;    // the device refused the captured step's cooperative node
     float shape_ms[4][2] = {};       // autotuner: per kShapes entry, force and list-build ms
 };
@@ -584,9 +586,12 @@ bbmd_status capture_step(bbmd_sim* sim, int nh, bool one_launch_sort) {
     cudaError_t e = cudaStreamEndCapture(sim->st, &g);
     if (refused != cudaSuccess) e = refused;
     if (e == cudaSuccess) e = cudaGraphInstantiate(&sim->graph[nh], g, 0);
+    size_t nodes = 0;
+    if (e == cudaSuccess) e = cudaGraphGetNodes(g, nullptr, &nodes);  // (kernels, all of them)
     if (e != cudaSuccess) sim->graph[nh] = nullptr;
     if (g) cudaGraphDestroy(g);
     CK(e);
+    sim->graph_kernels[nh] = (int64_t)nodes;
     return BBMD_OK;
 }
 
@@ -612,6 +617,7 @@ bbmd_status replay_steps(bbmd_sim* sim, int nh, int64_t nsteps) {
             e = cudaGraphLaunch(sim->graph[nh], sim->st);
         }
         CK(e);
+        sim->launched += sim->graph_kernels[nh];
     }
     return BBMD_OK;
 }
@@ -899,6 +905,7 @@ bbmd_status bbmd_step(bbmd_sim* sim, int64_t nsteps, double dt, const bbmd_therm
         }
     }
     if (nsteps == 0) return BBMD_OK;
+    const int64_t begin_kernels = dt != sim->last_dt && sim->pending ? 3 : 1;  // (finish: two)
     bool one_wave = false;
     const int grid = grid_step_grid(sim, &one_wave);
     if (grid > 0 && one_wave) {
@@ -908,12 +915,15 @@ bbmd_status bbmd_step(bbmd_sim* sim, int64_t nsteps, double dt, const bbmd_therm
         if (cap != cudaStreamCaptureStatusNone) return fail(sim, BBMD_ERR_CUDA, "the stream is capturing");
         begin_call(sim, nsteps, dt, nh ? th : nullptr);
         LAUNCHED("begin");
+        sim->launched += begin_kernels;
         int64_t done = 0;
         for (; done < nsteps; done += kGridSteps) {
             if (done > 0) launch_clear_grid_sync(sim->d, sim->st);
+            sim->launched += done > 0;
             if (launch_grid_step(sim->d, grid, sim->grid_wide, (int)std::min(kGridSteps, nsteps - done), nh != 0,
                                  sim->st) != cudaSuccess)
                 break;
+            ++sim->launched;
         }
         if (done >= nsteps) return BBMD_OK;
         keep_to_launches_per_phase(sim);
@@ -929,6 +939,7 @@ bbmd_status bbmd_step(bbmd_sim* sim, int64_t nsteps, double dt, const bbmd_therm
     }
     begin_call(sim, nsteps, dt, nh ? th : nullptr);
     LAUNCHED("begin");
+    sim->launched += begin_kernels;
     return replay_steps(sim, nh, nsteps);
 }
 
@@ -1320,6 +1331,8 @@ bbmd_status bbmd_get_info(const bbmd_sim* sim, bbmd_info* info) {
     info->device_bytes = sim->bytes;
     return BBMD_OK;
 }
+
+int64_t bbmd_step_launches(const bbmd_sim* sim) { return sim ? sim->launched : 0; }
 
 const char* bbmd_last_error(const bbmd_sim* sim) { return sim ? sim->err.c_str() : ""; }
 

@@ -58,6 +58,7 @@ cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t* g) {
     *g = (cudaGraph_t)&fake;
     return cudaSuccess;
 }
+cudaError_t cudaGraphGetNodes(cudaGraph_t, cudaGraphNode_t*, size_t* n) { return *n = 6, cudaSuccess; }
 cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
 cudaError_t cudaGraphInstantiate(cudaGraphExec_t* x, cudaGraph_t, unsigned long long) {
     if (fake.captured_sort && (fake.refuse & 4)) return cudaErrorCooperativeLaunchTooLarge;

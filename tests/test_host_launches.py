@@ -42,6 +42,8 @@ def lib(tmp_path_factory):
     L.bbmd_step.argtypes = [C.c_void_p, C.c_int64, C.c_double, C.c_void_p]
     L.bbmd_minimize.argtypes = [C.c_void_p, C.c_int64, C.c_double, C.c_double]
     L.bbmd_destroy.argtypes = [C.c_void_p]
+    L.bbmd_step_launches.argtypes = [C.c_void_p]
+    L.bbmd_step_launches.restype = C.c_int64
     return L
 
 
@@ -116,3 +118,19 @@ def test_nothing_refused(lib, handle):
     assert (c.grid_step, c.grid_relax, c.graph_launch, c.steps) == (2, 1, 0, 1530)
     assert lib.bbmd_step(g, 9, 0.005, None) == 0
     assert counts(lib).graph_launch == 9 and counts(lib).trigger_sort == 1
+
+
+def test_launches_are_counted(lib, handle):
+    h, g = handle(10, 1), handle(36, 1)
+    lib.fake_reset(0, 0)
+    assert lib.bbmd_step_launches(h) == 0
+    assert lib.bbmd_step(h, 2500, 0.005, None) == 0
+    assert lib.bbmd_step_launches(h) == 1 + 3 + 2  # begin, launches of 1024, barriers cleared between
+    assert lib.bbmd_step(h, 3, 0.002, None) == 0
+    assert lib.bbmd_step_launches(h) == 6 + 2 + 1 + 1  # another dt: the pending update first
+    assert lib.bbmd_step(g, 9, 0.005, None) == 0
+    assert lib.bbmd_step_launches(g) == 1 + 9 * 6  # (the fake's graphs have six nodes)
+    lib.fake_reset(1, 1)
+    h = handle(10, 1)
+    assert lib.bbmd_step(h, 1030, 0.005, None) == 0
+    assert lib.bbmd_step_launches(h) == 1 + 1 + 1 + 6 * 6  # begin, 1024 steps, cleared, the rest replayed
