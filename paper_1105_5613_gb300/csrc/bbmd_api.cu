@@ -705,8 +705,6 @@ bbmd_status bbmd_create(const bbmd_params* params, int64_t n, const double box[3
     D.wait_ns = kBarrierWaitNs;
     D.stage_tries = kStageTries;
     fill_pair_table(*params, D.pt);
-    for (int k = 0; k < 4; ++k)
-        D.pt.rcfix[k] = (long long)std::ceil(std::ldexp(D.pt.drc[k], D.kexp));
     double half = 0.5 * params->skin;
     D.disp2 = (float)(half * half * (1.0 - 1e-4));
     D.disp_thr = (float)(params->skin * (1.0 - 1e-4));

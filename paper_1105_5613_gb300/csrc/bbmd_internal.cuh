@@ -7,7 +7,7 @@
 //   id[npad]     int32   particle id;  sp[npad] uint8 species
 //   rel[npad]    float4  position relative to the frame of its build cell, w = species (0.f / 1.f)
 //   relb[npad]   float4  the same at the last rebuild, w = (cell << 1) | species
-//   F[npad]      float4  mixed-precision force (w = per-particle energy on energy passes)
+//   F[npad]      float4  force in FP32 (w = 0)
 //   Fd[3][npad]  double  FP64-form force
 //   list[lcap8][npad][8] uint16  Verlet list: offsets into the staged region (the cells
 //                                 around the particle's block of cells)
@@ -101,7 +101,6 @@ struct PairTab {
     float sig2[4], sig2lo[4], eps48[4], eps4[4], vshift[4], fcut[4], frc[4];
     // FP64 tables: exact decisions and the FP64 form
     double rc2[4], R2[4], dsig2[4], deps48[4], deps4[4], dvshift[4], dfcut[4], drc[4];
-    long long rcfix[4];           // ceil(rcut * 2^k): |dx| beyond it on some axis -> no pair
     float mass[2];
     double dmass[2];
     int potential, shift;
@@ -136,7 +135,7 @@ struct alignas(16) DevSim {
     int32_t *key, *cell_start, *count, *rank, *perm, *scan_part;
     uint16_t* list;
     uint16_t* rows;          // per particle: rows (8 entries each) of its Verlet list
-    double* partials;        // [kMaxPartials][4]
+    double* partials;        // [8][kMaxPartials]
     DevScalars* sc;
     uint32_t* gsync;         // grid-wide barrier of the one-launch step (kSyncWords words)
     uint64_t wait_ns;        // limit of a wait at it

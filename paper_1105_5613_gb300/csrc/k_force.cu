@@ -1,10 +1,11 @@
 // Pair forces of the truncated Lennard-Jones / soft-sphere mixture (Sec. 2.1, Eqs. lj0,
 // sc0, mod0) over the cell stencil (Sec. 2.2), and the Verlet-list build.
 //
-// Work unit: one CTA of 8 warps per 2x2x2 block of cells; warp w owns one cell of the block
-// (its "tile": up to 32 particles at a time, larger cells in chunks of 32).  The CTA stages
-// the 4x4x4 cells around the block -- the union of the eight 27-cell stencils -- into
-// shared memory as float4 {x, y, z, species} in one frame (the block's centre).  The raw
+// Work unit: one CTA per block of cells; its warps take the block's items in turn (list-mode
+// forces: chunks of 32 own particles of one species across the block's cells; stencil forces:
+// cells; list build: a cell's first 32 particles, and the rest).  The CTA stages the cells of the
+// block and one cell around it -- the union of their 27-cell stencils -- into shared memory
+// as float4 {x, y, z, species} in one frame (the block's centre).  The raw
 // frame-relative records of each cell arrive by one TMA bulk copy per cell (cells are
 // contiguous after the counting sort); the exact frame offsets are then added in shared
 // memory.  Each lane owns one particle i and accumulates its force in registers: a full
@@ -1420,7 +1421,7 @@ __device__ __forceinline__ bool list_build_body(const DevSim& s, int lb, int lg)
 // index and count where a sum depends on it, so the states are the same bit for bit), and
 // the phases are kept apart by a grid-wide barrier (about 1.3 us) only where one is needed:
 // two in a step in which nothing came near the rebuild trigger, two more for the trigger,
-// seven more for a rebuild.  Where it is used and what it measured: grid_step_grid
+// six or seven more for a rebuild.  Where it is used and what it measured: grid_step_grid
 // (bbmd_api.cu).  At 4000 particles (2 x 2 x 1 blocks, one per SM, four warps) a step's 41 us
 // were forces 14 (two rounds of chunks), barriers 6, finalize 6, integrate 2, and 0.2 rebuilds
 // of 70 (its list build 45, two rounds for a cell of more than 32).
