@@ -1221,10 +1221,11 @@ __device__ __forceinline__ bool list_build_body(const DevSim& s, int lb, int lg)
     if (threadIdx.x == 0) ss.next_cell[0] = ss.next_cell[1] = 0;
     int blk_it = 0;  // blocks of this CTA so far (the parity selects the cell counter)
     const float far = kFar;
+    uint16_t* buf = nullptr;
+    if constexpr (BUFFER) buf = entry_buffer(ss, 0, w, lane);
     return for_each_block(s, lb, lg, smem, s.smax + 1, R, mbar,
                           [&](const BlockPos& bp, const Region& Rc, const float4* sm, int b) {
-        uint16_t* buf = nullptr;
-        if constexpr (BUFFER) buf = entry_buffer(ss, b, w, lane);
+        if constexpr (BUFFER && kStageBuffers > 1) buf = entry_buffer(ss, b, w, lane);
         const int par = blk_it & 1;
         if (threadIdx.x == 0) ss.next_cell[par ^ 1] = 0;  // for the next block
         ++blk_it;
