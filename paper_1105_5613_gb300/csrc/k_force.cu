@@ -1641,7 +1641,7 @@ __global__ void __launch_bounds__(kBW * 32, 2) k_step_persistent(PersistentStep 
 //   - sums over the system (energy, virial) take each pair from one side only.
 // Measured against the form that ran the FP64 arithmetic for every candidate some lane of
 // the warp interacts with: energy and virial sums at 16.4 M particles (lists, skin 0.4)
-// 132 -> 23 ms, at 4 M in cell mode 121 -> 8.6 ms; forces of the FP64 form at 108 000
+// 132 -> 24 ms, at 4 M in cell mode 121 -> 8.6 ms; forces of the FP64 form at 108 000
 // 0.868 -> 0.347 ms.  (At 0.63e12 lanes a second the pairs' operations take 11, 2.7 and 0.19 ms.
 // Every shape measures the same at 2 M; converting the integers with two additions instead of
 // a conversion instruction was 15 % slower.)

@@ -250,9 +250,11 @@ __global__ void __launch_bounds__(kT) k_gr_all(DevSim s, GrArgs g, unsigned long
 // (rows after the lane's own, and later particles of its own row) and counted for both
 // orders when the CTA's histogram is added to the result.
 //
-// Bound: issue.  About 1000 ring entries and 310 binned pairs a particle at rmax = 5, against
-// 5700 candidates in 64-bit arithmetic on the coarse grid: 108 000 particles, 500 bins, 4.2 ->
-// 0.40 ms (0.51 when each ring word's pairs were binned on their own, chunks within cells).
+// Bound: dependent instructions (57 % of the issue slots; the waits between them, shared-memory
+// reads and the square roots the rest) of about 1000 ring entries and 310 binned
+// pairs a particle at rmax = 5, against 5700 candidates in 64-bit arithmetic on the coarse grid:
+// 108 000 particles, 500 bins, 4.2 -> 0.40 ms (0.51 when each ring word's pairs were binned on
+// their own, chunks within cells).
 
 constexpr int kRowWarps = 8;
 constexpr int kRowRing = 64;
