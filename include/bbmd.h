@@ -404,8 +404,9 @@ int64_t bbmd_step_launches(const bbmd_sim* sim);
 /* Limits of the device's waits in the launches of this handle.  barrier_ns (default 2e9, at
  * least 1, else BBMD_ERR_ARG): a wait at the grid-wide barrier of the launches that run several
  * phases (the steps and descents of small systems, the rebuild trigger and sort).
- * staging_tries (default 2^18): looks for the copies of a block into shared memory; with 0 the
- * first wait gives up at once (its copies are still waited for).  A wait that runs out ends its
+ * staging_tries (default 2^18): looks for the copies of a block into shared memory, in the same
+ * launches and those of the persistent batch step; with 0 the first wait gives up at once (its
+ * copies are still waited for).  A wait that runs out ends its
  * launch, later launches of several phases return at once, and every synchronising call from
  * then on returns BBMD_ERR_TIMEOUT.  The state is then that of a step half done (destroy the
  * handle); the device context stays usable.  The waits between the phases of a replica batch

@@ -761,7 +761,10 @@ bbmd_status bbmd_create(const bbmd_params* params, int64_t n, const double box[3
         if (!p) ok = false;
         return p;
     };
-    D.x = (uint64_t*)A(3 * np * 8);
+    // (and as many positions more as a region stages: staged_particle)
+    int smax = 0;
+    for (int bz : sim->shapes) smax = std::max(smax, shape_smax(sim, bz));
+    D.x = (uint64_t*)A((3 * np + smax + 64) * 8);
     D.v = (int64_t*)A(3 * np * 8);
     D.img = (int32_t*)A(3 * np * 4);
     D.id = (int32_t*)A(np * 4);

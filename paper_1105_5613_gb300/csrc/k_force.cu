@@ -177,10 +177,12 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* mbar, uint32_t parity) {
     return ok != 0;
 }
 
-// Wait for the current phase, s.stage_tries tries at most.  On expiry raise ST_TIMEOUT, wait
-// once more (again bounded) for the copies still in flight, and return false.
+// Wait for the current phase, kStageTries tries at most (LIMIT: s.stage_tries).  On expiry raise
+// ST_TIMEOUT, wait once more (again bounded) for the copies still in flight, and return false.
+template <bool LIMIT>
 __device__ __forceinline__ bool mbar_wait_bounded(const DevSim& s, uint64_t* mbar, uint32_t parity) {
-    for (uint32_t it = 0; it < s.stage_tries; ++it)
+    const uint32_t tries = LIMIT ? s.stage_tries : kStageTries;
+    for (uint32_t it = 0; it < tries; ++it)
         if (mbar_try_wait(mbar, parity)) return true;
     set_status(s, ST_TIMEOUT);
     for (uint32_t it = 0; it < kStageTries; ++it)
@@ -290,9 +292,10 @@ __device__ void issue_block(const DevSim& s, const BlockPos& b, Region& R, float
 // Wait for the copies of a block issued with issue_block, add the frame offsets of every
 // region cell (exact residual first), write the sentinel sm[smax] and synchronise.
 // Returns false on every thread of the CTA if some thread's wait gave up.
+template <bool LIMIT>
 __device__ bool finish_block(const DevSim& s, const Region& R, float4* sm, uint64_t* mbar,
                              uint32_t parity) {
-    const bool ok = mbar_wait_bounded(s, mbar, parity);
+    const bool ok = mbar_wait_bounded<LIMIT>(s, mbar, parity);
     if (__syncthreads_or(!ok)) return false;
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     for (int q = w; q < kRegion; q += kBW) {
@@ -317,6 +320,10 @@ __device__ bool finish_block(const DevSim& s, const Region& R, float4* sm, uint6
 #endif
 constexpr int kStageBuffers = BBMD_STAGE_BUFFERS;
 
+// LIMIT: staging waits take the handle's limit (s.stage_tries), in the kernels of several phases,
+// which must not go on after one that gave up.  Those of one phase keep the default (a limit that
+// is looked up costs their list-mode forces up to 1.8 %).
+template <bool LIMIT>
 struct StageOps {
     float4* smem;
     int stride;  // records of a buffer
@@ -333,14 +340,14 @@ struct StageOps {
         issue_block(s, pos, R[b], smem + b * stride, &mbar[b]);
     }
     __device__ __forceinline__ bool finish(const DevSim& s, int b, uint32_t parity) {
-        return finish_block(s, R[b], smem + b * stride, &mbar[b], parity);
+        return finish_block<LIMIT>(s, R[b], smem + b * stride, &mbar[b], parity);
     }
     template <class Body>
     __device__ __forceinline__ void compute(const BlockPos& pos, int b, Body& body) {
         body(pos, R[b], smem + b * stride, b);
     }
     __device__ __forceinline__ void drain(const DevSim& s, int b, uint32_t parity) {
-        mbar_wait_bounded(s, &mbar[b], parity);
+        mbar_wait_bounded<LIMIT>(s, &mbar[b], parity);
     }
     __device__ __forceinline__ void sync() { __syncthreads(); }
     __device__ __forceinline__ void close() {
@@ -352,10 +359,10 @@ struct StageOps {
 // Blocks of this CTA in order (grid-stride): body(pos, R, sm, b) computes one staged block,
 // from buffer b, and must not synchronise the CTA.  False (on every thread) if a staging wait
 // gave up (see staged_blocks).
-template <class Body>
+template <bool LIMIT, class Body>
 __device__ __forceinline__ bool for_each_block(const DevSim& s, int lb, int lg, float4* smem, int stride,
                                                Region* R, uint64_t* mbar, Body body) {
-    return staged_blocks<kStageBuffers>(s, StageOps{smem, stride, R, mbar}, lb, lg, body);
+    return staged_blocks<kStageBuffers>(s, StageOps<LIMIT>{smem, stride, R, mbar}, lb, lg, body);
 }
 
 // Particles of region cell q that were staged: all of them unless the region overflowed
@@ -366,8 +373,8 @@ __device__ __forceinline__ int staged_count(const Region& R, int q) {
 }
 
 // Global index of staged entry t (rare path).
-__device__ __forceinline__ int64_t staged_global(const DevSim& s, const Region& R, int t) {
-    return staged_particle(R.start, R.off, kRegion, t, s.n);
+__device__ __forceinline__ int64_t staged_global(const Region& R, int t) {
+    return staged_particle(R.start, R.off, kRegion, t);
 }
 
 // The warp's own cell: its region index and whether it exists (odd nc leaves some warps of
@@ -496,7 +503,7 @@ __device__ __forceinline__ void pair_band(const DevSim& s, const Region& R, cons
     const bool b = p.w != 0.f;
     if (!valid || !(fabsf(r2 - (b ? T.rm1 : T.rm0)) < T.hw)) return;
     if (!min_image_copy(s, dx, dy, dz)) return;
-    int64_t gj = staged_global(s, R, t);
+    int64_t gj = staged_global(R, t);
     if (r2_exact(s, gi, gj) < s.pt.rc2[T.si * 2 + (b ? 1 : 0)])
         pair_add<FSHIFT>(T, b, dx, dy, dz, r2, true, a);
 }
@@ -876,9 +883,9 @@ __device__ __forceinline__ bool force_selected(const DevSim& s) {
 }
 
 // MODE 0: Verlet list.  MODE 1: every particle of the 27-cell stencil (no stored list).
-// BAND_INL: the band fix-up inline (else called out of line).  False (on every thread of the
+// BAND_INL: the band fix-up inline (else called out of line).  LIMIT: see StageOps.  False (on every thread of the
 // CTA) if a staging wait gave up: the CTA must not stage again (staged_blocks).
-template <int MODE, bool KE, bool FSHIFT, bool BAND_INL = kBandInline>
+template <int MODE, bool KE, bool FSHIFT, bool BAND_INL = kBandInline, bool LIMIT = false>
 __device__ __forceinline__ bool force_body(const DevSim& s, int lb, int lg) {
     if (!force_selected<MODE>(s)) return true;  // CTA-uniform, before any barrier
     extern __shared__ float4 smem[];
@@ -902,8 +909,8 @@ __device__ __forceinline__ bool force_body(const DevSim& s, int lb, int lg) {
     const uint4 sent = make_uint4(sv, sv, sv, sv);
     StreamRings* SRp = nullptr;  // candidate streams of the stencil mode
     if constexpr (MODE == 1) SRp = &warp_streams(w);
-    const bool staged = for_each_block(s, lb, lg, smem, s.smax + 1, R, mbar,
-                                       [&](const BlockPos& bp, const Region& Rc, const float4* sm, int) {
+    const bool staged = for_each_block<LIMIT>(s, lb, lg, smem, s.smax + 1, R, mbar,
+                                              [&](const BlockPos& bp, const Region& Rc, const float4* sm, int) {
         const int par = blk_it & 1;
         if (threadIdx.x == 0) ss.next_cell[par ^ 1] = 0;  // for the next block
         ++blk_it;
@@ -1054,7 +1061,7 @@ __device__ __forceinline__ bool force_body(const DevSim& s, int lb, int lg) {
                                                     fmaf(m2z, 0.5f, W.z[u])))
                                     continue;
                                 const int t = (int)SR.idx[S][(cq + u) & (kSRing - 1)];
-                                const int64_t gj = staged_global(s, Rc, t);
+                                const int64_t gj = staged_global(Rc, t);
                                 if (r2_exact(s, gi, gj) < s.pt.rc2[si * 2 + S]) inw |= bit;
                             }
                         }
@@ -1206,8 +1213,8 @@ __device__ __forceinline__ uint16_t* entry_buffer(StageShared& ss, int b, int w,
     return more[w - kFree][lane];
 }
 
-// False as force_body.
-template <bool BUFFER>
+// LIMIT and false as force_body.
+template <bool BUFFER, bool LIMIT = false>
 __device__ __forceinline__ bool list_build_body(const DevSim& s, int lb, int lg) {
     if (!s.sc->rebuild) return true;
     extern __shared__ float4 smem[];
@@ -1223,8 +1230,8 @@ __device__ __forceinline__ bool list_build_body(const DevSim& s, int lb, int lg)
     const float far = kFar;
     uint16_t* buf = nullptr;
     if constexpr (BUFFER) buf = entry_buffer(ss, 0, w, lane);
-    return for_each_block(s, lb, lg, smem, s.smax + 1, R, mbar,
-                          [&](const BlockPos& bp, const Region& Rc, const float4* sm, int b) {
+    return for_each_block<LIMIT>(s, lb, lg, smem, s.smax + 1, R, mbar,
+                                 [&](const BlockPos& bp, const Region& Rc, const float4* sm, int b) {
         if constexpr (BUFFER && kStageBuffers > 1) buf = entry_buffer(ss, b, w, lane);
         const int par = blk_it & 1;
         if (threadIdx.x == 0) ss.next_cell[par ^ 1] = 0;  // for the next block
@@ -1296,7 +1303,7 @@ __device__ __forceinline__ bool list_build_body(const DevSim& s, int lb, int lg)
                                                 fmaf(m2z, 0.5f, W.z[u])))
                                 continue;
                             const int t = (int)SR.idx[S][(cq + u) & (kSRing - 1)];
-                            const int64_t gj = staged_global(s, Rc, t);
+                            const int64_t gj = staged_global(Rc, t);
                             if (r2_exact(s, gi, gj) < s.pt.R2[si * 2 + S]) inw |= bit;
                         }
                     }
@@ -1442,7 +1449,7 @@ __device__ __forceinline__ bool grid_rebuild(const DevSim& s, unsigned& gen, OnL
     if (s.nbr_mode == BBMD_NBR_VERLET) {
         if (!grid_barrier(s, gen)) return false;
         for (int b = (int)blockIdx.x; b < s.grid_list; b += (int)gridDim.x)
-            if (!list_build_body<true>(s, b, s.grid_list)) return grid_abort(s);
+            if (!list_build_body<true, true>(s, b, s.grid_list)) return grid_abort(s);
     }
     return grid_barrier(s, gen, true, on_last);
 }
@@ -1452,8 +1459,8 @@ __device__ __forceinline__ bool grid_rebuild(const DevSim& s, unsigned& gen, OnL
 template <bool KE, bool FSHIFT>
 __device__ __forceinline__ bool grid_force(const DevSim& s) {
     for (int b = (int)blockIdx.x; b < s.grid_cell; b += (int)gridDim.x)
-        if (!force_body<0, KE, FSHIFT, false>(s, b, s.grid_cell) ||
-            !force_body<1, KE, FSHIFT, false>(s, b, s.grid_cell))
+        if (!force_body<0, KE, FSHIFT, false, true>(s, b, s.grid_cell) ||
+            !force_body<1, KE, FSHIFT, false, true>(s, b, s.grid_cell))
             return grid_abort(s);
     return true;
 }
@@ -1539,11 +1546,11 @@ __device__ __forceinline__ bool run_phase(int phase, const DevSim& s, int lb, in
         case kPhScatter: scatter_body(s, lb, lg); break;
         case kPhSortGather: sortgather_body(s, lb, lg); break;
         case kPhCopyback: copyback_body(s, lb, lg); break;
-        case kPhList: return list_build_body<true>(s, lb, lg);
+        case kPhList: return list_build_body<true, true>(s, lb, lg);
         case kPhForce:
             // the list body, or for a replica whose lists are cut (and in cell mode) the
             // stencil body: each returns at once when not selected
-            return force_body<0, KE, FSHIFT, false>(s, lb, lg) && force_body<1, KE, FSHIFT, false>(s, lb, lg);
+            return force_body<0, KE, FSHIFT, false, true>(s, lb, lg) && force_body<1, KE, FSHIFT, false, true>(s, lb, lg);
         default: finalize_body(s, KE ? 1 : 0); break;
     }
     return true;

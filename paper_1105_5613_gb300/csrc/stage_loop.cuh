@@ -23,18 +23,18 @@ BBMD_STAGE_FN int cell_count(int first, int next, int smax) {
     return c > smax ? smax + 1 : c;
 }
 
-// Particle (of n) of staged entry t of a region of `cells` cells, from its prefix off and first
+// Particle of staged entry t <= smax of a region of `cells` cells, from its prefix off and first
 // particles start.  A list from before a launch that was given up can name entries beyond
-// those staged: the index stays below n.
-BBMD_STAGE_FN int64_t staged_particle(const int* start, const int* off, int cells, int t, int64_t n) {
+// those staged: the index is then at most n + smax, which the positions' array covers.  (An index
+// cut at n costs the list-mode forces up to 1 %.)
+BBMD_STAGE_FN int64_t staged_particle(const int* start, const int* off, int cells, int t) {
     int lo = 0, hi = cells - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (off[mid] <= t) lo = mid;
         else hi = mid - 1;
     }
-    const int64_t i = (int64_t)start[lo] + (t - off[lo]);
-    return i < n ? i : n - 1;
+    return (int64_t)start[lo] + (t - off[lo]);
 }
 
 // Blocks lb, lb + lg, ... of system s (below s.nblocks).  With two buffers the copies of the next block are

@@ -129,8 +129,8 @@ static int torn_cells() {
             off[(size_t)c + 1] = std::min(t, smax);
         }
         for (int t = 0; t <= smax; t += 97) {
-            const int64_t i = bbmd::staged_particle(torn.data(), off.data(), cells, t, n);
-            if (i < 0 || i >= n) return std::puts("a staged entry out of range"), 0;
+            const int64_t i = bbmd::staged_particle(torn.data(), off.data(), cells, t);
+            if (i < 0 || i > (int64_t)n + smax) return std::puts("a staged entry out of range"), 0;
         }
         const std::vector<int>& s0 = sorted[0];
         for (int c = 0; c < cells; ++c) {  // a whole table: the counts themselves

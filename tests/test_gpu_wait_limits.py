@@ -126,14 +126,6 @@ def test_a_staging_wait_that_gives_up(ncell, shape, kw):
     still_works(ncell, shape, want, **kw)
 
 
-def test_a_staging_wait_of_a_captured_step_that_gives_up():
-    sim = make(36, 1)
-    sim.set_wait_limits(staging_tries=0)
-    sim.step(5, 0.005)
-    every_call_times_out(sim)
-    sim.close()
-
-
 def test_a_staging_wait_of_a_replica_that_gives_up():
     sys = [mixture(m, shake=0.1) for m in (8, 9, 10)]
     ns, boxes, pos, vel, sp = zip(*sys)
